@@ -13,8 +13,8 @@
 // logarithm of the small-q r regime a linear function of an input.
 // It is trained on the plan's own exact FP64 table (the tables the method
 // itself generates) by the kernels of this file: a tiled FP32 GEMM used for
-// the forward pass and both backward products, SiLU and its derivative, the
-// mean-squared loss, bias reductions and Adam.  For inference the weights are
+// the forward pass and both backward products with SiLU and its derivative in
+// the epilogues, the mean-squared loss, split weight gradients and Adam.  For inference the weights are
 // rounded to bf16 values and the products accumulate in FP32 (fused
 // tensor-core kernel in fbc_mlp_tc.cu).
 //
@@ -47,7 +47,9 @@ struct fbc_surrogate {
     int step = 0;
     // training scratch (sized for the largest batch used)
     int cap = 0;
-    float* d_act = nullptr;    // Z1 A1 Z2 A2 Z3 A3 (cap x H each), Y, dY (cap x 6), T, B0, B1 (cap x H)
+    float* d_act = nullptr;    // Z1 A1 Z2 A2 Z3 A3 (cap x H each), Y, dY (cap x 6), dZ1, dZ2, dZ3 (cap x H)
+    int splits = 1;            // row splits of the weight gradients at most, and their partials [splits][n_params]
+    float* d_part = nullptr;
     double* d_loss = nullptr;
     int* d_status = nullptr;   // error word of the fused inference kernel
 };
@@ -57,57 +59,100 @@ namespace {
 
 constexpr int kOut = 6;
 
-// ---- generic FP32 GEMM: C[M x N] = op(A)[M x K] op(B)[K x N] (+ bias) (+ beta C) ----
-// TA: A stored K x M (transposed); TB: B stored N x K (transposed).
-template <bool TA, bool TB>
-__global__ void k_gemm(int M, int N, int K, const float* __restrict__ A, int lda, const float* __restrict__ B, int ldb,
-                       float* __restrict__ C, int ldc, const float* __restrict__ bias, float beta) {
-    constexpr int BM = 64, BN = 64, BK = 16;
-    __shared__ float sa[BK][BM + 1];
-    __shared__ float sb[BK][BN + 1];
-    const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;  // 16 x 16 threads, 4 x 4 outputs each
-    const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
-    float acc[4][4] = {};
-    for (int k0 = 0; k0 < K; k0 += BK) {
-        for (int e = threadIdx.x; e < BM * BK; e += 256) {
-            const int kk = e / BM, mm = e % BM;
-            const int m = m0 + mm, k = k0 + kk;
-            float v = 0.f;
-            if (m < M && k < K) v = TA ? A[(size_t)k * lda + m] : A[(size_t)m * lda + k];
-            sa[kk][mm] = v;
-        }
-        for (int e = threadIdx.x; e < BN * BK; e += 256) {
-            const int kk = e / BN, nn = e % BN;
-            const int n = n0 + nn, k = k0 + kk;
-            float v = 0.f;
-            if (n < N && k < K) v = TB ? B[(size_t)n * ldb + k] : B[(size_t)k * ldb + n];
-            sb[kk][nn] = v;
-        }
-        __syncthreads();
+// ---- FP32 GEMM of the training path: C[M x N] = op(A)[M x K] op(B)[K x N] ----
+// A 64 x 64 tile per block of 256 threads, 4 x 4 outputs per thread, K in steps of 32 through two
+// shared-memory buffers: the next step's words are loaded into registers (16-byte loads where the leading
+// dimension and the base allow them) while the current step is multiplied, one barrier per step.  What
+// bounds it at a batch of 4096 rows and width 128 (128 blocks): the chain of K / 32 loads and the FP32 pipe,
+// not memory: 12 us a 128 x 128 layer (28 us with scalar loads and two barriers per 16 columns).  The
+// products of one output are added in the order of K.
+constexpr int kBM = 64, kBN = 64, kBK = 32;
+
+// One operand's tile [kBK][64] in registers: element (k, m) of op(X), KM: stored K x M (m contiguous),
+// otherwise M x K (k contiguous).  Outside [0, Mx) x [k0, k1) zero.
+template <bool KM>
+struct TileLoad {
+    const float* X;
+    int ld, m0, Mx;
+    bool vec;
+    float4 r[2];
+    __device__ void init(const float* x, int l, int m, int mx) {
+        X = x, ld = l, m0 = m, Mx = mx;
+        vec = (l % 4 == 0) && (((size_t)x & 15) == 0);
+    }
+    __device__ void load(int k0, int k1) {
 #pragma unroll
-        for (int kk = 0; kk < BK; kk++) {
-            float a[4], b[4];
+        for (int h = 0; h < 2; h++) {
+            const int e = threadIdx.x + 256 * h;
+            const int i = KM ? k0 + e / 16 : m0 + e / 8;         // row of the stored matrix
+            const int j = KM ? m0 + (e % 16) * 4 : k0 + (e % 8) * 4;  // its column
+            const int ni = KM ? k1 : Mx, nj = KM ? Mx : k1;
+            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (i < ni && j < nj) {
+                const float* p = X + (size_t)i * ld + j;
+                if (vec && j + 3 < nj) v = *(const float4*)p;
+                else {
+                    v.x = p[0];
+                    if (j + 1 < nj) v.y = p[1];
+                    if (j + 2 < nj) v.z = p[2];
+                    if (j + 3 < nj) v.w = p[3];
+                }
+            }
+            r[h] = v;
+        }
+    }
+    __device__ void store(float (*s)[kBM + 4]) const {
 #pragma unroll
-            for (int i = 0; i < 4; i++) a[i] = sa[kk][ty * 4 + i], b[i] = sb[kk][tx * 4 + i];
+        for (int h = 0; h < 2; h++) {
+            const int e = threadIdx.x + 256 * h;
+            if (KM) {
+                *(float4*)&s[e / 16][(e % 16) * 4] = r[h];
+            } else {
+                const int k = (e % 8) * 4, m = e / 8;
+                s[k][m] = r[h].x, s[k + 1][m] = r[h].y, s[k + 2][m] = r[h].z, s[k + 3][m] = r[h].w;
+            }
+        }
+    }
+};
+
+// acc += op(A)[m0.., k0..k1) op(B)[k0..k1), n0..]; bsum (where wanted) += the column sums of op(B)
+template <bool TA, bool TB, bool BSUM>
+__device__ __forceinline__ void gemm_tile(const float* A, int lda, int m0, int M, const float* B, int ldb, int n0, int N,
+                                          int k0, int k1, float (&acc)[4][4], float (&bsum)[4]) {
+    __shared__ __align__(16) float sa[2][kBK][kBM + 4];
+    __shared__ __align__(16) float sb[2][kBK][kBN + 4];
+    const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
+    TileLoad<TA> la;
+    TileLoad<!TB> lb;
+    la.init(A, lda, m0, M);
+    lb.init(B, ldb, n0, N);
+    la.load(k0, k1);
+    lb.load(k0, k1);
+    int buf = 0;
+    for (int k = k0; k < k1; k += kBK, buf ^= 1) {
+        la.store(sa[buf]);
+        lb.store(sb[buf]);
+        __syncthreads();  // the other buffer is free again: every thread is past the step before
+        if (k + kBK < k1) la.load(k + kBK, k1), lb.load(k + kBK, k1);
+        const int kn = min(kBK, k1 - k);
+        auto step = [&](int kk) {
+            const float4 av = *(const float4*)&sa[buf][kk][ty * 4], bv = *(const float4*)&sb[buf][kk][tx * 4];
+            const float a[4] = {av.x, av.y, av.z, av.w}, b[4] = {bv.x, bv.y, bv.z, bv.w};
 #pragma unroll
             for (int i = 0; i < 4; i++)
 #pragma unroll
                 for (int j = 0; j < 4; j++) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+            if (BSUM)
+#pragma unroll
+                for (int j = 0; j < 4; j++) bsum[j] += b[j];
+        };
+        if (kn == kBK) {
+#pragma unroll 8
+            for (int kk = 0; kk < kBK; kk++) step(kk);
+        } else {
+            for (int kk = 0; kk < kn; kk++) step(kk);
         }
-        __syncthreads();
     }
-#pragma unroll
-    for (int i = 0; i < 4; i++)
-#pragma unroll
-        for (int j = 0; j < 4; j++) {
-            const int m = m0 + ty * 4 + i, n = n0 + tx * 4 + j;
-            if (m < M && n < N) {
-                float v = acc[i][j];
-                if (bias) v += bias[n];
-                if (beta != 0.f) v += beta * C[(size_t)m * ldc + n];
-                C[(size_t)m * ldc + n] = v;
-            }
-        }
 }
 
 __device__ __forceinline__ float silu(float z) { return z / (1.f + expf(-z)); }
@@ -116,14 +161,83 @@ __device__ __forceinline__ float silu_grad(float z) {
     return s * (1.f + z * (1.f - s));
 }
 
-__global__ void k_silu(const float* __restrict__ z, float* __restrict__ a, size_t n) {
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-        a[i] = silu(z[i]);
+// Epilogues: the forward pass writes Z = acc + bias and, for a hidden layer, A = SiLU(Z) beside it; the
+// backward pass turns the gradient with respect to a layer's input into the gradient with respect to the
+// previous layer's Z, dZ = acc silu'(Z).  (Separate kernels re-read and re-wrote [rows][H] for each.)
+enum { kEpiBias = 0, kEpiSilu = 1, kEpiBack = 2 };
+template <bool TB, int EPI>
+__global__ void __launch_bounds__(256) k_gemm(int M, int N, int K, const float* __restrict__ A, int lda,
+                                              const float* __restrict__ B, int ldb, float* __restrict__ C, int ldc,
+                                              const float* __restrict__ bias, const float* __restrict__ Z,
+                                              float* __restrict__ act) {
+    const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
+    const int m0 = blockIdx.y * kBM, n0 = blockIdx.x * kBN;
+    float acc[4][4] = {}, bs[4];
+    gemm_tile<false, TB, false>(A, lda, m0, M, B, ldb, n0, N, 0, K, acc, bs);
+#pragma unroll
+    for (int i = 0; i < 4; i++) {
+        const int m = m0 + ty * 4 + i;
+        if (m >= M) break;
+#pragma unroll
+        for (int j = 0; j < 4; j++) {
+            const int n = n0 + tx * 4 + j;
+            if (n >= N) break;
+            const size_t o = (size_t)m * ldc + n;
+            if (EPI == kEpiBack) {
+                C[o] = acc[i][j] * silu_grad(Z[o]);
+            } else {
+                const float v = acc[i][j] + bias[n];
+                C[o] = v;
+                if (EPI == kEpiSilu) act[o] = silu(v);
+            }
+        }
+    }
 }
-__global__ void k_silu_back(const float* __restrict__ z, const float* __restrict__ da, float* __restrict__ dz, size_t n) {
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-        dz[i] = da[i] * silu_grad(z[i]);
+
+// Weight and bias gradients of all four layers in one launch: dW_l = A_l^T dZ_l over the batch's rows, db_l =
+// the column sums of dZ_l.  The contraction runs over the rows and the outputs are few (a 128 x 128 layer has
+// four tiles), so the rows are split over blocks: one launch per layer with one block per tile took 1.1 ms of a
+// 3.0 ms step at 4096 rows, width 128, and the column sums, one thread per column, 0.2 ms more; split, the
+// launch takes 0.020 ms and its reduction 0.007 ms.  Block x = (layer, tile), y = split; the partial
+// of split s goes to part[s][n_params], summed in the order of s by k_wgrad_sum.
+struct WgradArgs {
+    const float* A[4];   // [rows][din]
+    const float* dZ[4];  // [rows][dout]
+    int din[4], dout[4], tile0[5], off_w[4], off_b[4];
+    int rows, per, n_params;
+};
+__global__ void __launch_bounds__(256) k_wgrad(WgradArgs W, float* __restrict__ part) {
+    int l = 0;
+    while (l < 3 && (int)blockIdx.x >= W.tile0[l + 1]) l++;
+    const int t = blockIdx.x - W.tile0[l], din = W.din[l], dout = W.dout[l];
+    const int tn = (dout + kBN - 1) / kBN;
+    const int m0 = t / tn * kBM, n0 = t % tn * kBN;
+    const int k0 = blockIdx.y * W.per, k1 = min(W.rows, k0 + W.per);
+    const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
+    float acc[4][4] = {}, bs[4] = {};
+    gemm_tile<true, false, true>(W.A[l], din, m0, din, W.dZ[l], dout, n0, dout, k0, k1, acc, bs);
+    float* o = part + (size_t)blockIdx.y * W.n_params;
+#pragma unroll
+    for (int j = 0; j < 4; j++) {
+        const int n = n0 + tx * 4 + j;
+        if (n >= dout) break;
+        if (m0 == 0 && ty == 0) o[W.off_b[l] + n] = bs[j];
+#pragma unroll
+        for (int i = 0; i < 4; i++) {
+            const int m = m0 + ty * 4 + i;
+            if (m < din) o[W.off_w[l] + m * dout + n] = acc[i][j];
+        }
+    }
 }
+__global__ void k_wgrad_sum(const float* __restrict__ part, int splits, int n, float* __restrict__ g) {
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        float s = 0.f;
+#pragma unroll 8
+        for (int k = 0; k < splits; k++) s += part[(size_t)k * n + i];
+        g[i] = s;
+    }
+}
+
 // dY = 2 (Y - T) / (B * 6), loss partials in FP64 (one slot per block, fixed order later)
 __global__ void k_mse(const float* __restrict__ y, const float* __restrict__ t, float* __restrict__ dy, int n,
                       double* __restrict__ part) {
@@ -142,14 +256,6 @@ __global__ void k_mse(const float* __restrict__ y, const float* __restrict__ t, 
         __syncthreads();
     }
     if (threadIdx.x == 0) part[blockIdx.x] = red[0];
-}
-// column sums: db[j] = sum_i dZ[i][j]
-__global__ void k_colsum(const float* __restrict__ dz, int rows, int cols, float* __restrict__ db) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= cols) return;
-    float s = 0.f;
-    for (int i = 0; i < rows; i++) s += dz[(size_t)i * cols + j];
-    db[j] = s;
 }
 __global__ void k_adam(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m, float* __restrict__ v,
                        int n, float lr, float b1, float b2, float c1, float c2, float eps) {
@@ -219,13 +325,14 @@ cudaError_t surrogate_forward(const fbc_surrogate* S, const float* params, const
     const int din[4] = {4, H, H, H}, dout[4] = {H, H, H, kOut};
     const float* in = X;
     for (int l = 0; l < 4; l++) {
-        float* z = (l < 3) ? act + (size_t)(2 * l) * cap * H : Y;
-        float* a = (l < 3) ? act + (size_t)(2 * l + 1) * cap * H : nullptr;
-        dim3 g((dout[l] + 63) / 64, (n + 63) / 64);
-        k_gemm<false, false><<<g, 256, 0, st>>>(n, dout[l], din[l], in, din[l], W[l], dout[l], z, dout[l], b[l], 0.f);
+        const dim3 g((dout[l] + kBN - 1) / kBN, (n + kBM - 1) / kBM);
         if (l < 3) {
-            k_silu<<<grid_for((size_t)n * H), 256, 0, st>>>(z, a, (size_t)n * H);
+            float* z = act + (size_t)(2 * l) * cap * H;
+            float* a = act + (size_t)(2 * l + 1) * cap * H;
+            k_gemm<false, kEpiSilu><<<g, 256, 0, st>>>(n, H, din[l], in, din[l], W[l], H, z, H, b[l], nullptr, a);
             in = a;
+        } else {
+            k_gemm<false, kEpiBias><<<g, 256, 0, st>>>(n, kOut, H, in, H, W[l], kOut, Y, kOut, b[l], nullptr, nullptr);
         }
     }
     return cudaGetLastError();
@@ -295,8 +402,8 @@ constexpr int kMaxRows = 65535 * 64;
 int ensure_cap(fbc_surrogate* S, int n) {
     if (n > kMaxRows) return sfail(FBC_ERR_INVALID_ARG, "more than 65535 * 64 rows in one evaluation");
     if (n <= S->cap) return FBC_OK;
-    if (S->d_act) cudaFree(S->d_act), S->d_act = nullptr;
-    // Z1 A1 Z2 A2 Z3 A3, Y, dY, and three gradient buffers T, B0, B1
+    if (S->d_act) cudaFree(S->d_act), S->d_act = nullptr, S->cap = 0;
+    // Z1 A1 Z2 A2 Z3 A3, Y, dY, dZ1, dZ2, dZ3
     const size_t per = (size_t)n * (9 * S->width + 2 * 6);
     cudaError_t e = cudaMalloc((void**)&S->d_act, per * sizeof(float));
     if (e) return scuda(e, "surrogate scratch");
@@ -313,8 +420,8 @@ int loss_and_grad(fbc_surrogate* S, const float* X, const float* T, int n, cudaS
     float* act = S->d_act;
     float* Y = act + (size_t)6 * cap * H;
     float* dY = Y + (size_t)cap * kOut;
-    float* Tb = dY + (size_t)cap * kOut;   // gradient with respect to a layer's input activations
-    float* Bz[2] = {Tb + (size_t)cap * H, Tb + (size_t)2 * cap * H};  // gradients with respect to Z, alternating
+    float* dZ[3];  // gradients with respect to Z1, Z2, Z3
+    for (int l = 0; l < 3; l++) dZ[l] = dY + (size_t)cap * kOut + (size_t)l * cap * H;
     cudaError_t e = surrogate_forward(S, S->d_p, X, n, Y, act, cap, st);
     if (e) return scuda(e, "surrogate forward");
     const int nb = 64;
@@ -322,22 +429,24 @@ int loss_and_grad(fbc_surrogate* S, const float* X, const float* T, int n, cudaS
     const int din[4] = {4, H, H, H}, dout[4] = {H, H, H, kOut};
     const float* A_in[4] = {X, act + (size_t)1 * cap * H, act + (size_t)3 * cap * H, act + (size_t)5 * cap * H};
     const float* Zs[3] = {act, act + (size_t)2 * cap * H, act + (size_t)4 * cap * H};
-    const float* dcur = dY;  // gradient with respect to the current layer's output (pre-activation)
-    for (int l = 3; l >= 0; l--) {
-        float* dW = S->d_g + S->off[2 * l];
-        float* db = S->d_g + S->off[2 * l + 1];
-        dim3 gw((dout[l] + 63) / 64, (din[l] + 63) / 64);
-        k_gemm<true, false><<<gw, 256, 0, st>>>(din[l], dout[l], n, A_in[l], din[l], dcur, dout[l], dW, dout[l], nullptr, 0.f);
-        k_colsum<<<(dout[l] + 127) / 128, 128, 0, st>>>(dcur, n, dout[l], db);
-        if (l > 0) {
-            const float* Wl = S->d_p + S->off[2 * l];
-            dim3 gx((din[l] + 63) / 64, (n + 63) / 64);
-            k_gemm<false, true><<<gx, 256, 0, st>>>(n, din[l], dout[l], dcur, dout[l], Wl, dout[l], Tb, din[l], nullptr, 0.f);
-            float* out = Bz[l & 1];
-            k_silu_back<<<grid_for((size_t)n * H), 256, 0, st>>>(Zs[l - 1], Tb, out, (size_t)n * H);
-            dcur = out;
-        }
+    for (int l = 3; l > 0; l--) {  // dZ_l = (dZ_(l+1) W_(l+1)^T) silu'(Z_l)
+        const dim3 g((H + kBN - 1) / kBN, (n + kBM - 1) / kBM);
+        const float* up = l == 3 ? dY : dZ[l];
+        k_gemm<true, kEpiBack><<<g, 256, 0, st>>>(n, H, dout[l], up, dout[l], S->d_p + S->off[2 * l], dout[l], dZ[l - 1],
+                                                  H, nullptr, Zs[l - 1], nullptr);
     }
+    WgradArgs W;
+    W.rows = n, W.n_params = S->n_params, W.tile0[0] = 0;
+    for (int l = 0; l < 4; l++) {
+        W.A[l] = A_in[l], W.dZ[l] = l == 3 ? dY : dZ[l];
+        W.din[l] = din[l], W.dout[l] = dout[l], W.off_w[l] = S->off[2 * l], W.off_b[l] = S->off[2 * l + 1];
+        W.tile0[l + 1] = W.tile0[l] + ((din[l] + kBM - 1) / kBM) * ((dout[l] + kBN - 1) / kBN);
+    }
+    int splits = std::max(1, std::min(S->splits, (n + kBK - 1) / kBK));
+    W.per = ((n + splits - 1) / splits + kBK - 1) / kBK * kBK;
+    splits = (n + W.per - 1) / W.per;
+    k_wgrad<<<dim3(W.tile0[4], splits), 256, 0, st>>>(W, S->d_part);
+    k_wgrad_sum<<<(S->n_params + 127) / 128, 128, 0, st>>>(S->d_part, splits, S->n_params, S->d_g);
     if ((e = cudaGetLastError())) return scuda(e, "surrogate backward");
     if (loss) {
         std::vector<double> part(nb);
@@ -381,6 +490,12 @@ int fbc_surrogate_create(int32_t width, uint64_t seed, fbc_surrogate** out) {
     float** bufs[5] = {&S->d_p, &S->d_pb, &S->d_g, &S->d_m, &S->d_v};
     for (auto b : bufs)
         if (!e) e = cudaMalloc((void**)b, sizeof(float) * o);
+    // weight-gradient blocks: about four per SM over the layers' tiles, so that few enough partials are
+    // written and read back (64 splits at most: width 128 takes 50, width 1024 one)
+    int tiles = 0;
+    for (int l = 0; l < 4; l++) tiles += (((l ? H : 4) + 63) / 64) * (((l < 3 ? H : 6) + 63) / 64);
+    S->splits = std::max(1, std::min(64, 608 / tiles));
+    if (!e) e = cudaMalloc((void**)&S->d_part, sizeof(float) * (size_t)o * S->splits);
     if (!e) e = cudaMalloc((void**)&S->d_loss, 64 * sizeof(double));
     if (!e) e = cudaMalloc((void**)&S->d_status, sizeof(int));
     if (!e) e = cudaMemset(S->d_status, 0, sizeof(int));
@@ -410,8 +525,7 @@ int fbc_surrogate_params(fbc_surrogate* S, float* host_out, const float* host_in
 int fbc_surrogate_forward(fbc_surrogate* S, const float* x, float* y, int32_t n, int32_t bf16_weights, void* stream) {
     fbc::report_error(FBC_OK, "");
     if (!S || !x || !y || n < 1) return sfail(FBC_ERR_INVALID_ARG, "bad arguments");
-    int s = ensure_cap(S, n);
-    if (s) return s;
+    if (n > kMaxRows) return sfail(FBC_ERR_INVALID_ARG, "more than 65535 * 64 rows in one evaluation");
     cudaStream_t st = (cudaStream_t)stream;
     const float* params = S->d_p;
     if (bf16_weights) {
@@ -424,6 +538,8 @@ int fbc_surrogate_forward(fbc_surrogate* S, const float* x, float* y, int32_t n,
             return e ? scuda(e, "fused surrogate inference") : FBC_OK;
         }
     }
+    int s = ensure_cap(S, n);  // the fused kernel keeps no activations in memory
+    if (s) return s;
     cudaError_t e = fbc::surrogate_forward(S, params, x, n, y, S->d_act, S->cap, st);
     return e ? scuda(e, "surrogate forward") : FBC_OK;
 }
@@ -654,7 +770,7 @@ int fbc_surrogate_sync_status(fbc_surrogate* S, void* stream) {
 
 void fbc_surrogate_destroy(fbc_surrogate* S) {
     if (!S) return;
-    void* bufs[] = {S->d_p, S->d_pb, S->d_g, S->d_m, S->d_v, S->d_act, S->d_loss, S->d_status};
+    void* bufs[] = {S->d_p, S->d_pb, S->d_g, S->d_m, S->d_v, S->d_part, S->d_act, S->d_loss, S->d_status};
     for (void* b : bufs)
         if (b) cudaFree(b);
     delete S;
