@@ -65,10 +65,14 @@ struct Plan {
     int n_ta = 0, n_tb = 0, NIpad = 0, NPpad = 0;
     int box_x0 = 0, box_y0 = 0, Dx = 0, Dy = 0;  // difference table box
     int W = 0, H = 0;                             // largest tile-pair sub-box
-    int n_used = 0;
+    int n_used = 0, n_rep = 0;
     fbc_options opt{};
     MaterialDev mat{};
     TabulateParams tp{};
+    // cubic medium: quadrature nodes and scaled constants of the tabulation (made on first use)
+    MaterialDev tab_mat{};
+    double tab_pre = 0.0;
+    std::vector<double> tab_nodes;
     bool tabulated = false;
     int precision = FBC_PREC_FP64;
 
@@ -85,6 +89,7 @@ struct Plan {
     int* d_perm_i = nullptr;     // [NIpad]
     int* d_perm_p = nullptr;     // [NPpad]
     int2* d_used = nullptr;      // [n_used] differences that occur
+    int4* d_rep = nullptr;       // [n_rep] (x, y, mirror, 0): one of each pair d, -d; mirror: -d occurs too
     double2* d_tw = nullptr;     // [L/2] exp(-2 pi i t / L), then the same as [L/2] float2
     double2* d_twL = nullptr;    // [L] (cos, sin)(2 pi t / L) for the table DFT
     float2* d_twl = nullptr;     // [L] exp(-2 pi i t / L) in FP32: the Stockham FP32 line transforms

@@ -192,7 +192,7 @@ int dev_alloc(T** p, size_t count, size_t& acc, const char* what) {
 
 void free_plan(fbc::Plan& P) {
     void* bufs[] = {P.d_xy_p,  P.d_off_i,    P.d_bbox_a, P.d_bbox_b, P.d_perm_i, P.d_perm_p,
-                    P.d_used,  P.d_tw,       P.d_twL,    P.d_twl,    P.d_table,  P.d_table32, P.d_table_x2, P.d_table_x2_k0,
+                    P.d_used,  P.d_rep,      P.d_tw,       P.d_twL,    P.d_twl,    P.d_table,  P.d_table32, P.d_table_x2, P.d_table_x2_k0,
                     P.d_fh,    P.d_uh,       P.d_part,   P.d_stage_f, P.d_stage_u, P.d_status, P.d_bprep,
                     P.d_relax, P.d_uh32};
     for (void* b : bufs)
@@ -427,6 +427,13 @@ int fbc_plan_create(const fbc_geometry* geom, const fbc_material* mat, const fbc
         for (int ix = 0; ix < P.Dx; ix++)
             if (used[(size_t)iy * P.Dx + ix]) used_list.push_back(make_int2(ix + P.box_x0, iy + P.box_y0));
     P.n_used = (int)used_list.size();
+    std::vector<int4> rep_list;  // the differences to evaluate: one of each pair d, -d
+    for (const int2& d : used_list) {
+        const int mx = -d.x - P.box_x0, my = -d.y - P.box_y0;
+        const bool mirror = (d.x || d.y) && mx >= 0 && mx < P.Dx && my >= 0 && my < P.Dy && used[(size_t)my * P.Dx + mx];
+        if (!mirror || d.y < 0 || (d.y == 0 && d.x < 0)) rep_list.push_back(make_int4(d.x, d.y, mirror ? 1 : 0, 0));
+    }
+    P.n_rep = (int)rep_list.size();
 
     // material for the device
     P.mat.kind = mat->kind;
@@ -469,6 +476,7 @@ int fbc_plan_create(const fbc_geometry* geom, const fbc_material* mat, const fbc
     ALLOC(P.d_perm_i, P.NIpad, "perm_i");
     ALLOC(P.d_perm_p, P.NPpad, "perm_p");
     ALLOC(P.d_used, P.n_used, "used");
+    ALLOC(P.d_rep, P.n_rep, "rep");
     ALLOC(P.d_tw, L / 2 + L / 4 + 1, "twiddles");  // L/2 double2, then L/2 float2
     ALLOC(P.d_twL, L, "table_twiddles");
     ALLOC(P.d_twl, L, "line_twiddles");
@@ -512,6 +520,7 @@ int fbc_plan_create(const fbc_geometry* geom, const fbc_material* mat, const fbc
     UP(P.d_perm_i, tb.perm.data(), P.NIpad);
     UP(P.d_perm_p, ta.perm.data(), P.NPpad);
     if (P.n_used) UP(P.d_used, used_list.data(), P.n_used);
+    if (P.n_rep) UP(P.d_rep, rep_list.data(), P.n_rep);
     UP(P.d_tw, tw.data(), L / 2 + L / 4 + 1);
     UP(P.d_twL, twL.data(), L);
     UP(P.d_twl, twl.data(), L);

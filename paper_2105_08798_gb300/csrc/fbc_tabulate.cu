@@ -24,6 +24,11 @@
 //     G(r) = 1/(8 pi^2 |r|) int_0^{2 pi} (zz)^{-1} dpsi,
 // for a cubic one, evaluated by the trapezoid rule on [0, pi) (the integrand
 // has period pi) with the nodes' cosines and sines in constant memory.
+//
+// The reference terms G(0, 0, +-m l3) depend on m alone and are computed once; of each pair d, -d only one is
+// evaluated.  Together four times fewer Green functions than one thread per (d, s) evaluating all of
+// them: an isotropic slab of 4000 x 6000 columns, L = 256, 23.5 ms before, 8.9 ms now.
+#include <algorithm>
 #include <cmath>
 #include <vector>
 
@@ -34,25 +39,31 @@ namespace {
 
 __constant__ MaterialDev c_mat;
 __constant__ TabulateParams c_tp;
-__constant__ double c_qcos[kMaxQuad];
+__constant__ double c_qcos[kMaxQuad];     // the quadrature nodes psi
 __constant__ double c_qsin[kMaxQuad];
+__constant__ double c_node[kMaxQuad][6];  // cos and sin of 2 psi, 4 psi and 6 psi at the quadrature nodes
+__constant__ double c_pre;                // cubic medium: (scale of the constants) / (pi nquad)
 
-// G as six entries (11, 12, 22, 33, 13, 23) of the symmetric tensor.
-__device__ void green6(double rx, double ry, double rz, double g[6]) {
+// G as six entries (11, 12, 22, 33, 13, 23) of the symmetric tensor: Kelvin's closed form.
+__device__ void green_isotropic(double rx, double ry, double rz, double g[6]) {
     const double R2 = rx * rx + ry * ry + rz * rz;
     const double R = sqrt(R2);
-    if (c_mat.kind == FBC_MATERIAL_ISOTROPIC) {
-        const double pre = c_mat.kelvin_pre / R;
-        const double iR2 = 1.0 / R2;
-        const double a = c_mat.kelvin_a;
-        g[0] = pre * (a + rx * rx * iR2);
-        g[1] = pre * (rx * ry * iR2);
-        g[2] = pre * (a + ry * ry * iR2);
-        g[3] = pre * (a + rz * rz * iR2);
-        g[4] = pre * (rx * rz * iR2);
-        g[5] = pre * (ry * rz * iR2);
-        return;
-    }
+    const double pre = c_mat.kelvin_pre / R;
+    const double iR2 = 1.0 / R2;
+    const double a = c_mat.kelvin_a;
+    g[0] = pre * (a + rx * rx * iR2);
+    g[1] = pre * (rx * ry * iR2);
+    g[2] = pre * (a + ry * ry * iR2);
+    g[3] = pre * (a + rz * rz * iR2);
+    g[4] = pre * (rx * rz * iR2);
+    g[5] = pre * (ry * rz * iR2);
+}
+
+// Barnett's integral for a cubic medium node by node: the Christoffel matrix M of z = cos(psi) e1 + sin(psi) e2,
+// its cofactors and a division at every node, about 88 FP64 operations each.
+__device__ void green_nodes(double rx, double ry, double rz, double g[6]) {
+    const double R2 = rx * rx + ry * ry + rz * rz;
+    const double R = sqrt(R2);
     // unit direction and an orthonormal pair spanning the plane normal to it
     const double iR = 1.0 / R;
     const double hx = rx * iR, hy = ry * iR, hz = rz * iR;
@@ -105,15 +116,190 @@ __device__ void green6(double rx, double ry, double rz, double g[6]) {
     g[5] = pre * s3;
 }
 
-// Stage 1: one thread per (used difference, s in [0, L/2]).
-__global__ void k_periodic(const int2* __restrict__ used, int n_used, double* __restrict__ gs) {
+// What the polynomial form below keeps for all points r = (d, z) of one in-plane difference d: rho = |d|, the in-plane unit vector e1 normal to r, and e1's part of the Christoffel matrix.
+struct CubicDir {
+    double rho2, rho, e1x, e1y, p[6], k11[6];
+};
+
+__device__ __forceinline__ void christoffel(const double (&p)[6], double (&m)[6]) {
+#pragma unroll
+    for (int I = 0; I < 6; I++) {
+        double v = 0.0;
+#pragma unroll
+        for (int J = 0; J < 6; J++) v = fma(c_mat.K[6 * I + J], p[J], v);
+        m[I] = v;
+    }
+}
+
+__device__ __forceinline__ CubicDir cubic_dir(double rx, double ry) {
+    CubicDir D;
+    const bool line = rx == 0.0 && ry == 0.0;  // r along the line: any in-plane direction
+    D.rho2 = fma(rx, rx, ry * ry);
+    D.rho = sqrt(D.rho2);
+    const double i = line ? 0.0 : 1.0 / D.rho2;
+    D.e1x = line ? 1.0 : -ry / D.rho;
+    D.e1y = line ? 0.0 : rx / D.rho;
+    D.p[0] = line ? 1.0 : ry * ry * i;
+    D.p[1] = rx * rx * i;
+    D.p[2] = D.p[3] = D.p[4] = 0.0;
+    D.p[5] = -(rx * ry) * i;
+    christoffel(D.p, D.k11);
+    return D;
+}
+
+// The same sum with the work per node reduced; FP64 issue bounds the tabulation (this part's FP64 pipe runs at
+// 1/64 of the FP32 rate).  2 M = u + v cos 2psi + w sin 2psi exactly, so its cofactors are trigonometric polynomials
+// of degree 2 in 2 psi (five coefficients each, once per point) and its determinant one of degree 3 (seven), and
+//     sum_q cof_ij(psi_q) / det(psi_q) = sum_t coef_ij,t  sum_q basis_t(psi_q) / det(psi_q):
+// five sums serve all six entries.  With an even number of nodes psi and psi + pi/2 are both nodes; the even
+// part E and odd part O of the determinant serve both, 1/(E+O) +- 1/(E-O) = (2 E, -2 O) / ((E+O)(E-O)), and
+// one division serves two such pairs.  About 11 FP64 operations a node and 400 a point.  The coefficients' rounding is
+// the same at every node and does not average out, so the directions enter as quotients of exact squares, the
+// products are fused and the sums are taken in groups of eight pairs: emulated against 64-bit mantissas over a
+// slab's points the entries' error is then that of the node-by-node form (3.11e-16 and 3.12e-16 of |G|).
+// The 1000 x 1500, L = 64 cubic slab's table: 112.3 ms with its first update before, 6.9 ms now;
+// 4000 x 6000, L = 256: 1676 ms before, 97 ms now (433 ms with the node-by-node form).
+__device__ void green_cubic(const CubicDir& D, double rx, double ry, double rz, double g[6]) {
+    const double R2 = fma(rz, rz, D.rho2), R = sqrt(R2), iR = 1.0 / R, i2 = 1.0 / R2;
+    const double hz = rz * iR, hr = D.rho * iR, zz = rz * rz * i2;
+    double u[6], v[6], w[6];  // 2 M = u + v cos 2psi + w sin 2psi, entries (00, 11, 22, 12, 02, 01)
+    {
+        // e2 = (-hz e1y, hz e1x, hr)
+        const double p22[6] = {zz * D.p[1], zz * D.p[0], D.rho2 * i2, -(rz * ry) * i2, -(rz * rx) * i2, -zz * D.p[5]};
+        double k22[6];
+        christoffel(p22, k22);
+        const double x = 2.0 * hz * D.p[5];
+        const double p12[6] = {-x, x, 0.0, D.e1y * hr, D.e1x * hr, hz * (D.p[0] - D.p[1])};
+        christoffel(p12, w);
+#pragma unroll
+        for (int t = 0; t < 6; t++) u[t] = D.k11[t] + k22[t], v[t] = D.k11[t] - k22[t];
+    }
+    // cofactors times 2 in the basis (1, cos 2psi, sin 2psi, cos 4psi, sin 4psi)
+    double A[6][5];  // 00, 11, 22, 12, 02, 01
+    auto cof = [&](double (&q)[5], int i, int j, int k, int l) {  // m_i m_j - m_k m_l
+        const double vv = fma(v[i], v[j], -(v[k] * v[l])), ww = fma(w[i], w[j], -(w[k] * w[l]));
+        q[0] = fma(2.0, fma(u[i], u[j], -(u[k] * u[l])), vv + ww);
+        q[1] = 2.0 * (fma(u[i], v[j], v[i] * u[j]) - fma(u[k], v[l], v[k] * u[l]));
+        q[2] = 2.0 * (fma(u[i], w[j], w[i] * u[j]) - fma(u[k], w[l], w[k] * u[l]));
+        q[3] = vv - ww;
+        q[4] = fma(v[i], w[j], w[i] * v[j]) - fma(v[k], w[l], w[k] * v[l]);
+    };
+    cof(A[0], 1, 2, 3, 3);
+    cof(A[1], 0, 2, 4, 4);
+    cof(A[2], 0, 1, 5, 5);
+    cof(A[3], 4, 5, 0, 3);
+    cof(A[4], 3, 5, 1, 4);
+    cof(A[5], 3, 4, 2, 5);
+    // four times the determinant in the basis (1, cos, sin of 2psi, of 4psi, of 6psi)
+    double d0 = 0, d1 = 0, d2 = 0, d3 = 0, d4 = 0, d5 = 0, d6 = 0;
+    auto det = [&](int i, const double (&q)[5]) {
+        const double ui = 2.0 * u[i], vi = v[i], wi = w[i];
+        d0 = fma(ui, q[0], fma(vi, q[1], fma(wi, q[2], d0)));
+        d1 = fma(ui, q[1], fma(2.0 * vi, q[0], fma(vi, q[3], fma(wi, q[4], d1))));
+        d2 = fma(ui, q[2], fma(2.0 * wi, q[0], fma(vi, q[4], fma(-wi, q[3], d2))));
+        d3 = fma(ui, q[3], fma(vi, q[1], fma(-wi, q[2], d3)));
+        d4 = fma(ui, q[4], fma(vi, q[2], fma(wi, q[1], d4)));
+        d5 = fma(vi, q[3], fma(-wi, q[4], d5));
+        d6 = fma(vi, q[4], fma(wi, q[3], d6));
+    };
+    det(4, A[4]);
+    det(5, A[5]);
+    det(0, A[0]);
+    double s0 = 0, s1 = 0, s2 = 0, s3 = 0, s4 = 0, t0 = 0, t1 = 0, t2 = 0, t3 = 0, t4 = 0;
+    auto parts = [&](int q, double& E, double& O) {
+        const double* n = c_node[q];
+        E = fma(n[3], d4, fma(n[2], d3, d0));
+        O = fma(n[5], d6, fma(n[4], d5, fma(n[1], d2, n[0] * d1)));
+    };
+    auto add = [&](int q, double e, double o) {  // e, o: the even and odd parts of the node's 1 / det
+        const double* n = c_node[q];
+        t0 += e;
+        t1 = fma(n[0], o, t1);
+        t2 = fma(n[1], o, t2);
+        t3 = fma(n[2], e, t3);
+        t4 = fma(n[3], e, t4);
+    };
+    auto join = [&]() {
+        s0 += t0, s1 += t1, s2 += t2, s3 += t3, s4 += t4;
+        t0 = t1 = t2 = t3 = t4 = 0.0;
+    };
+    const int nq = c_mat.nquad;
+    double scale;
+    if (nq % 4 == 0) {
+        for (int q = 0; q < nq / 2; q += 2) {
+            double E, O, F, Q;
+            parts(q, E, O);
+            parts(q + 1, F, Q);
+            const double p = (E + O) * (E - O), r = (F + Q) * (F - Q);
+            const double i = 1.0 / (p * r);
+            const double ip = i * r, ir = i * p;
+            add(q, E * ip, -O * ip);
+            add(q + 1, F * ir, -Q * ir);
+            if (q % 8 == 6) join();
+        }
+        scale = 2.0;
+    } else {
+        for (int q = 0; q < nq; q++) {
+            double E, O;
+            parts(q, E, O);
+            const double i = 1.0 / (E + O);
+            add(q, i, i);
+            if (q % 8 == 7) join();
+        }
+        scale = 1.0;
+    }
+    join();
+    const double pre = scale * c_pre * iR;
+    auto entry = [&](const double (&q)[5]) {
+        return pre * fma(q[0], s0, fma(q[1], s1, fma(q[2], s2, fma(q[3], s3, q[4] * s4))));
+    };
+    g[0] = entry(A[0]);
+    g[1] = entry(A[5]);
+    g[2] = entry(A[1]);
+    g[3] = entry(A[2]);
+    g[4] = entry(A[4]);
+    g[5] = entry(A[3]);
+}
+
+// Which Green function a launch evaluates.  The polynomial form serves the plans of the FP64-accurate precisions.
+// The others round the table to 32 bits or fewer, where a last-bit change of a few FP64 entries moves the
+// rounding of some (1e-9 to 4e-9 of an update, more than those forms differ by from run to run): they and the
+// H-matrix's FP32 table keep the node-by-node form's bits.
+enum { kGreenIso = 0, kGreenNodes = 1, kGreenPoly = 2 };
+
+// G(0, 0, m l3) + G(0, 0, -m l3) for the images m = 1 .. n + N: the same for every difference and offset.
+template <int KIND>
+__global__ void k_reference(double* __restrict__ ref) {
+    const int m = threadIdx.x + 1;
+    if (m > c_tp.rich_n + c_tp.rich_N) return;
+    const double zm = (double)m * ((double)c_tp.L * c_tp.c);
+    double g[6], h[6];
+    if (KIND == kGreenIso) {
+        green_isotropic(0.0, 0.0, zm, g);
+        green_isotropic(0.0, 0.0, -zm, h);
+    } else if (KIND == kGreenNodes) {
+        green_nodes(0.0, 0.0, zm, g);
+        green_nodes(0.0, 0.0, -zm, h);
+    } else {
+        const CubicDir D = cubic_dir(0.0, 0.0);
+        green_cubic(D, 0.0, 0.0, zm, g);
+        green_cubic(D, 0.0, 0.0, -zm, h);
+    }
+    for (int t = 0; t < 6; t++) ref[(m - 1) * 6 + t] = g[t] + h[t];
+}
+
+// Stage 1: one thread per (listed difference, s in [0, L/2]).  Of a pair of used differences d and -d only one
+// is listed: G(-d, s) is G(d, s) with the odd entries (13, 23) negated, bit for bit, so stage 2 writes both.
+template <int KIND>
+__global__ void __launch_bounds__(128) k_periodic(const int4* __restrict__ rep, int n_rep,
+                                                  const double* __restrict__ ref, double* __restrict__ gs) {
     const int Lh = c_tp.Lh;
     const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const long long total = (long long)n_used * (Lh + 1);
+    const long long total = (long long)n_rep * (Lh + 1);
     if (tid >= total) return;
     const int di = (int)(tid / (Lh + 1));
     const int s = (int)(tid % (Lh + 1));
-    const int2 d = used[di];
+    const int4 d = rep[di];
     if (d.x == 0 && d.y == 0) {  // self-terms (FBC_PLAN_SELF_TERMS): filled by the lattice near field
         double* o0 = gs + ((size_t)di * (Lh + 1) + s) * 6;
         for (int t = 0; t < 6; t++) o0[t] = 0.0;
@@ -122,23 +308,29 @@ __global__ void k_periodic(const int2* __restrict__ used, int n_used, double* __
     const double rx = (double)d.x, ry = (double)d.y;
     const double l3 = (double)c_tp.L * c_tp.c;
     const double z0 = (double)s * c_tp.c;  // centred representative: s <= L/2
-    double acc[6], g[6], h[6], gr[6], hr[6];
-    green6(rx, ry, z0, acc);
+    CubicDir D;
+    if (KIND == kGreenPoly) D = cubic_dir(rx, ry);
+    auto green = [&](double z, double (&g)[6]) {
+        if (KIND == kGreenIso) green_isotropic(rx, ry, z, g);
+        else if (KIND == kGreenNodes) green_nodes(rx, ry, z, g);
+        else green_cubic(D, rx, ry, z, g);
+    };
+    double acc[6], g[6], h[6];
+    green(z0, acc);
     const int n = c_tp.rich_n, N = c_tp.rich_N;
     double tail[6] = {0, 0, 0, 0, 0, 0};
     for (int m = 1; m <= n + N; m++) {
         const double zm = (double)m * l3;
-        green6(rx, ry, z0 + zm, g);
-        green6(rx, ry, z0 - zm, h);
-        green6(0.0, 0.0, zm, gr);
-        green6(0.0, 0.0, -zm, hr);
+        green(z0 + zm, g);
+        green(z0 - zm, h);
+        const double* rf = ref + (m - 1) * 6;
         if (m <= n) {
 #pragma unroll
-            for (int t = 0; t < 6; t++) acc[t] += ((g[t] + h[t]) - (gr[t] + hr[t]));
+            for (int t = 0; t < 6; t++) acc[t] += ((g[t] + h[t]) - rf[t]);
         } else {
             const double w = c_tp.W[m - n - 1];
 #pragma unroll
-            for (int t = 0; t < 6; t++) tail[t] = fma(w, (g[t] + h[t]) - (gr[t] + hr[t]), tail[t]);
+            for (int t = 0; t < 6; t++) tail[t] = fma(w, (g[t] + h[t]) - rf[t], tail[t]);
         }
     }
     double* o = gs + ((size_t)di * (Lh + 1) + s) * 6;
@@ -154,8 +346,9 @@ __global__ void k_periodic(const int2* __restrict__ used, int n_used, double* __
     }
 }
 
-// Stage 2: one CTA per used difference; threads over k.
-__global__ void k_line_dft(const int2* __restrict__ used, const double* __restrict__ gs,
+// Stage 2: one CTA per listed difference; threads over k.  The table entry of -d is that of d with the odd
+// entries negated.
+__global__ void k_line_dft(const int4* __restrict__ rep, const double* __restrict__ gs,
                            const double2* __restrict__ twL, double* __restrict__ table) {
     extern __shared__ double sg[];  // [Lh+1][6]
     const int Lh = c_tp.Lh, L = c_tp.L, K = c_tp.K;
@@ -163,8 +356,9 @@ __global__ void k_line_dft(const int2* __restrict__ used, const double* __restri
     const double* src = gs + (size_t)di * (Lh + 1) * 6;
     for (int t = threadIdx.x; t < (Lh + 1) * 6; t += blockDim.x) sg[t] = src[t];
     __syncthreads();
-    const int2 d = used[di];
+    const int4 d = rep[di];
     const int ix = d.x - c_tp.box_x0, iy = d.y - c_tp.box_y0;
+    const int mx = -d.x - c_tp.box_x0, my = -d.y - c_tp.box_y0;  // -d, in the box where it is used
     for (int k = threadIdx.x; k < K; k += blockDim.x) {
         const double sgn = (k & 1) ? -1.0 : 1.0;
         double A0 = 0, A1 = 0, A2 = 0, A3 = 0, B4 = 0, B5 = 0;
@@ -183,13 +377,21 @@ __global__ void k_line_dft(const int2* __restrict__ used, const double* __restri
         }
         const double* g0 = sg;
         const double* gh = sg + Lh * 6;
+        double v[6];
+        v[0] = g0[0] + sgn * gh[0] + 2.0 * A0;
+        v[1] = g0[1] + sgn * gh[1] + 2.0 * A1;
+        v[2] = g0[2] + sgn * gh[2] + 2.0 * A2;
+        v[3] = g0[3] + sgn * gh[3] + 2.0 * A3;
+        v[4] = -2.0 * B4;
+        v[5] = -2.0 * B5;
         double* o = table + (((size_t)k * c_tp.Dy + iy) * c_tp.Dx + ix) * 6;
-        o[0] = g0[0] + sgn * gh[0] + 2.0 * A0;
-        o[1] = g0[1] + sgn * gh[1] + 2.0 * A1;
-        o[2] = g0[2] + sgn * gh[2] + 2.0 * A2;
-        o[3] = g0[3] + sgn * gh[3] + 2.0 * A3;
-        o[4] = -2.0 * B4;
-        o[5] = -2.0 * B5;
+#pragma unroll
+        for (int t = 0; t < 6; t++) o[t] = v[t];
+        if (d.z) {
+            double* q = table + (((size_t)k * c_tp.Dy + my) * c_tp.Dx + mx) * 6;
+#pragma unroll
+            for (int t = 0; t < 6; t++) q[t] = t < 4 ? v[t] : -v[t];
+        }
     }
 }
 
@@ -222,101 +424,119 @@ __global__ void k_derive_x2(const double* __restrict__ t64, float* __restrict__ 
 }  // namespace
 
 // The plan's medium and tabulation parameters into this file's constant memory (shared by every
-// plan: uploaded again before each use).
-static cudaError_t upload_tabulate_constants(Plan& P, cudaStream_t st) {
+// plan: uploaded again before each use).  The copies' sources live in the plan.
+static cudaError_t upload_tabulate_constants(Plan& P, int kind, cudaStream_t st) {
+    auto put = [&](const auto& symbol, const void* src, size_t bytes) {
+        return cudaMemcpyToSymbolAsync(symbol, src, bytes, 0, cudaMemcpyHostToDevice, st);
+    };
     cudaError_t e;
-    if ((e = cudaMemcpyToSymbolAsync(c_mat, &P.mat, sizeof(MaterialDev), 0, cudaMemcpyHostToDevice, st))) return e;
-    if ((e = cudaMemcpyToSymbolAsync(c_tp, &P.tp, sizeof(TabulateParams), 0, cudaMemcpyHostToDevice, st))) return e;
-    if (P.mat.kind == FBC_MATERIAL_CUBIC) {
-        static thread_local std::vector<double> qc, qs;
-        qc.assign(kMaxQuad, 0.0);
-        qs.assign(kMaxQuad, 0.0);
-        for (int q = 0; q < P.mat.nquad; q++) {
-            const double psi = M_PI * (double)q / (double)P.mat.nquad;
-            qc[q] = cos(psi);
-            qs[q] = sin(psi);
+    const int nq = P.mat.nquad;
+    if (kind != kGreenIso && P.tab_nodes.empty()) {
+        P.tab_nodes.assign((size_t)nq * 8, 0.0);  // [nq] cos, [nq] sin of psi, then [nq][6]
+        for (int q = 0; q < nq; q++) {
+            const double psi = M_PI * (double)q / (double)nq;
+            P.tab_nodes[q] = cos(psi), P.tab_nodes[nq + q] = sin(psi);
+            for (int j = 0; j < 3; j++) {
+                const double a = M_PI * (double)((2LL * (j + 1) * q) % (2LL * nq)) / (double)nq;
+                P.tab_nodes[(size_t)2 * nq + q * 6 + 2 * j] = cos(a);
+                P.tab_nodes[(size_t)2 * nq + q * 6 + 2 * j + 1] = sin(a);
+            }
         }
-        if ((e = cudaMemcpyToSymbolAsync(c_qcos, qc.data(), sizeof(double) * kMaxQuad, 0, cudaMemcpyHostToDevice, st)))
-            return e;
-        if ((e = cudaMemcpyToSymbolAsync(c_qsin, qs.data(), sizeof(double) * kMaxQuad, 0, cudaMemcpyHostToDevice, st)))
-            return e;
-        // the host vectors must outlive the asynchronous copies
-        if ((e = cudaStreamSynchronize(st))) return e;
+        // the constants scaled by a power of two to a largest magnitude in [1, 2): products of four
+        // determinants stay in range whatever the unit of stress
+        double top = 0.0;
+        for (int t = 0; t < 36; t++) top = std::max(top, std::fabs(P.mat.K[t]));
+        const double sc = std::ldexp(1.0, -std::ilogb(top));
+        P.tab_mat = P.mat;
+        for (int t = 0; t < 36; t++) P.tab_mat.K[t] = P.mat.K[t] * sc;
+        P.tab_pre = sc / (M_PI * (double)nq);
     }
-    return cudaSuccess;
+    if (kind == kGreenNodes) {
+        if ((e = put(c_qcos, P.tab_nodes.data(), sizeof(double) * nq))) return e;
+        if ((e = put(c_qsin, P.tab_nodes.data() + nq, sizeof(double) * nq))) return e;
+    }
+    if (kind == kGreenPoly) {
+        if ((e = put(c_node, P.tab_nodes.data() + 2 * (size_t)nq, sizeof(double) * 6 * nq))) return e;
+        if ((e = put(c_pre, &P.tab_pre, sizeof(double)))) return e;
+    }
+    if ((e = put(c_mat, kind == kGreenPoly ? &P.tab_mat : &P.mat, sizeof(MaterialDev)))) return e;
+    return put(c_tp, &P.tp, sizeof(TabulateParams));
 }
 
-cudaError_t launch_tabulate(Plan& P, cudaStream_t st) {
+// Stage 1 of nd listed differences from d0 on (ref: the images' reference sums).
+template <int KIND>
+static cudaError_t launch_periodic(Plan& P, int d0, int nd, double* ref, double* gs, cudaStream_t st) {
+    if (d0 == 0) k_reference<KIND><<<1, 64, 0, st>>>(ref);
+    const long long threads = (long long)nd * (P.L / 2 + 1);
+    k_periodic<KIND><<<(unsigned)((threads + 127) / 128), 128, 0, st>>>(P.d_rep + d0, nd, ref, gs);
+    return cudaGetLastError();
+}
+
+// Constants, the stage-1 buffer (differences in chunks of at most 256 MB) after the reference sums, and
+// `stage2(d0, nd, gs)` for every chunk.
+template <class F>
+static cudaError_t tabulate_chunks(Plan& P, int kind, cudaStream_t st, F stage2) {
     cudaError_t e;
-    if ((e = upload_tabulate_constants(P, st))) return e;
-    if (P.n_used == 0) return cudaSuccess;
-    const int Lh = P.L / 2;
-    // process the differences in chunks so the stage-1 buffer stays bounded
-    const size_t per_d = (size_t)(Lh + 1) * 6 * sizeof(double);
-    int chunk = (int)std::min<size_t>((size_t)P.n_used, std::max<size_t>(1, (size_t)256 << 20) / per_d);
-    if (chunk < 1) chunk = 1;
-    double* gs = nullptr;
-    if ((e = cudaMallocAsync((void**)&gs, per_d * chunk, st))) return e;
-    const size_t smem = per_d;
-    if (smem > 32 * 1024) {
-        if ((e = cudaFuncSetAttribute(k_line_dft, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem))) {
-            cudaFreeAsync(gs, st);
-            return e;
-        }
+    if ((e = upload_tabulate_constants(P, kind, st))) return e;
+    if (P.n_rep == 0) return cudaSuccess;
+    const size_t per_d = (size_t)(P.L / 2 + 1) * 6 * sizeof(double);
+    const size_t n_ref = kMaxRichImages * 6;
+    const int chunk = (int)std::min<size_t>((size_t)P.n_rep, std::max<size_t>(1, ((size_t)256 << 20) / per_d));
+    double* buf = nullptr;
+    if ((e = cudaMallocAsync((void**)&buf, n_ref * sizeof(double) + per_d * chunk, st))) return e;
+    double* gs = buf + n_ref;
+    for (int d0 = 0; d0 < P.n_rep && !e; d0 += chunk) {
+        const int nd = std::min(chunk, P.n_rep - d0);
+        e = kind == kGreenIso     ? launch_periodic<kGreenIso>(P, d0, nd, buf, gs, st)
+            : kind == kGreenNodes ? launch_periodic<kGreenNodes>(P, d0, nd, buf, gs, st)
+                                  : launch_periodic<kGreenPoly>(P, d0, nd, buf, gs, st);
+        if (!e) e = stage2(d0, nd, gs);
     }
-    for (int d0 = 0; d0 < P.n_used; d0 += chunk) {
-        const int nd = std::min(chunk, P.n_used - d0);
-        const long long threads = (long long)nd * (Lh + 1);
-        const int bs = 128;
-        k_periodic<<<(unsigned)((threads + bs - 1) / bs), bs, 0, st>>>(P.d_used + d0, nd, gs);
-        if ((e = cudaGetLastError())) break;
-        const int bt = std::min(256, std::max(32, ((P.K + 31) / 32) * 32));
-        k_line_dft<<<nd, bt, smem, st>>>(P.d_used + d0, gs, P.d_twL, P.d_table);
-        if ((e = cudaGetLastError())) break;
-    }
-    cudaError_t e2 = cudaFreeAsync(gs, st);
+    cudaError_t e2 = cudaFreeAsync(buf, st);
     return e ? e : e2;
 }
 
-// Stage-1 output of a chunk of used differences, rounded to FP32 and placed at each difference's
-// cell of the box: out[cell][s][6] for s = 0..L/2.
-__global__ void k_real_space_scatter(const int2* __restrict__ used, int n_used, const double* __restrict__ gs,
+cudaError_t launch_tabulate(Plan& P, cudaStream_t st) {
+    const size_t smem = (size_t)(P.L / 2 + 1) * 6 * sizeof(double);
+    if (smem > 32 * 1024) {
+        cudaError_t e = cudaFuncSetAttribute(k_line_dft, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e) return e;
+    }
+    const int kind = P.mat.kind == FBC_MATERIAL_ISOTROPIC ? kGreenIso : line_fp32(P.precision) ? kGreenNodes : kGreenPoly;
+    return tabulate_chunks(P, kind, st, [&](int d0, int nd, const double* gs) {
+        const int bt = std::min(256, std::max(32, ((P.K + 31) / 32) * 32));
+        k_line_dft<<<nd, bt, smem, st>>>(P.d_rep + d0, gs, P.d_twL, P.d_table);
+        return cudaGetLastError();
+    });
+}
+
+// Stage-1 output of a chunk of listed differences, rounded to FP32 and placed at each difference's
+// cell of the box (and its mirror's, the odd entries negated): out[cell][s][6] for s = 0..L/2.
+__global__ void k_real_space_scatter(const int4* __restrict__ rep, int n_rep, const double* __restrict__ gs,
                                      float* __restrict__ out) {
     const int Lh = c_tp.Lh;
     const long long per = (long long)(Lh + 1) * 6;
-    const long long total = (long long)n_used * per;
+    const long long total = (long long)n_rep * per;
     for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < total;
          t += (long long)gridDim.x * blockDim.x) {
         const int di = (int)(t / per);
         const long long r = t - (long long)di * per;
-        const int2 d = used[di];
-        const long long cell = (long long)(d.y - c_tp.box_y0) * c_tp.Dx + (d.x - c_tp.box_x0);
-        out[cell * per + r] = (float)gs[t];
+        const int4 d = rep[di];
+        const float v = (float)gs[t];
+        out[((long long)(d.y - c_tp.box_y0) * c_tp.Dx + (d.x - c_tp.box_x0)) * per + r] = v;
+        if (d.z) out[((long long)(-d.y - c_tp.box_y0) * c_tp.Dx + (-d.x - c_tp.box_x0)) * per + r] = r % 6 < 4 ? v : -v;
     }
 }
 
 cudaError_t launch_real_space_table(Plan& P, float* out, cudaStream_t st) {
-    cudaError_t e;
-    if ((e = upload_tabulate_constants(P, st))) return e;
-    const int Lh = P.L / 2;
     const size_t cells = (size_t)P.Dx * P.Dy;
-    if ((e = cudaMemsetAsync(out, 0, cells * (Lh + 1) * 6 * sizeof(float), st))) return e;
-    if (P.n_used == 0) return cudaSuccess;
-    const size_t per_d = (size_t)(Lh + 1) * 6 * sizeof(double);
-    int chunk = (int)std::min<size_t>((size_t)P.n_used, std::max<size_t>(1, (size_t)256 << 20) / per_d);
-    if (chunk < 1) chunk = 1;
-    double* gs = nullptr;
-    if ((e = cudaMallocAsync((void**)&gs, per_d * chunk, st))) return e;
-    for (int d0 = 0; d0 < P.n_used; d0 += chunk) {
-        const int nd = std::min(chunk, P.n_used - d0);
-        const long long threads = (long long)nd * (Lh + 1);
-        k_periodic<<<(unsigned)((threads + 127) / 128), 128, 0, st>>>(P.d_used + d0, nd, gs);
-        if ((e = cudaGetLastError())) break;
-        k_real_space_scatter<<<1216, 256, 0, st>>>(P.d_used + d0, nd, gs, out);
-        if ((e = cudaGetLastError())) break;
-    }
-    cudaError_t e2 = cudaFreeAsync(gs, st);
-    return e ? e : e2;
+    cudaError_t e = cudaMemsetAsync(out, 0, cells * (P.L / 2 + 1) * 6 * sizeof(float), st);
+    if (e) return e;
+    const int kind = P.mat.kind == FBC_MATERIAL_ISOTROPIC ? kGreenIso : kGreenNodes;
+    return tabulate_chunks(P, kind, st, [&](int d0, int nd, const double* gs) {
+        k_real_space_scatter<<<1216, 256, 0, st>>>(P.d_rep + d0, nd, gs, out);
+        return cudaGetLastError();
+    });
 }
 
 cudaError_t launch_derive_tables(Plan& P, int precision, cudaStream_t st) {
