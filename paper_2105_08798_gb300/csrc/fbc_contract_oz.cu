@@ -46,7 +46,7 @@
 //     others;
 //   * one thread streams the force operand, split once per apply (3 x 6 blocks
 //     of 64 x 16 bf16 per stage, 36 KB), with bulk copies into a ring of stages;
-//   * one thread issues 3 x 26 tcgen05.mma (M = 128, N = 64, K = 16) per stage
+//   * one warp (an elected lane) issues 3 x 26 tcgen05.mma (M = 128, N = 64, K = 16) per stage
 //     into the five accumulators;
 //   * at the start of every tile the builders drain the previous tile's group
 //     into their running double-float sums.
@@ -385,50 +385,37 @@ __global__ void __launch_bounds__(kThreads, 1) k_contract_oz(OzArgs O, int wl, i
             for (int j = max(0, il - kS); j < il; j++) tc::mbar_wait(&sy.bfull[j % kS], (uint32_t)(j / kS) & 1u);
         }
     } else if (warp == kMmaWarp) {
-        // ---- tensor-core issue: 3 x 26 products per stage ----
-        if (lane == 0) {
-            const uint32_t id = tc::idesc(1, kRows, kN);
-            const uint64_t dB0 = tc::sdesc(tc::smem_u32(sB), 128, kSBO);
-            for (int il = 0; il < n_it; il++) {
-                const int s = il % kS;
-                const uint32_t par = (uint32_t)(il / kS) & 1u;
-                if (!tc::wait_or_abort_sleep(&sy.bfull[s], par, &s_abort, wl, kSleepNs)) {
-                    s_abort = 1;
-                    break;
-                }
-                const uint64_t dBs = dB0 + (uint64_t)(((size_t)s * kChunk) >> 4);
-                const uint32_t ta0 = tmem + kAcol;
-                const bool first = (il % kStages) == 0;  // a new group overwrites the accumulators
-                bool stop = false;
+        // ---- tensor-core issue: 3 x 26 products per stage, from the whole warp (one elected lane issues) ----
+        const uint32_t el = tc::elect_one();
+        const uint32_t id = tc::idesc(1, kRows, kN);
+        const uint64_t dB0 = tc::sdesc(tc::smem_u32(sB), 128, kSBO);
+        bool stop = false;
+        for (int il = 0; il < n_it && !stop; il++) {
+            const int s = il % kS;
+            const uint32_t par = (uint32_t)(il / kS) & 1u;
+            stop = !__all_sync(0xffffffffu, tc::wait_or_abort_sleep(&sy.bfull[s], par, &s_abort, wl, kSleepNs));
+            if (stop) break;
+            const uint64_t dBs = dB0 + (uint64_t)(((size_t)s * kChunk) >> 4);
+            const uint32_t ta0 = tmem + kAcol;
+            const bool first = (il % kStages) == 0;  // a new group overwrites the accumulators
 #pragma unroll
-                for (int ci = 0; ci < 3; ci++) {
-                    // the A blocks of input component ci, stored by the builders while the others' products run
-                    if (!tc::wait_or_abort(&sy.afull[ci], (uint32_t)il & 1u, &s_abort, wl)) {
-                        stop = true;
-                        break;
-                    }
-                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            for (int ci = 0; ci < 3; ci++) {
+                // the A blocks of input component ci, stored by the builders while the others' products run
+                stop = !__all_sync(0xffffffffu, tc::wait_or_abort(&sy.afull[ci], (uint32_t)il & 1u, &s_abort, wl));
+                if (stop) break;
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
-                    for (int p = 0; p < kNPair; p++) {
-                        const uint32_t ta = ta0 + (uint32_t)(ci * kNS + oz_pi(p) - 1) * 8u;
-                        const uint64_t db = dBs + (uint64_t)(((uint32_t)(ci * kNS + oz_pj(p) - 1) * kBBlk) >> 4);
-                        const uint32_t dt = tmem + (uint32_t)oz_acc(p) * (uint32_t)kN;
-                        const uint32_t en = (first && ci == 0 && oz_first(p)) ? 0u : 1u;
-                        asm volatile(
-                            "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-                            "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(dt),
-                            "r"(ta), "l"(db), "r"(id), "r"(en));
-                    }
-                    tc::commit(&sy.aempty[ci]);
-                }
-                if (stop) {
-                    s_abort = 1;
-                    break;
-                }
-                tc::commit(&sy.empty[s]);
+                for (int p = 0; p < kNPair; p++)
+                    tc::mma_ts<false>(tmem + (uint32_t)oz_acc(p) * (uint32_t)kN,
+                                      ta0 + (uint32_t)(ci * kNS + oz_pi(p) - 1) * 8u,
+                                      dBs + (uint64_t)(((uint32_t)(ci * kNS + oz_pj(p) - 1) * kBBlk) >> 4), id,
+                                      (first && ci == 0 && oz_first(p)) ? 0u : 1u, el);
+                tc::commit_elected(&sy.aempty[ci], el);
             }
-            tc::commit(&sy.done);  // also after a stop: fires once the issued products are complete
+            if (!stop) tc::commit_elected(&sy.empty[s], el);
         }
+        if (stop) s_abort = 1;
+        tc::commit_elected(&sy.done, el);  // also after a stop: fires once the issued products are complete
     } else {
         // ---- builders (warps 0..7): table slices into tensor memory, drains, output ----
         const int tid = threadIdx.x;               // 0 .. 255

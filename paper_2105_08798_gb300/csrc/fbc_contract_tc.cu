@@ -17,7 +17,7 @@
 //   * the force operand X_0, X_1, X_2 was split once per apply by k_prep_b
 //     into the same layout, one contiguous chunk per (k, rhs group, stage);
 //     one thread streams each chunk in with a bulk copy (cp.async.bulk);
-//   * one thread issues the 9 block products per split-product pair with
+//   * one warp (an elected lane) issues the 9 block products per split-product pair with
 //     tcgen05.mma (M = 128, N = 2 R, K = 16 bf16 / 8 tf32) into three TMEM
 //     accumulators (one per output component); the -B13, -B23 entries use
 //     the instruction's negate-A bit; a commit to the stage's "empty" barrier
@@ -254,75 +254,57 @@ __device__ __forceinline__ void tc_item(const TcJob& J, const int4 wk, const uin
                 }
             }
         } else if (warp == kMmaWarp) {
-            // ---- tensor-core issue ----
-            if (lane == 0) {
-                const uint32_t id = idesc(C::FMT, kRows, NP), idn = id | (1u << 13);  // bit 13: negate A
-                // descriptor of B block 0 of stage 0; the others differ by (byte offset >> 4) in the address field
-                const uint64_t dB0 = sdesc(smem_u32(sB), 128, Lt::SBO);
-                const uint64_t dA0 = sdesc(smem_u32(sA), 128, Lt::SBO);
-                const uint32_t bblk16 = (uint32_t)(bblk >> 4);
-                int gpos = 0;  // position of the stage in its accumulation group
-                for (int il = 0; il < n_it; il++) {
-                    const uint32_t it = it_base + il;
-                    const int s = it % S;
-                    const uint32_t par = (it / S) & 1u;
-                    uint64_t* af = C::ATM ? &afull : &full[s];
-                    const uint32_t apar = C::ATM ? (it & 1u) : par;
-                    if (!wait_or_abort(af, apar, &s_abort, wl) || !wait_or_abort(&bfull[s], par, &s_abort, wl)) {
-                        s_abort = 1;
-                        break;
-                    }
-                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    const uint64_t dBs = dB0 + (uint64_t)((s * Lt::B_STAGE) >> 4);
-                    const uint64_t dAs = dA0 + (uint64_t)((s * Lt::A_STAGE) >> 4);
-                    // a new accumulation group starts by overwriting the accumulators
-                    const uint32_t first = gpos == 0 ? 0u : 1u;
-                    if (++gpos == gs) gpos = 0;
+            // ---- tensor-core issue, from the whole warp (one elected lane issues) ----
+            const uint32_t el = tc::elect_one();
+            const uint32_t id = idesc(C::FMT, kRows, NP), idn = id | (1u << 13);  // bit 13: negate A
+            // descriptor of B block 0 of stage 0; the others differ by (byte offset >> 4) in the address field
+            const uint64_t dB0 = sdesc(smem_u32(sB), 128, Lt::SBO);
+            const uint64_t dA0 = sdesc(smem_u32(sA), 128, Lt::SBO);
+            const uint32_t bblk16 = (uint32_t)(bblk >> 4);
+            int gpos = 0;  // position of the stage in its accumulation group
+            bool stop = false;
+            for (int il = 0; il < n_it; il++) {
+                const uint32_t it = it_base + il;
+                const int s = it % S;
+                const uint32_t par = (it / S) & 1u;
+                uint64_t* af = C::ATM ? &afull : &full[s];
+                const uint32_t apar = C::ATM ? (it & 1u) : par;
+                stop = !__all_sync(0xffffffffu, wait_or_abort(af, apar, &s_abort, wl) &&
+                                                    wait_or_abort(&bfull[s], par, &s_abort, wl));
+                if (stop) break;
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                const uint64_t dBs = dB0 + (uint64_t)((s * Lt::B_STAGE) >> 4);
+                const uint64_t dAs = dA0 + (uint64_t)((s * Lt::A_STAGE) >> 4);
+                // a new accumulation group starts by overwriting the accumulators
+                const uint32_t first = gpos == 0 ? 0u : 1u;
+                if (++gpos == gs) gpos = 0;
 #pragma unroll
-                    for (int co = 0; co < 3; co++)
+                for (int co = 0; co < 3; co++)
 #pragma unroll
-                        for (int ci = 0; ci < 3; ci++)
+                    for (int ci = 0; ci < 3; ci++)
 #pragma unroll
-                            for (int pr = 0; pr < C::NPROD; pr++)
+                        for (int pr = 0; pr < C::NPROD; pr++)
 #pragma unroll
-                                for (int ks = 0; ks < kKC / C::KMMA; ks++) {
-                                    constexpr int kEnt[3][3] = {{0, 1, 4}, {1, 2, 5}, {4, 5, 3}};
-                                    constexpr int kPa[6] = {0, 0, 1, 0, 2, 1}, kPb[6] = {0, 1, 0, 2, 0, 1};
-                                    const int ablk = kEnt[co][ci] * C::NS + kPa[pr];
-                                    const uint64_t db = dBs + (uint64_t)((ci * C::NS + kPb[pr]) * bblk16 + 16 * ks);
-                                    const uint32_t idd = (ci == 2 && co < 2) ? idn : id;
-                                    const uint32_t dt = tmem + (uint32_t)(co * NP);
-                                    // the first product into each accumulator overwrites it
-                                    const uint32_t en = (ci | pr | ks) ? 1u : first;
-                                    if (C::ATM) {
-                                        // A from tensor memory: block ablk, K step ks (8 columns per MMA)
-                                        const uint32_t ta = tmem + kAcol + (uint32_t)ablk * Lt::ACOLS + 8u * ks;
-                                        if (C::FMT == 2)
-                                            asm volatile(
-                                                "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-                                                "tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, p;\n}\n" ::"r"(dt),
-                                                "r"(ta), "l"(db), "r"(idd), "r"(en));
-                                        else
-                                            asm volatile(
-                                                "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-                                                "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(dt),
-                                                "r"(ta), "l"(db), "r"(idd), "r"(en));
-                                    } else {
-                                        const uint64_t da = dAs + (uint64_t)((ablk * Lt::ABLK + 256 * ks) >> 4);
-                                        if (C::FMT == 2)
-                                            asm volatile(
-                                                "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-                                                "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}\n" ::"r"(dt),
-                                                "l"(da), "l"(db), "r"(idd), "r"(en));
-                                        else
-                                            tc::mma_bf16(dt, da, db, idd, en);
-                                    }
-                                }
-                    if (C::ATM) tc::commit(&aempty);
-                    tc::commit(&empty[s]);
-                }
-                tc::commit(&done);  // also after a stop: fires once the issued products are complete
+                            for (int ks = 0; ks < kKC / C::KMMA; ks++) {
+                                constexpr int kEnt[3][3] = {{0, 1, 4}, {1, 2, 5}, {4, 5, 3}};
+                                constexpr int kPa[6] = {0, 0, 1, 0, 2, 1}, kPb[6] = {0, 1, 0, 2, 0, 1};
+                                const int ablk = kEnt[co][ci] * C::NS + kPa[pr];
+                                const uint64_t db = dBs + (uint64_t)((ci * C::NS + kPb[pr]) * bblk16 + 16 * ks);
+                                const uint32_t idd = (ci == 2 && co < 2) ? idn : id;
+                                const uint32_t dt = tmem + (uint32_t)(co * NP);
+                                // the first product into each accumulator overwrites it
+                                const uint32_t en = (ci | pr | ks) ? 1u : first;
+                                if (C::ATM)  // A from tensor memory: block ablk, K step ks (8 columns per MMA)
+                                    tc::mma_ts<C::FMT == 2>(dt, tmem + kAcol + (uint32_t)ablk * Lt::ACOLS + 8u * ks, db, idd,
+                                                            en, el);
+                                else
+                                    tc::mma_ss(dt, dAs + (uint64_t)((ablk * Lt::ABLK + 256 * ks) >> 4), db, idd, en, el);
+                            }
+                if (C::ATM) tc::commit_elected(&aempty, el);
+                tc::commit_elected(&empty[s], el);
             }
+            if (stop) s_abort = 1;
+            tc::commit_elected(&done, el);  // also after a stop: fires once the issued products are complete
         } else {
             // ---- builders (warps 0..7) ----
             const int tid = threadIdx.x;                  // 0 .. 255

@@ -87,6 +87,44 @@ __device__ __forceinline__ void commit(uint64_t* m) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(m)));
 }
 
+// Issue of products from a whole, converged warp: the warp runs the loop, and one elected lane's predicate
+// guards each instruction.  Issued from a branch that only one thread takes, a product cost 45 to 83 cycles
+// whatever its size (its operands then pass through per-thread registers); issued this way M = 128, K = 16
+// products of N columns take N / 2 cycles, the tensor pipe's rate, from N = 32 up.  Every lane keeps the same
+// elected lane for the kernel's lifetime: commits track the products of the thread that issued them.
+__device__ __forceinline__ uint32_t elect_one() {
+    uint32_t p;
+    asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}\n" : "=r"(p));
+    return p;
+}
+// D[tmem_d] (+)= A[tmem_a] B[db]: A from tensor memory, bf16 (TF32: tf32) operands
+template <bool TF32>
+__device__ __forceinline__ void mma_ts(uint32_t tmem_d, uint32_t tmem_a, uint64_t db, uint32_t id, uint32_t accum, uint32_t el) {
+    if (TF32)
+        asm volatile(
+            "{\n.reg .pred p, q;\nsetp.ne.b32 p, %4, 0;\nsetp.ne.b32 q, %5, 0;\n"
+            "@q tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, p;\n}\n" ::"r"(tmem_d),
+            "r"(tmem_a), "l"(db), "r"(id), "r"(accum), "r"(el));
+    else
+        asm volatile(
+            "{\n.reg .pred p, q;\nsetp.ne.b32 p, %4, 0;\nsetp.ne.b32 q, %5, 0;\n"
+            "@q tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(tmem_d),
+            "r"(tmem_a), "l"(db), "r"(id), "r"(accum), "r"(el));
+}
+// the same with A from shared memory (bf16)
+__device__ __forceinline__ void mma_ss(uint32_t tmem_d, uint64_t da, uint64_t db, uint32_t id, uint32_t accum, uint32_t el) {
+    asm volatile(
+        "{\n.reg .pred p, q;\nsetp.ne.b32 p, %4, 0;\nsetp.ne.b32 q, %5, 0;\n"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem_d),
+        "l"(da), "l"(db), "r"(id), "r"(accum), "r"(el));
+}
+__device__ __forceinline__ void commit_elected(uint64_t* m, uint32_t el) {
+    asm volatile(
+        "{\n.reg .pred q;\nsetp.ne.b32 q, %1, 0;\n"
+        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(smem_u32(m)), "r"(el)
+        : "memory");
+}
+
 // 16 consecutive FP32 accumulator columns of this thread's TMEM lane
 __device__ __forceinline__ void ld16(uint32_t taddr, float (&v)[16]) {
     uint32_t u[16];
