@@ -125,6 +125,8 @@ struct Plan {
     void* d_bprep = nullptr;
     size_t bprep_bytes = 0;
     int bprep_prec = -1;
+    int* d_off_oz = nullptr;  // FBC_PREC_BF16X6: [NIpad] x_b + oz_pitch * y_b of the sorted interface sites, [NPpad] row order
+    int oz_pitch = 0;         // row pitch of its cut sub-boxes
     int wait_limit = 0;  // polls per pipeline wait of the tensor-core contraction (0: the default bound)
     bool timing = false, timed_once = false;
     size_t table_bytes = 0, workspace_bytes = 0;
@@ -229,6 +231,7 @@ cudaError_t launch_contract_tc_batch(int precision, const TcJob* d_jobs, const i
 size_t contract_oz_smem(int HW);
 size_t contract_oz_prep_bytes(const Plan& P);
 int contract_oz_rhs_group();  // right-hand sides per CTA
+int contract_oz_layout(const Plan& P, int* rows);  // row pitch of its cut sub-boxes and the rows' order
 cudaError_t launch_contract_oz(const ContractArgs& A, const Plan& P, int n_rhs, cudaStream_t st);
 inline bool is_tensor_precision(int p) { return p == FBC_PREC_TF32 || p == FBC_PREC_BF16X2 || p == FBC_PREC_BF16X3; }
 int batch_rhs_block();

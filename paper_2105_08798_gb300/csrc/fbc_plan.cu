@@ -194,7 +194,7 @@ void free_plan(fbc::Plan& P) {
     void* bufs[] = {P.d_xy_p,  P.d_off_i,    P.d_bbox_a, P.d_bbox_b, P.d_perm_i, P.d_perm_p,
                     P.d_used,  P.d_rep,      P.d_tw,       P.d_twL,    P.d_twl,    P.d_table,  P.d_table32, P.d_table_x2, P.d_table_x2_k0,
                     P.d_fh,    P.d_uh,       P.d_part,   P.d_stage_f, P.d_stage_u, P.d_status, P.d_bprep,
-                    P.d_relax, P.d_uh32};
+                    P.d_relax, P.d_uh32, P.d_off_oz};
     for (void* b : bufs)
         if (b) cudaFree(b);
     for (auto& e : P.ev)
@@ -251,6 +251,19 @@ int ensure_derived(fbc::Plan& P, int precision) {
             P.d_bprep = q, P.bprep_bytes = want;
         }
         P.bprep_prec = precision;
+    }
+    if (precision == FBC_PREC_BF16X6 && !P.d_off_oz) {
+        int s = dev_alloc(&P.d_off_oz, P.NIpad + P.NPpad, acc, "off_oz");
+        if (s) return s;
+        std::vector<int> off(P.NIpad + P.NPpad);
+        P.oz_pitch = fbc::contract_oz_layout(P, off.data() + P.NIpad);
+        for (int t = 0; t < P.NIpad; t++) off[t] = P.xy_i_sorted[t].x + P.oz_pitch * P.xy_i_sorted[t].y;
+        cudaError_t e = cudaMemcpy(P.d_off_oz, off.data(), sizeof(int) * off.size(), cudaMemcpyHostToDevice);
+        if (e != cudaSuccess) {
+            cudaFree(P.d_off_oz);
+            P.d_off_oz = nullptr;
+            return cuda_fail(e, "off_oz");
+        }
     }
     if ((precision == FBC_PREC_F32X2 || precision == FBC_PREC_BF16X6) && !P.d_table_x2) {
         int s = dev_alloc(&P.d_table_x2, cells * 12, acc, "table_x2");

@@ -97,6 +97,7 @@ __device__ __forceinline__ uint32_t elect_one() {
     asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}\n" : "=r"(p));
     return p;
 }
+__device__ __forceinline__ uint64_t desc64(uint32_t lo, uint32_t hi) { return ((uint64_t)hi << 32) | lo; }
 // D[tmem_d] (+)= A[tmem_a] B[db]: A from tensor memory, bf16 (TF32: tf32) operands
 template <bool TF32>
 __device__ __forceinline__ void mma_ts(uint32_t tmem_d, uint32_t tmem_a, uint64_t db, uint32_t id, uint32_t accum, uint32_t el) {
@@ -185,6 +186,18 @@ __device__ __forceinline__ bool builders_sync_any(int flag) {
     return r != 0;
 }
 
+// the same among the NT threads of the slicer warps, on named barrier 2
+template <int NT>
+__device__ __forceinline__ bool slicers_sync_any(int flag) {
+    uint32_t r;
+    asm volatile(
+        "{\n.reg .pred p, q;\nsetp.ne.s32 p, %1, 0;\nbar.red.or.pred q, 2, %2, p;\nselp.u32 %0, 1, 0, q;\n}\n"
+        : "=r"(r)
+        : "r"(flag), "n"(NT)
+        : "memory");
+    return r != 0;
+}
+
 __device__ __forceinline__ void cp_async8(void* dst, const void* src, int src_bytes) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(src_bytes)
                  : "memory");
@@ -204,11 +217,32 @@ __device__ __forceinline__ void cp_async16z(void* dst, const void* src, int src_
                  : "memory");
 }
 
+// 4 consecutive FP32 accumulator columns of this thread's TMEM lane (no wait: follow with tcgen05.wait::ld)
+__device__ __forceinline__ void ld4_nowait(uint32_t taddr, uint32_t (&u)[4]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(u[0]), "=r"(u[1]), "=r"(u[2]), "=r"(u[3])
+                 : "r"(taddr));
+}
+
 // 8 consecutive FP32 accumulator columns of this thread's TMEM lane (no wait: follow with tcgen05.wait::ld)
 __device__ __forceinline__ void ld8_nowait(uint32_t taddr, uint32_t (&u)[8]) {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                  : "=r"(u[0]), "=r"(u[1]), "=r"(u[2]), "=r"(u[3]), "=r"(u[4]), "=r"(u[5]), "=r"(u[6]), "=r"(u[7])
                  : "r"(taddr));
+}
+
+// 32 (16) consecutive 32-bit columns of this thread's TMEM lane (no wait: follow with tcgen05.wait::st)
+__device__ __forceinline__ void st32(uint32_t taddr, const uint32_t* w) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};" ::"r"(taddr),
+        "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7]), "r"(w[8]), "r"(w[9]), "r"(w[10]), "r"(w[11]), "r"(w[12]), "r"(w[13]), "r"(w[14]), "r"(w[15]), "r"(w[16]), "r"(w[17]), "r"(w[18]), "r"(w[19]), "r"(w[20]), "r"(w[21]), "r"(w[22]), "r"(w[23]), "r"(w[24]), "r"(w[25]), "r"(w[26]), "r"(w[27]), "r"(w[28]), "r"(w[29]), "r"(w[30]), "r"(w[31])
+        : "memory");
+}
+__device__ __forceinline__ void st16(uint32_t taddr, const uint32_t* w) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};" ::"r"(taddr),
+        "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7]), "r"(w[8]), "r"(w[9]), "r"(w[10]), "r"(w[11]), "r"(w[12]), "r"(w[13]), "r"(w[14]), "r"(w[15])
+        : "memory");
 }
 
 __device__ __forceinline__ void mbar_arrive(uint64_t* m) {
