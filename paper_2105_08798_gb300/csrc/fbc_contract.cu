@@ -21,6 +21,7 @@
 // running total, FP64-accurate on the FP32 pipes).
 #include <cuda.h>  // CUtensorMap and its encoder's types (the encoder is reached through the runtime)
 
+#include "fbc_f32x2.cuh"
 #include "fbc_internal.cuh"
 #include "fbc_tc.cuh"
 
@@ -247,6 +248,48 @@ __device__ __forceinline__ void df_mac(float ah, float al, float xh, float xl, f
     E = __fadd_rn(E, __fadd_rn(lost, rest));
 }
 
+// df_mac on a pair of sums (the x and y' halves of a force, which meet the same table entry): the same operations,
+// so the same bits, in half the issue slots.  The 18 MACs of a pair-mode take 180 cycles of the FP32 pipe per warp; as
+// scalar instructions they also took 180 issue slots, beside which every load, address and loop instruction cost
+// time; packed they take 99.  4000 x 6000, L = 256, one right-hand side: 18.8 ms before, 17.0 ms now (0.82 of the pipe's
+// rate).
+// The rounded products come from scalar multiplies: the assembler joins a packed multiply and add into a packed FMA,
+// and with the sum's product unrounded the two-sum is no longer exact when S + p cancels (1e-8 instead of 1e-13).
+__device__ __forceinline__ void df_mac2(uint64_t ah, uint64_t al, uint64_t xh, uint64_t xl, uint64_t& S, uint64_t& E) {
+    float a, b, x, y;
+    upk2(ah, a, b);
+    upk2(xh, x, y);
+    const uint64_t p = pk2(__fmul_rn(a, x), __fmul_rn(b, y));
+    const uint64_t s = add2(S, p);
+    const uint64_t nb = sub2(S, s);  // -bb
+    const uint64_t lost = sub2(S, add2(s, nb));
+    uint64_t rest = fma2(ah, xh, nb);
+    rest = fma2(ah, xl, rest);
+    rest = fma2(al, xh, rest);
+    S = s;
+    E = add2(E, add2(lost, rest));
+}
+
+// The 18 products of one pair-mode: table entries (three records, each entry as hi, lo) times the force records
+// q_c = (x_c hi, y'_c hi, x_c lo, y'_c lo), into the pairs (x, y') of sums S[0..2], E[0..2].
+__device__ __forceinline__ void df_pair_mode(const float4& t0, const float4& t1, const float4& t2, const ulonglong2& q0,
+                                             const ulonglong2& q1, const ulonglong2& q2, uint64_t (&S)[3],
+                                             uint64_t (&E)[3]) {
+    const uint64_t a11h = pk2(t0.x, t0.x), a11l = pk2(t0.y, t0.y), a12h = pk2(t0.z, t0.z), a12l = pk2(t0.w, t0.w);
+    const uint64_t a22h = pk2(t1.x, t1.x), a22l = pk2(t1.y, t1.y), a33h = pk2(t1.z, t1.z), a33l = pk2(t1.w, t1.w);
+    const uint64_t b13h = pk2(t2.x, t2.x), b13l = pk2(t2.y, t2.y), b23h = pk2(t2.z, t2.z), b23l = pk2(t2.w, t2.w);
+    const uint64_t n2h = neg2(q2.x), n2l = neg2(q2.y);  // -b13, -b23 act on the third component: its sign instead
+    df_mac2(a11h, a11l, q0.x, q0.y, S[0], E[0]);
+    df_mac2(a12h, a12l, q0.x, q0.y, S[1], E[1]);
+    df_mac2(b13h, b13l, q0.x, q0.y, S[2], E[2]);
+    df_mac2(a12h, a12l, q1.x, q1.y, S[0], E[0]);
+    df_mac2(a22h, a22l, q1.x, q1.y, S[1], E[1]);
+    df_mac2(b23h, b23l, q1.x, q1.y, S[2], E[2]);
+    df_mac2(b13h, b13l, n2h, n2l, S[0], E[0]);
+    df_mac2(b23h, b23l, n2h, n2l, S[1], E[1]);
+    df_mac2(a33h, a33l, q2.x, q2.y, S[2], E[2]);
+}
+
 // T += (S + E) in double-float arithmetic (accurate sum of two pairs).
 __device__ __forceinline__ void df_fold(float& Thi, float& Tlo, float S, float E) {
     float s, e;
@@ -307,7 +350,7 @@ __device__ __forceinline__ bool x2_box_wait(const ContractArgs& A, const void* t
 }
 
 // Double-float: the table sub-box staged as above and each interface column as
-// four records: the (hi, lo) pairs of x and y' and off_b.
+// four records: x and y' by component (df_pair_mode) and off_b.
 // K0: the tile of the one-mode k = 0 launches (a separate instance, so that the
 // all-modes loop keeps its own code).
 template <int TA, int TB, bool K0>
@@ -335,9 +378,8 @@ __device__ __forceinline__ void tile_x2(const ContractArgs& A, int tA, int k, in
                 h[c] = (float)v;
                 l[c] = (float)(v - (double)h[c]);
             }
-            s_f[4 * j + 0] = make_float4(h[0], l[0], h[1], l[1]);
-            s_f[4 * j + 1] = make_float4(h[2], l[2], h[3], l[3]);
-            s_f[4 * j + 2] = make_float4(h[4], l[4], h[5], l[5]);
+#pragma unroll
+            for (int c = 0; c < 3; c++) s_f[4 * j + c] = make_float4(h[c], h[c + 3], l[c], l[c + 3]);
             s_f[4 * j + 3] = make_float4(__int_as_float(A.off_i[tB * TB + j]), 0.f, 0.f, 0.f);
         }
         if (x2_box_wait(A, tmap, bar, tB)) return;
@@ -350,44 +392,28 @@ __device__ __forceinline__ void tile_x2(const ContractArgs& A, int tA, int k, in
             // transform discards at k = 0, are written as zeros below)
 #pragma unroll 4
             for (int j = 0; j < TB; j++) {
-                const float4 f0 = s_f[4 * j], f2 = s_f[4 * j + 2], f3 = s_f[4 * j + 3];
+                const float4 f0 = s_f[4 * j], f1 = s_f[4 * j + 1], f2 = s_f[4 * j + 2], f3 = s_f[4 * j + 3];
                 const int idx = base - __float_as_int(f3.x);
                 const float4 t0 = s_tab[3 * idx], t1 = s_tab[3 * idx + 1];
-                df_mac(t0.x, t0.y, f0.x, f0.y, S[0], E[0]);
-                df_mac(t0.z, t0.w, f0.z, f0.w, S[0], E[0]);
-                df_mac(t0.z, t0.w, f0.x, f0.y, S[1], E[1]);
-                df_mac(t1.x, t1.y, f0.z, f0.w, S[1], E[1]);
-                df_mac(t1.z, t1.w, f2.z, f2.w, S[5], E[5]);
+                df_mac(t0.x, t0.y, f0.x, f0.z, S[0], E[0]);
+                df_mac(t0.z, t0.w, f1.x, f1.z, S[0], E[0]);
+                df_mac(t0.z, t0.w, f0.x, f0.z, S[1], E[1]);
+                df_mac(t1.x, t1.y, f1.x, f1.z, S[1], E[1]);
+                df_mac(t1.z, t1.w, f2.y, f2.w, S[5], E[5]);
             }
 #pragma unroll
             for (int c = 0; c < 6; c++) df_fold(Th[c], Tl[c], S[c], E[c]);
             continue;
         }
-#pragma unroll 2
+        uint64_t S2[3] = {0, 0, 0}, E2[3] = {0, 0, 0};
+#pragma unroll 8  // (2: 18.2 ms at 4000 x 6000, L = 256; the table reads of later columns cover the sums of earlier ones)
         for (int j = 0; j < TB; j++) {
-            const float4 f0 = s_f[4 * j], f1 = s_f[4 * j + 1], f2 = s_f[4 * j + 2], f3 = s_f[4 * j + 3];
-            const int idx = base - __float_as_int(f3.x);
-            const float4 t0 = s_tab[3 * idx], t1 = s_tab[3 * idx + 1], t2 = s_tab[3 * idx + 2];
-            // x = (f0.x, f0.y) (f0.z, f0.w) (f1.x, f1.y); y' = (f1.z, f1.w) (f2.x, f2.y) (f2.z, f2.w)
-            df_mac(t0.x, t0.y, f0.x, f0.y, S[0], E[0]);
-            df_mac(t0.z, t0.w, f0.z, f0.w, S[0], E[0]);
-            df_mac(-t2.x, -t2.y, f1.x, f1.y, S[0], E[0]);
-            df_mac(t0.z, t0.w, f0.x, f0.y, S[1], E[1]);
-            df_mac(t1.x, t1.y, f0.z, f0.w, S[1], E[1]);
-            df_mac(-t2.z, -t2.w, f1.x, f1.y, S[1], E[1]);
-            df_mac(t2.x, t2.y, f0.x, f0.y, S[2], E[2]);
-            df_mac(t2.z, t2.w, f0.z, f0.w, S[2], E[2]);
-            df_mac(t1.z, t1.w, f1.x, f1.y, S[2], E[2]);
-            df_mac(t0.x, t0.y, f1.z, f1.w, S[3], E[3]);
-            df_mac(t0.z, t0.w, f2.x, f2.y, S[3], E[3]);
-            df_mac(-t2.x, -t2.y, f2.z, f2.w, S[3], E[3]);
-            df_mac(t0.z, t0.w, f1.z, f1.w, S[4], E[4]);
-            df_mac(t1.x, t1.y, f2.x, f2.y, S[4], E[4]);
-            df_mac(-t2.z, -t2.w, f2.z, f2.w, S[4], E[4]);
-            df_mac(t2.x, t2.y, f1.z, f1.w, S[5], E[5]);
-            df_mac(t2.z, t2.w, f2.x, f2.y, S[5], E[5]);
-            df_mac(t1.z, t1.w, f2.z, f2.w, S[5], E[5]);
+            const ulonglong2* q = (const ulonglong2*)(s_f + 4 * j);
+            const int idx = base - __float_as_int(s_f[4 * j + 3].x);
+            df_pair_mode(s_tab[3 * idx], s_tab[3 * idx + 1], s_tab[3 * idx + 2], q[0], q[1], q[2], S2, E2);
         }
+#pragma unroll
+        for (int c = 0; c < 3; c++) upk2(S2[c], S[c], S[c + 3]), upk2(E2[c], E[c], E[c + 3]);
 #pragma unroll
         for (int c = 0; c < 6; c++) df_fold(Th[c], Tl[c], S[c], E[c]);
     }
@@ -445,9 +471,8 @@ __device__ __forceinline__ void tile_x2_rb(const ContractArgs& A, int tA, int k,
                     l[c] = (float)(v - (double)h[c]);
                 }
             }
-            s_f[3 * e + 0] = make_float4(h[0], l[0], h[1], l[1]);
-            s_f[3 * e + 1] = make_float4(h[2], l[2], h[3], l[3]);
-            s_f[3 * e + 2] = make_float4(h[4], l[4], h[5], l[5]);
+#pragma unroll
+            for (int c = 0; c < 3; c++) s_f[3 * e + c] = make_float4(h[c], h[c + 3], l[c], l[c + 3]);
         }
         for (int e = threadIdx.x; e < TB; e += NT) s_off[e] = A.off_i[tB * TB + e];
         if (x2_box_wait(A, tmap, bar, tB)) return;
@@ -458,45 +483,39 @@ __device__ __forceinline__ void tile_x2_rb(const ContractArgs& A, int tA, int k,
 #pragma unroll
             for (int c = 0; c < 6; c++) S[q][c] = E[q][c] = 0.f;
         const float4* fg = s_f + 3 * (g * RB) * TB;  // this group's right-hand sides
+        if (K0) {
 #pragma unroll 2
-        for (int j = 0; j < TB; j++) {
-            const int idx = base - s_off[j];
-            const float4 t0 = s_tab[3 * idx], t1 = s_tab[3 * idx + 1];
-            const float4 t2 = K0 ? make_float4(0, 0, 0, 0) : s_tab[3 * idx + 2];
+            for (int j = 0; j < TB; j++) {
+                const int idx = base - s_off[j];
+                const float4 t0 = s_tab[3 * idx], t1 = s_tab[3 * idx + 1];
 #pragma unroll
-            for (int q = 0; q < RB; q++) {
-                const float4* fq = fg + 3 * (q * TB + j);
-                const float4 f0 = fq[0], f2 = fq[2];
-                if (K0) {
+                for (int q = 0; q < RB; q++) {
                     // k = 0: the five non-zero products of tile_x2's k = 0 branch, in its order
-                    df_mac(t0.x, t0.y, f0.x, f0.y, S[q][0], E[q][0]);
-                    df_mac(t0.z, t0.w, f0.z, f0.w, S[q][0], E[q][0]);
-                    df_mac(t0.z, t0.w, f0.x, f0.y, S[q][1], E[q][1]);
-                    df_mac(t1.x, t1.y, f0.z, f0.w, S[q][1], E[q][1]);
-                    df_mac(t1.z, t1.w, f2.z, f2.w, S[q][5], E[q][5]);
-                    continue;
+                    const float4* fq = fg + 3 * (q * TB + j);
+                    const float4 f0 = fq[0], f1 = fq[1], f2 = fq[2];
+                    df_mac(t0.x, t0.y, f0.x, f0.z, S[q][0], E[q][0]);
+                    df_mac(t0.z, t0.w, f1.x, f1.z, S[q][0], E[q][0]);
+                    df_mac(t0.z, t0.w, f0.x, f0.z, S[q][1], E[q][1]);
+                    df_mac(t1.x, t1.y, f1.x, f1.z, S[q][1], E[q][1]);
+                    df_mac(t1.z, t1.w, f2.y, f2.w, S[q][5], E[q][5]);
                 }
-                const float4 f1 = fq[1];
-                // x = (f0.x, f0.y) (f0.z, f0.w) (f1.x, f1.y); y' = (f1.z, f1.w) (f2.x, f2.y) (f2.z, f2.w)
-                df_mac(t0.x, t0.y, f0.x, f0.y, S[q][0], E[q][0]);
-                df_mac(t0.z, t0.w, f0.z, f0.w, S[q][0], E[q][0]);
-                df_mac(-t2.x, -t2.y, f1.x, f1.y, S[q][0], E[q][0]);
-                df_mac(t0.z, t0.w, f0.x, f0.y, S[q][1], E[q][1]);
-                df_mac(t1.x, t1.y, f0.z, f0.w, S[q][1], E[q][1]);
-                df_mac(-t2.z, -t2.w, f1.x, f1.y, S[q][1], E[q][1]);
-                df_mac(t2.x, t2.y, f0.x, f0.y, S[q][2], E[q][2]);
-                df_mac(t2.z, t2.w, f0.z, f0.w, S[q][2], E[q][2]);
-                df_mac(t1.z, t1.w, f1.x, f1.y, S[q][2], E[q][2]);
-                df_mac(t0.x, t0.y, f1.z, f1.w, S[q][3], E[q][3]);
-                df_mac(t0.z, t0.w, f2.x, f2.y, S[q][3], E[q][3]);
-                df_mac(-t2.x, -t2.y, f2.z, f2.w, S[q][3], E[q][3]);
-                df_mac(t0.z, t0.w, f1.z, f1.w, S[q][4], E[q][4]);
-                df_mac(t1.x, t1.y, f2.x, f2.y, S[q][4], E[q][4]);
-                df_mac(-t2.z, -t2.w, f2.z, f2.w, S[q][4], E[q][4]);
-                df_mac(t2.x, t2.y, f1.z, f1.w, S[q][5], E[q][5]);
-                df_mac(t2.z, t2.w, f2.x, f2.y, S[q][5], E[q][5]);
-                df_mac(t1.z, t1.w, f2.z, f2.w, S[q][5], E[q][5]);
             }
+        } else {
+            uint64_t S2[RB][3] = {}, E2[RB][3] = {};
+#pragma unroll 2
+            for (int j = 0; j < TB; j++) {
+                const int idx = base - s_off[j];
+                const float4 t0 = s_tab[3 * idx], t1 = s_tab[3 * idx + 1], t2 = s_tab[3 * idx + 2];
+#pragma unroll
+                for (int q = 0; q < RB; q++) {
+                    const ulonglong2* fq = (const ulonglong2*)(fg + 3 * (q * TB + j));
+                    df_pair_mode(t0, t1, t2, fq[0], fq[1], fq[2], S2[q], E2[q]);
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < RB; q++)
+#pragma unroll
+                for (int c = 0; c < 3; c++) upk2(S2[q][c], S[q][c], S[q][c + 3]), upk2(E2[q][c], E[q][c], E[q][c + 3]);
         }
 #pragma unroll
         for (int q = 0; q < RB; q++)

@@ -66,6 +66,7 @@
 
 #include <algorithm>
 
+#include "fbc_f32x2.cuh"
 #include "fbc_internal.cuh"
 #include "fbc_tc.cuh"
 
@@ -289,34 +290,6 @@ struct OzSync {
     uint32_t tbase;
     volatile int abort;
 };
-
-// Packed FP32 pairs (two lanes per instruction, each rounded to nearest as the scalar operation).
-__device__ __forceinline__ uint64_t pk2(float a, float b) {
-    uint64_t r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-    return r;
-}
-__device__ __forceinline__ void upk2(uint64_t r, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(r)); }
-__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
-    uint64_t r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ uint64_t sub2(uint64_t a, uint64_t b) {
-    uint64_t r;
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
-    uint64_t r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
-    uint64_t r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
 
 // oz_split on two values at once: (hi, lo) pairs of two values, s a pair of powers of two.
 __device__ __forceinline__ void oz_split2(uint64_t hi, uint64_t lo, uint64_t s, uint64_t (&t)[kNS]) {
