@@ -260,20 +260,24 @@ int fbc_batch_create(fbc_plan* const* plans, int32_t n_plans, const double* cons
         const double per_tile = (double)P.n_tb * P.TA * P.TB;
         for (int k = 0; k < P.K; k++)
             for (int tA = 0; tA < P.n_ta; tA++) {
+                // an item per segment of the plan's interface sum: rhs | segment << 16
+                auto push = [&](std::vector<Item>& to, int r, const fbc::Seg& g, double rate) {
+                    for (int q = 0; q < g.n; q++)
+                        to.push_back({make_int4(i, k, tA, r | q << 16), per_tile / rate / g.n});
+                };
                 if (fbc::is_tensor_precision(prec) && k > 0) {
                     continue;  // the tensor-core items are built below for the batch's rhs group
-                } else if (fbc::is_tensor_precision(prec)) {  // k = 0 in double-float, as in a single plan
-                    for (int r = 0; r < R; r++) b->con_items[0].push_back({make_int4(i, k, tA, r), per_tile / 130.0});
-                } else if (prec == FBC_PREC_FP32 && k > 0) {
+                } else if (fbc::is_tensor_precision(prec) || (prec == FBC_PREC_FP32 && k == 0)) {
+                    // k = 0 in double-float, as in a single plan
+                    for (int r = 0; r < R; r++) push(b->con_items[0], r, P.seg0, 130.0);
+                } else if (prec == FBC_PREC_FP32) {
                     for (int rb = 0; rb < (R + RB - 1) / RB; rb++) {
                         const int cnt = std::min(RB, R - rb * RB);
                         b->con_items[1].push_back({make_int4(i, k, tA, rb), per_tile * cnt / 1500.0});
                     }
-                } else if (prec == FBC_PREC_FP32) {  // k = 0 in double-float
-                    for (int r = 0; r < R; r++) b->con_items[0].push_back({make_int4(i, k, tA, r), per_tile / 130.0});
                 } else {
-                    const double rate = (prec == FBC_PREC_F32X2) ? 130.0 : 34.0;
-                    for (int r = 0; r < R; r++) b->con_items[1].push_back({make_int4(i, k, tA, r), per_tile / rate});
+                    for (int r = 0; r < R; r++)
+                        push(b->con_items[1], r, prec == FBC_PREC_F32X2 ? P.segx2 : P.seg64, prec == FBC_PREC_F32X2 ? 130.0 : 34.0);
                 }
             }
         b->pair_modes += (double)P.n_p * P.n_i * P.K * R;

@@ -19,6 +19,9 @@
 // unevaluated pair of FP32 numbers -- Dekker's exact product via FMA, Knuth's
 // two-sum -- and each interface tile's partial folded into a double-float
 // running total, FP64-accurate on the FP32 pipes).
+#include <algorithm>
+#include <cmath>
+
 #include <cuda.h>  // CUtensorMap and its encoder's types (the encoder is reached through the runtime)
 
 #include "fbc_f32x2.cuh"
@@ -29,8 +32,29 @@ namespace fbc {
 namespace {
 
 
+// Counts a finished segment of tile `idx`; true for every thread of the CTA that finished the last of n, which then
+// sees the other CTAs' partial sums.  The counter is zero again afterwards.
+__device__ __forceinline__ bool seg_last(const ContractArgs& A, size_t idx, int n) {
+    __shared__ int s_last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        s_last = atomicAdd(&A.seg_cnt[idx], 1) == n - 1;
+        if (s_last) A.seg_cnt[idx] = 0;
+    }
+    __syncthreads();
+    const bool last = s_last;
+    if (last) __threadfence();
+    __syncthreads();  // s_last may be written again
+    return last;
+}
+// six partial sums of pad slot a, right-hand side r and mode kk (of Kp) in segment s
+__device__ __forceinline__ double* seg_slot(const ContractArgs& A, int s, int r, int kk, int Kp, int a) {
+    return A.seg_part + ((((size_t)s * A.max_rhs + r) * Kp + kk) * A.NPpad + a) * 6;
+}
+
 template <int TA, int TB>
-__device__ __forceinline__ void tile_fp64(const ContractArgs& A, int tA, int k, int r, void* smem_raw) {
+__device__ __forceinline__ void tile_fp64(const ContractArgs& A, int tA, int k, int r, int seg, void* smem_raw) {
     double* smem64 = (double*)smem_raw;
     const int HW = A.H * A.W;
     double* s_tab = smem64;              // [6][HW]
@@ -42,7 +66,10 @@ __device__ __forceinline__ void tile_fp64(const ContractArgs& A, int tA, int k, 
     double acc0 = 0, acc1 = 0, acc2 = 0, acc3 = 0, acc4 = 0, acc5 = 0;
     const double* fk = A.fh + ((size_t)r * A.K + k) * A.NIpad * 6;
     const double* tk = A.tab + (size_t)(k - A.kbase) * A.Dy * A.Dx * 6;
-    for (int tB = 0; tB < A.n_tb; tB++) {
+    const int c0 = seg * A.seg64.units * 16, c1 = A.seg64.n > 1 ? min(A.n_cols, c0 + A.seg64.units * 16) : A.NIpad;
+    for (int c = c0; c < c1;) {  // the segment's columns, interface tile by interface tile
+        const int tB = c / TB, j0 = c % TB, j1 = min(TB, j0 + c1 - c);
+        c += j1 - j0;
         const int4 bB = A.bbox_b[tB];
         const int ox = bA.x - bB.y, oy = bA.z - bB.w;
         __syncthreads();
@@ -63,7 +90,7 @@ __device__ __forceinline__ void tile_fp64(const ContractArgs& A, int tA, int k, 
         __syncthreads();
         const int base = (xa.x - ox) + A.W * (xa.y - oy);
 #pragma unroll 4
-        for (int j = 0; j < TB; j++) {
+        for (int j = j0; j < j1; j++) {
             const int idx = base - s_off[j];
             const double a11 = s_tab[idx], a12 = s_tab[HW + idx], a22 = s_tab[2 * HW + idx];
             const double a33 = s_tab[3 * HW + idx], b13 = s_tab[4 * HW + idx], b23 = s_tab[5 * HW + idx];
@@ -75,6 +102,16 @@ __device__ __forceinline__ void tile_fp64(const ContractArgs& A, int tA, int k, 
             acc3 = fma(a11, y0, fma(a12, y1, fma(-b13, y2, acc3)));
             acc4 = fma(a12, y0, fma(a22, y1, fma(-b23, y2, acc4)));
             acc5 = fma(b13, y0, fma(b23, y1, fma(a33, y2, acc5)));
+        }
+    }
+    if (A.seg64.n > 1) {
+        double* p = seg_slot(A, seg, r, k, A.K, a);
+        p[0] = acc0, p[1] = acc1, p[2] = acc2, p[3] = acc3, p[4] = acc4, p[5] = acc5;
+        if (!seg_last(A, ((size_t)r * A.K + k) * A.n_ta + tA, A.seg64.n)) return;
+        acc0 = acc1 = acc2 = acc3 = acc4 = acc5 = 0.0;
+        for (int t = 0; t < A.seg64.n; t++) {
+            const double* q = seg_slot(A, t, r, k, A.K, a);
+            acc0 += q[0], acc1 += q[1], acc2 += q[2], acc3 += q[3], acc4 += q[4], acc5 += q[5];
         }
     }
     double* o = A.uh + (((size_t)r * A.K + k) * A.NPpad + a) * 6;
@@ -299,6 +336,21 @@ __device__ __forceinline__ void df_fold(float& Thi, float& Tlo, float S, float E
     Tlo = __fsub_rn(e, __fsub_rn(Thi, s));
 }
 
+// The segments' partial totals of one output column, folded in order.
+__device__ __forceinline__ void df_fold_segments(const ContractArgs& A, int n, int r, int kk, int Kp, int a, float (&Th)[6],
+                                                 float (&Tl)[6]) {
+#pragma unroll
+    for (int c = 0; c < 6; c++) Th[c] = Tl[c] = 0.f;
+    for (int t = 0; t < n; t++) {
+        const float2* q = (const float2*)seg_slot(A, t, r, kk, Kp, a);
+#pragma unroll
+        for (int c = 0; c < 6; c++) {
+            const float2 v = q[c];
+            df_fold(Th[c], Tl[c], v.x, v.y);
+        }
+    }
+}
+
 // Double-float sub-box staging.  The table holds each entry as three 16-byte
 // records (a11h, a11l, a12h, a12l), (a22h, a22l, a33h, a33l), (b13h, b13l,
 // b23h, b23l), the layout kept in shared memory, so the W x H sub-box of a
@@ -353,9 +405,15 @@ __device__ __forceinline__ bool x2_box_wait(const ContractArgs& A, const void* t
 // four records: x and y' by component (df_pair_mode) and off_b.
 // K0: the tile of the one-mode k = 0 launches (a separate instance, so that the
 // all-modes loop keeps its own code).
-template <int TA, int TB, bool K0>
-__device__ __forceinline__ void tile_x2(const ContractArgs& A, int tA, int k, int r, void* smem_raw,
+// SEG: the plan's sum is in segments and this tile sums segment `seg` (an instance of its own, so that whole sums keep
+// their code: 17.6 against 17.9 ms at 4000 x 6000, L = 256).
+template <int TA, int TB, bool K0, bool SEG>
+__device__ __forceinline__ void tile_x2(const ContractArgs& A, int tA, int k, int r, int seg, void* smem_raw,
                                         const void* tmap = nullptr, uint64_t* bar = nullptr) {
+    const Seg& sg = K0 ? A.seg0 : A.segx2;
+    const bool split = SEG && sg.n > 1;
+    const int t0 = split ? seg * sg.units / (TB / 16) : 0;
+    const int t1 = split ? min(A.n_tb, t0 + sg.units / (TB / 16)) : A.n_tb;
     float4* smemx2 = (float4*)smem_raw;
     const int HW = A.H * A.W;
     float4* s_tab = smemx2;            // [HW][3]
@@ -365,7 +423,7 @@ __device__ __forceinline__ void tile_x2(const ContractArgs& A, int tA, int k, in
     const int4 bA = A.bbox_a[tA];
     float Th[6] = {0, 0, 0, 0, 0, 0}, Tl[6] = {0, 0, 0, 0, 0, 0};
     const double* fk = A.fh + ((size_t)r * A.K + k) * A.NIpad * 6;
-    for (int tB = 0; tB < A.n_tb; tB++) {
+    for (int tB = t0; tB < t1; tB++) {
         const int4 bB = A.bbox_b[tB];
         const int ox = bA.x - bB.y, oy = bA.z - bB.w;
         __syncthreads();
@@ -382,7 +440,10 @@ __device__ __forceinline__ void tile_x2(const ContractArgs& A, int tA, int k, in
             for (int c = 0; c < 3; c++) s_f[4 * j + c] = make_float4(h[c], h[c + 3], l[c], l[c + 3]);
             s_f[4 * j + 3] = make_float4(__int_as_float(A.off_i[tB * TB + j]), 0.f, 0.f, 0.f);
         }
-        if (x2_box_wait(A, tmap, bar, tB)) return;
+        if (x2_box_wait(A, tmap, bar, tB - t0)) {
+            if (split) seg_last(A, ((size_t)r * (K0 ? 1 : A.K) + (K0 ? 0 : k)) * A.n_ta + tA, sg.n);
+            return;
+        }
         const int base = (xa.x - ox) + A.W * (xa.y - oy);
         float S[6] = {0, 0, 0, 0, 0, 0}, E[6] = {0, 0, 0, 0, 0, 0};
         if (K0) {
@@ -417,6 +478,14 @@ __device__ __forceinline__ void tile_x2(const ContractArgs& A, int tA, int k, in
 #pragma unroll
         for (int c = 0; c < 6; c++) df_fold(Th[c], Tl[c], S[c], E[c]);
     }
+    if (split) {
+        const int kk = K0 ? 0 : k, Kp = K0 ? 1 : A.K;
+        float2* p = (float2*)seg_slot(A, seg, r, kk, Kp, a);
+#pragma unroll
+        for (int c = 0; c < 6; c++) p[c] = make_float2(Th[c], Tl[c]);
+        if (!seg_last(A, ((size_t)r * Kp + kk) * A.n_ta + tA, sg.n)) return;
+        df_fold_segments(A, sg.n, r, kk, Kp, a, Th, Tl);
+    }
     double* o = A.uh + (((size_t)r * A.K + k) * A.NPpad + a) * 6;
 #pragma unroll
     for (int c = 0; c < 6; c++) o[c] = (double)Th[c] + (double)Tl[c];
@@ -435,9 +504,13 @@ __device__ __forceinline__ void tile_x2(const ContractArgs& A, int tA, int k, in
 // those of tile_x2, so each right-hand side gets the same bits as from the
 // one-rhs tile.  grid.z = ceil(n_rhs / (NG RB)); force records [NG RB][TB][3]
 // (hi/lo pairs of x and y').
-template <int TA, int TB, int NG, int RB, bool K0>
-__device__ __forceinline__ void tile_x2_rb(const ContractArgs& A, int tA, int k, int rb, int n_rhs, void* smem_raw,
-                                           const void* tmap, uint64_t* bar) {
+template <int TA, int TB, int NG, int RB, bool K0, bool SEG>
+__device__ __forceinline__ void tile_x2_rb(const ContractArgs& A, int tA, int k, int rb, int n_rhs, int seg,
+                                           void* smem_raw, const void* tmap, uint64_t* bar) {
+    const Seg& sg = K0 ? A.seg0 : A.segx2;
+    const bool split = SEG && sg.n > 1;
+    const int t0 = split ? seg * sg.units / (TB / 16) : 0;
+    const int t1 = split ? min(A.n_tb, t0 + sg.units / (TB / 16)) : A.n_tb;
     constexpr int NT = TA * NG, NR = NG * RB;
     float4* smemx2 = (float4*)smem_raw;
     const int HW = A.H * A.W;
@@ -454,7 +527,8 @@ __device__ __forceinline__ void tile_x2_rb(const ContractArgs& A, int tA, int k,
     for (int q = 0; q < RB; q++)
 #pragma unroll
         for (int c = 0; c < 6; c++) Th[q][c] = Tl[q][c] = 0.f;
-    for (int tB = 0; tB < A.n_tb; tB++) {
+    const int kk = K0 ? 0 : k, Kp = K0 ? 1 : A.K;
+    for (int tB = t0; tB < t1; tB++) {
         const int4 bB = A.bbox_b[tB];
         const int ox = bA.x - bB.y, oy = bA.z - bB.w;
         __syncthreads();
@@ -475,7 +549,10 @@ __device__ __forceinline__ void tile_x2_rb(const ContractArgs& A, int tA, int k,
             for (int c = 0; c < 3; c++) s_f[3 * e + c] = make_float4(h[c], h[c + 3], l[c], l[c + 3]);
         }
         for (int e = threadIdx.x; e < TB; e += NT) s_off[e] = A.off_i[tB * TB + e];
-        if (x2_box_wait(A, tmap, bar, tB)) return;
+        if (x2_box_wait(A, tmap, bar, tB - t0)) {
+            if (split) seg_last(A, ((size_t)r0 * Kp + kk) * A.n_ta + tA, sg.n);
+            return;
+        }
         const int base = (xa.x - ox) + A.W * (xa.y - oy);
         float S[RB][6], E[RB][6];
 #pragma unroll
@@ -522,6 +599,22 @@ __device__ __forceinline__ void tile_x2_rb(const ContractArgs& A, int tA, int k,
 #pragma unroll
             for (int c = 0; c < 6; c++) df_fold(Th[q][c], Tl[q][c], S[q][c], E[q][c]);
     }
+    if (split) {
+#pragma unroll
+        for (int q = 0; q < RB; q++) {
+            const int r = r0 + g * RB + q;
+            if (r >= n_rhs) break;
+            float2* p = (float2*)seg_slot(A, seg, r, kk, Kp, a);
+#pragma unroll
+            for (int c = 0; c < 6; c++) p[c] = make_float2(Th[q][c], Tl[q][c]);
+        }
+        if (!seg_last(A, ((size_t)r0 * Kp + kk) * A.n_ta + tA, sg.n)) return;
+#pragma unroll
+        for (int q = 0; q < RB; q++) {
+            const int r = r0 + g * RB + q;
+            if (r < n_rhs) df_fold_segments(A, sg.n, r, kk, Kp, a, Th[q], Tl[q]);
+        }
+    }
 #pragma unroll
     for (int q = 0; q < RB; q++) {
         const int r = r0 + g * RB + q;
@@ -538,7 +631,7 @@ __device__ __forceinline__ void tile_x2_rb(const ContractArgs& A, int tA, int k,
 template <int TA, int TB>
 __global__ void __launch_bounds__(TA) k_contract_fp64(ContractArgs A) {
     extern __shared__ float4 smem_raw[];
-    tile_fp64<TA, TB>(A, blockIdx.x, A.k0 + blockIdx.y, blockIdx.z, smem_raw);
+    tile_fp64<TA, TB>(A, blockIdx.x, A.k0 + blockIdx.y, blockIdx.z / A.seg64.n, blockIdx.z % A.seg64.n, smem_raw);
 }
 template <int TA, int TB>
 __global__ void __launch_bounds__(TA) k_contract_fp32(ContractArgs A) {
@@ -562,28 +655,31 @@ __device__ __forceinline__ float4* x2_smem_setup(float4* smem_raw, uint64_t* bar
     const uint32_t pad = (128u - (tc::smem_u32(smem_raw) & 127u)) & 127u;
     return (float4*)((char*)smem_raw + pad);
 }
-template <int TA, int TB, bool K0, bool TMA>
+template <int TA, int TB, bool K0, bool TMA, bool SEG>
 __global__ void __launch_bounds__(TA) k_contract_x2(ContractArgs A, const __grid_constant__ CUtensorMap tm) {
     extern __shared__ float4 smem_raw[];
     __shared__ uint64_t bar;
     float4* smem = x2_smem_setup(smem_raw, &bar, TMA);
-    tile_x2<TA, TB, K0>(A, blockIdx.x, A.k0 + blockIdx.y, blockIdx.z, smem, TMA ? &tm : nullptr, &bar);
+    const int n = SEG ? (K0 ? A.seg0.n : A.segx2.n) : 1;
+    tile_x2<TA, TB, K0, SEG>(A, blockIdx.x, A.k0 + blockIdx.y, blockIdx.z / n, blockIdx.z % n, smem, TMA ? &tm : nullptr, &bar);
 }
 // grid (pad tiles, rhs groups, modes): the modes outermost, so the CTAs of all rhs groups of one mode run
 // together and read that mode's table slice from L2
-template <int TA, int TB, int NG, int RB, bool K0, bool TMA>
+template <int TA, int TB, int NG, int RB, bool K0, bool TMA, bool SEG>
 __global__ void __launch_bounds__(TA * NG) k_contract_x2_rb(ContractArgs A, const __grid_constant__ CUtensorMap tm,
                                                             int n_rhs) {
     extern __shared__ float4 smem_raw[];
     __shared__ uint64_t bar;
     float4* smem = x2_smem_setup(smem_raw, &bar, TMA);
-    tile_x2_rb<TA, TB, NG, RB, K0>(A, blockIdx.x, A.k0 + blockIdx.z, blockIdx.y, n_rhs, smem, TMA ? &tm : nullptr,
-                                   &bar);
+    const int n = SEG ? (K0 ? A.seg0.n : A.segx2.n) : 1;
+    tile_x2_rb<TA, TB, NG, RB, K0, SEG>(A, blockIdx.x, A.k0 + blockIdx.z, blockIdx.y / n, n_rhs, blockIdx.y % n, smem,
+                                   TMA ? &tm : nullptr, &bar);
 }
 
 // ---- batched: one persistent launch drains a cost-sorted work list ----------
-// Item (inst, k, pad tile, r): r is a right-hand side, or a block of RB
-// right-hand sides for the multi-rhs FP32 tile (k >= 1).  CTAs take items
+// Item (inst, k, pad tile, r): r is a right-hand side (with the segment in the
+// upper 16 bits), or a block of RB right-hand sides for the multi-rhs FP32 tile
+// (k >= 1).  CTAs take items
 // from a global counter with atomicAdd; no CTA ever waits for another.
 constexpr int kBatchRB = 8;
 template <int TA, int TB, int PREC, int PHASE>
@@ -602,11 +698,11 @@ __global__ void __launch_bounds__(TA) k_batch_contract(const ContractArgs* __res
         const int4 w = items[it];
         const ContractArgs A = args[w.x];
         if (PREC == FBC_PREC_FP64) {
-            tile_fp64<TA, TB>(A, w.z, w.y, w.w, smem_raw);
+            tile_fp64<TA, TB>(A, w.z, w.y, w.w & 0xffff, w.w >> 16, smem_raw);
         } else if (PREC == FBC_PREC_F32X2) {
-            tile_x2<TA, TB, false>(A, w.z, w.y, w.w, smem_raw);
+            tile_x2<TA, TB, false, true>(A, w.z, w.y, w.w & 0xffff, w.w >> 16, smem_raw);
         } else if (PHASE == 0) {
-            tile_x2<TA, TB, true>(A, w.z, w.y, w.w, smem_raw);  // the k = 0 items
+            tile_x2<TA, TB, true, true>(A, w.z, w.y, w.w & 0xffff, w.w >> 16, smem_raw);  // the k = 0 items
         } else {
             tile_fp32_rb<TA, TB, kBatchRB>(A, w.z, w.y, w.w, n_rhs_arr[w.x], smem_raw);
         }
@@ -674,25 +770,30 @@ cudaError_t launch_one(KernelT kern, const ContractArgs& A, dim3 grid, int threa
 // The double-float contraction of every mode (n_modes = K) or of the k = 0 mode alone (n_modes = 0:
 // the one-mode instances).  Both tiles take the sub-box by TMA where the map can be made (measured
 // faster than thread staging in each); otherwise the thread-staged instances run.
-template <bool K0, bool TMA>
+template <bool K0, bool TMA, bool SEG>
 cudaError_t launch_x2_instance(Plan& P, const ContractArgs& A, int n_modes, int n_rhs, const CUtensorMap& tm,
                                cudaStream_t st) {
+    const int n = SEG ? (K0 ? A.seg0.n : A.segx2.n) : 1;
     if (n_rhs >= 2) {
-        return launch_one(k_contract_x2_rb<kTileA, kTileB, kX2NG, kX2RB, K0, TMA>, A,
-                          dim3(P.n_ta, (n_rhs + kX2R - 1) / kX2R, n_modes), kTileA * kX2NG, x2_rb_smem(P), st, tm,
+        return launch_one(k_contract_x2_rb<kTileA, kTileB, kX2NG, kX2RB, K0, TMA, SEG>, A,
+                          dim3(P.n_ta, (n_rhs + kX2R - 1) / kX2R * n, n_modes), kTileA * kX2NG, x2_rb_smem(P), st, tm,
                           n_rhs);
     }
-    return launch_one(k_contract_x2<kTileA, kTileB, K0, TMA>, A, dim3(P.n_ta, n_modes, n_rhs), kTileA, x2_smem(P), st,
-                      tm);
+    return launch_one(k_contract_x2<kTileA, kTileB, K0, TMA, SEG>, A, dim3(P.n_ta, n_modes, n_rhs * n), kTileA, x2_smem(P),
+                      st, tm);
+}
+template <bool K0>
+cudaError_t launch_x2_modes(Plan& P, const ContractArgs& A, int n_modes, int n_rhs, cudaStream_t st) {
+    CUtensorMap tm{};
+    const bool tma = encode_x2_map(A, A.tabx2 == P.d_table_x2 ? P.K : 1, &tm), seg = (K0 ? A.seg0.n : A.segx2.n) > 1;
+    if (tma)
+        return seg ? launch_x2_instance<K0, true, true>(P, A, n_modes, n_rhs, tm, st)
+                   : launch_x2_instance<K0, true, false>(P, A, n_modes, n_rhs, tm, st);
+    return seg ? launch_x2_instance<K0, false, true>(P, A, n_modes, n_rhs, tm, st)
+               : launch_x2_instance<K0, false, false>(P, A, n_modes, n_rhs, tm, st);
 }
 cudaError_t launch_contract_x2(Plan& P, const ContractArgs& A, int n_modes, int n_rhs, cudaStream_t st) {
-    CUtensorMap tm{};
-    const bool tma = encode_x2_map(A, A.tabx2 == P.d_table_x2 ? P.K : 1, &tm);
-    if (n_modes == 0)
-        return tma ? launch_x2_instance<true, true>(P, A, 1, n_rhs, tm, st)
-                   : launch_x2_instance<true, false>(P, A, 1, n_rhs, tm, st);
-    return tma ? launch_x2_instance<false, true>(P, A, n_modes, n_rhs, tm, st)
-               : launch_x2_instance<false, false>(P, A, n_modes, n_rhs, tm, st);
+    return n_modes == 0 ? launch_x2_modes<true>(P, A, 1, n_rhs, st) : launch_x2_modes<false>(P, A, n_modes, n_rhs, st);
 }
 
 }  // namespace
@@ -703,7 +804,7 @@ cudaError_t launch_contract(Plan& P, int n_rhs, cudaStream_t st) {
     const size_t s64 = contract_smem<double>(P, kTileB, 8);
     if (s64 > 220 * 1024) return cudaErrorInvalidConfiguration;
     if (P.precision == FBC_PREC_FP64) {
-        return launch_one(k_contract_fp64<kTileA, kTileB>, A, dim3(P.n_ta, P.K, n_rhs), kTileA, s64, st);
+        return launch_one(k_contract_fp64<kTileA, kTileB>, A, dim3(P.n_ta, P.K, n_rhs * A.seg64.n), kTileA, s64, st);
     }
     if (P.precision == FBC_PREC_FP32) {
         // logarithmic k = 0 mode in double-float (FP64-accurate), the rest in FP32
@@ -748,7 +849,47 @@ ContractArgs make_contract_args(const Plan& P) {
     A.n_tb = P.n_tb, A.K = P.K, A.Dx = P.Dx, A.Dy = P.Dy, A.box_x0 = P.box_x0, A.box_y0 = P.box_y0;
     A.W = P.W, A.H = P.H, A.NIpad = P.NIpad, A.NPpad = P.NPpad, A.k0 = 0, A.kbase = 0;
     A.status = P.d_status;
+    A.seg64 = P.seg64, A.segx2 = P.segx2, A.seg0 = P.seg0;
+    A.n_cols = (P.n_i + 15) / 16 * 16, A.n_ta = P.n_ta, A.max_rhs = P.opt.max_rhs;
+    A.seg_part = P.d_seg_part, A.seg_cnt = P.d_seg_cnt;
     return A;
+}
+
+// Segments of a sum over `units` runs of 16 columns for `ctas` tiles, in multiples of `step` units (4: whole interface
+// tiles): enough for `target` CTAs, of the next few counts the one that divides best, at most 16.
+static Seg choose_segments(double ctas, int units, int step, int target) {
+    Seg best;
+    const int steps = (units + step - 1) / step;
+    const int want = std::min((int)std::ceil(target / ctas), std::min(steps, 16));
+    int waste = 0;
+    for (int n = want; n >= 2 && n <= std::min(want + 2, std::min(steps, 16)); n++) {
+        const int per = (steps + n - 1) / n, cnt = (steps + per - 1) / per;
+        if (best.n == 1 || per * cnt - steps < waste) best.units = per * step, best.n = cnt, waste = per * cnt - steps;
+    }
+    return best;
+}
+
+// Where the line lies: a tile's CTA has four warps, and an SM needs about three of them to keep the FP64 pipe (two of
+// them, by shared memory, the FP32 pipe) busy, so plans with fewer than 456 FP64 tiles or 912 double-float ones (six an
+// SM: the last of few waves is shared out) are split.  200 x 300 columns, L = 16, FP64: 27 CTAs with a chain of 200
+// columns each take 181 us, 41 us in 16-column segments.  Double-float, 1000 x 1500 columns, L = 64: 396 CTAs take 365 us,
+// 1584 take 324; k = 0 of 3001 x 4502 columns with 16 right-hand sides: 144 CTAs 667 us, 864 take 548.
+size_t contract_segments(Plan& P, size_t* counters) {
+    const int units = (P.n_i + 15) / 16, groups = (P.opt.max_rhs + kX2R - 1) / kX2R;
+    P.seg64 = choose_segments((double)P.n_ta * P.K * P.opt.max_rhs, units, 1, 456);
+    if (P.seg64.n > 1 && P.seg64.units > 2) P.seg64 = choose_segments((double)P.n_ta * P.K * P.opt.max_rhs, units, 4, 456);
+    P.segx2 = choose_segments((double)P.n_ta * P.K * groups, units, 4, 912);
+    P.seg0 = choose_segments((double)P.n_ta * groups, units, 4, 608);
+    const size_t per_mode = (size_t)P.opt.max_rhs * P.NPpad * 6;
+    size_t part = 0;
+    *counters = 0;
+    auto need = [&](const Seg& g, int modes) {
+        if (g.n < 2) return;
+        part = std::max(part, per_mode * modes * g.n);
+        *counters = std::max(*counters, (size_t)P.opt.max_rhs * modes * P.n_ta);
+    };
+    need(P.seg64, P.K), need(P.segx2, P.K), need(P.seg0, 1);
+    return part;
 }
 
 cudaError_t launch_contract_x2_k0(Plan& P, const ContractArgs& A, int n_rhs, cudaStream_t st) {

@@ -55,6 +55,14 @@ struct TabulateParams {
     int box_x0, box_y0, Dx, Dy;
 };
 
+// Segments of the interface sum for plans whose (pad tile, mode, rhs) tiles leave SMs idle: n segments of `units` runs
+// of 16 interface columns, each summed on its own and folded in order by the CTA that finishes last.  A plan's
+// segments depend on the plan alone, so every way to run it (one right-hand side or several, alone or in a batch)
+// adds in the same order.
+struct Seg {
+    int units = 0, n = 1;
+};
+
 struct FftGrid;  // in-plane FFT form (fbc_fft2d.cu)
 
 struct Plan {
@@ -127,6 +135,9 @@ struct Plan {
     int bprep_prec = -1;
     int* d_off_oz = nullptr;  // FBC_PREC_BF16X6: [NIpad] x_b + oz_pitch * y_b of the sorted interface sites, [NPpad] row order
     int oz_pitch = 0;         // row pitch of its cut sub-boxes
+    Seg seg64, segx2, seg0;        // segments of the interface sum (small plans)
+    double* d_seg_part = nullptr;  // their partial sums and counters
+    int* d_seg_cnt = nullptr;
     int wait_limit = 0;  // polls per pipeline wait of the tensor-core contraction (0: the default bound)
     bool timing = false, timed_once = false;
     size_t table_bytes = 0, workspace_bytes = 0;
@@ -148,6 +159,11 @@ struct ContractArgs {
     int n_tb, K, Dx, Dy, box_x0, box_y0, W, H, NIpad, NPpad, k0;
     int kbase;  // the tables hold mode slices kbase, kbase + 1, ... (0: all K; else a streamed chunk)
     int* status;  // device error word (a bounded wait that gave up)
+    Seg seg64, segx2, seg0;  // of the FP64 tiles, the double-float tiles, and these at k = 0 alone
+    int n_cols;              // interface columns in whole units
+    int n_ta, max_rhs;
+    double* seg_part;        // [segment][max_rhs][modes][NPpad][6] partial sums (the double-float tiles': two floats)
+    int* seg_cnt;            // [max_rhs][modes][n_ta] segments done, zero between launches
 };
 
 // One instance's share of a tensor-core contraction launch (fbc_contract_tc.cu).
@@ -207,6 +223,8 @@ cudaError_t launch_fft_tables(Plan& P, int precision, cudaStream_t st);
 cudaError_t launch_contract_fft(Plan& P, int n_rhs, cudaStream_t st);
 void fft_free(Plan& P);
 void fft_info(const Plan& P, int* mx, int* my, int* rows_i, int* rows_p, int* chunk_items);
+// chooses a plan's segments; returns the doubles of seg_part and sets *counters
+size_t contract_segments(Plan& P, size_t* counters);
 ContractArgs make_contract_args(const Plan& P);
 cudaError_t launch_contract_tc(const ContractArgs& A, const Plan& P, int n_rhs, cudaStream_t st, int n_modes = -1);
 // contraction of modes k0 .. k0 + n_modes - 1 in the plan's precision (k0 >= 1 for the FP32 and tensor forms)

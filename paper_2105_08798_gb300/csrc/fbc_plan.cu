@@ -194,7 +194,7 @@ void free_plan(fbc::Plan& P) {
     void* bufs[] = {P.d_xy_p,  P.d_off_i,    P.d_bbox_a, P.d_bbox_b, P.d_perm_i, P.d_perm_p,
                     P.d_used,  P.d_rep,      P.d_tw,       P.d_twL,    P.d_twl,    P.d_table,  P.d_table32, P.d_table_x2, P.d_table_x2_k0,
                     P.d_fh,    P.d_uh,       P.d_part,   P.d_stage_f, P.d_stage_u, P.d_status, P.d_bprep,
-                    P.d_relax, P.d_uh32, P.d_off_oz};
+                    P.d_relax, P.d_uh32, P.d_off_oz, P.d_seg_part, P.d_seg_cnt};
     for (void* b : bufs)
         if (b) cudaFree(b);
     for (auto& e : P.ev)
@@ -501,6 +501,12 @@ int fbc_plan_create(const fbc_geometry* geom, const fbc_material* mat, const fbc
     ALLOC(P.d_part, (size_t)opt.max_rhs * nlb * 3, "partials");
     ALLOC(P.d_relax, (size_t)opt.max_rhs * (fbc::kRelaxBlocks * 2 + nlb), "relaxation");
     ALLOC(P.d_status, 1, "status");
+    size_t n_cnt = 0;
+    const size_t n_seg = fbc::contract_segments(P, &n_cnt);
+    if (n_seg) {
+        ALLOC(P.d_seg_part, n_seg, "segment sums");
+        ALLOC(P.d_seg_cnt, n_cnt, "segment counters");
+    }
 #undef ALLOC
     P.workspace_bytes = acc - P.table_bytes;
     if (int s_ = ensure_derived(P, P.precision)) {
@@ -542,6 +548,7 @@ int fbc_plan_create(const fbc_geometry* geom, const fbc_material* mat, const fbc
     // padding columns of fh stay zero for ever: the forward transform never writes them
     if (e == cudaSuccess) e = cudaMemset(P.d_fh, 0, (size_t)opt.max_rhs * P.K * P.NIpad * 6 * sizeof(double));
     if (e == cudaSuccess) e = cudaMemset(P.d_status, 0, sizeof(int));
+    if (e == cudaSuccess && n_cnt) e = cudaMemset(P.d_seg_cnt, 0, sizeof(int) * n_cnt);
     if (e != cudaSuccess) {
         int s = cuda_fail(e, "plan upload");
         free_plan(P);
