@@ -250,7 +250,7 @@ int fbc_batch_create(fbc_plan* const* plans, int32_t n_plans, const double* cons
         const int NC = la[i].NC;
         for (int r = 0; r < R; r++) {
             for (int blk = 0; blk < P.NIpad / NC; blk++) b->fwd.push_back(make_int4(i, blk, r, 0));
-            b->proj.push_back(make_int4(i, 0, r, 0));
+            for (int c = 0; c < fbc::line_project_chunks(P.NIpad); c++) b->proj.push_back(make_int4(i, c, r, 0));
             for (int blk = 0; blk < P.NPpad / NC; blk++) b->inv.push_back(make_int4(i, blk, r, 0));
             const size_t n_el = (size_t)P.n_p * P.L * 3;
             const int nch = (int)std::max<size_t>(1, std::min<size_t>(64, (n_el + 4095) / 4096));

@@ -110,6 +110,7 @@ struct Plan {
     double* d_uh = nullptr;      // [max_rhs][K][NPpad][6]
     float* d_uh32 = nullptr;     // [max_rhs][K][NPpad][6]: the modes k >= 1 of the tensor-core forms (FP32 sums)
     double* d_part = nullptr;    // [max_rhs][n_line_blocks_p][3] zero-mean partial sums
+    double* d_fpart = nullptr;   // [max_rhs][n_line_blocks_i][3] net forces (k = 0 sums) of the forward transform's blocks
     double* d_relax = nullptr;   // [max_rhs][kRelaxBlocks][2] dot products, then [max_rhs][n_line_blocks_p] maxima
     double* d_stage_f = nullptr; // host-apply staging
     double* d_stage_u = nullptr;
@@ -192,6 +193,7 @@ struct LineArgs {
     const int* perm_p;
     const double2* tw;
     double* part;
+    double* fpart;
     int n_i, n_p, L, logL, K, NIpad, NPpad, NC;
 };
 
@@ -207,7 +209,9 @@ cudaError_t launch_contract(Plan& P, int n_rhs, cudaStream_t st);
 // gmax_part (optional): only record per (rhs, line block) the largest |value|, write nothing
 cudaError_t launch_inverse(Plan& P, double* u, int n_rhs, double alpha, double beta, bool zero_mean,
                            cudaStream_t st, const double* alpha_dev = nullptr, double alpha_dev_scale = 0.0,
-                           double* gmax_part = nullptr);
+                           double* gmax_part = nullptr, bool keep_g = false);
+// FP64 line transforms: launch_inverse(..., gmax_part, keep_g) leaves g = G f in d_uh; u -= alpha_dev g from there
+cudaError_t launch_kept_update(Plan& P, double* u, int n_rhs, const double* alpha_dev, bool zero_mean, cudaStream_t st);
 // residual-based relaxation (fbc_relax.cu)
 constexpr int kRelaxBlocks = 128;  // blocks per right-hand side of the dot-product pass
 cudaError_t launch_relax_dots(const double* f_new, const double* f_old, size_t n_per_rhs, int n_rhs, double* part,
@@ -254,6 +258,7 @@ cudaError_t launch_contract_oz(const ContractArgs& A, const Plan& P, int n_rhs, 
 inline bool is_tensor_precision(int p) { return p == FBC_PREC_TF32 || p == FBC_PREC_BF16X2 || p == FBC_PREC_BF16X3; }
 int batch_rhs_block();
 LineArgs make_line_args(const Plan& P, const double* f, double* u);
+int line_project_chunks(int NIpad);  // projection items per right-hand side
 // dynamic shared memory of one instance's batched line transforms (FP64 or FP32 form; a batch launches
 // with the largest over its instances)
 size_t line_args_smem(const LineArgs& A, bool fp32);
@@ -353,6 +358,19 @@ inline int line_cols(int L) {
     if (nc < 2) nc = 2;
     if (nc > 64) nc = 64;
     return nc;
+}
+
+// ... and fewer in the FP64 form where that leaves SMs idle: at least 304 CTAs (two an SM) over the plan's right-hand
+// sides, down to two columns.  (200 columns, L = 16: 16 us forward and 19 us back with four CTAs of 64 columns, 7 and
+// 9 us with 128 and 192 of two; 1000 and 1500 columns, L = 64: 35 and 35 us, now 12 and 18 us.)  The
+// FP32 form keeps line_cols.
+inline int line_nc64(int L, int NIpad, int max_rhs) {
+    int nc = line_cols(L);
+    while (nc > 2 && (long long)(NIpad / nc) * max_rhs < 304) nc /= 2;
+    return nc;
+}
+inline int line_nc(const Plan& P, int precision) {
+    return line_fp32(precision) ? line_cols(P.L) : line_nc64(P.L, P.NIpad, P.opt.max_rhs);
 }
 
 }  // namespace fbc

@@ -103,11 +103,19 @@ __device__ void fft_block(typename Cx<R>::T* buf, int nseq, int L, int logL, con
     }
 }
 
+// Sums of v[0..2] over a warp (a fixed shuffle tree).
+__device__ __forceinline__ void warp_sum3(double (&v)[3]) {
+#pragma unroll
+    for (int c = 0; c < 3; c++)
+        for (int o = 16; o > 0; o >>= 1) v[c] += __shfl_xor_sync(0xffffffffu, v[c], o);
+}
+
 // Forward transform of NC columns (block blk of right-hand side r).
 template <typename R>
 __device__ __forceinline__ void fwd_block(const double* __restrict__ f, const int* __restrict__ perm,
                                           const double2* __restrict__ tw, double* __restrict__ fh, int n_i, int L,
-                                          int logL, int K, int NIpad, int NC, int blk, int r, void* sraw) {
+                                          int logL, int K, int NIpad, int NC, int blk, int r,
+                                          double* __restrict__ fpart, void* sraw) {
     using T2 = typename Cx<R>::T;
     constexpr bool kF32 = sizeof(R) == 4;
     const int logNC = __ffs(NC) - 1;  // NC and L are powers of two: shifts, no integer division
@@ -163,6 +171,23 @@ __device__ __forceinline__ void fwd_block(const double* __restrict__ f, const in
     }
     __syncthreads();
     fft_block<R>(zs, NC + NC / 2, L, logL, tw, false);
+    // the block's sums of the k = 0 entries, for the projection
+    if (threadIdx.x < 32) {
+        double v[3] = {0.0, 0.0, 0.0};
+        for (int j = threadIdx.x; j < NC; j += 32) {
+            if constexpr (kF32) {
+                v[0] += s0[j][0], v[1] += s0[j][1], v[2] += s0[j][2];
+            } else {
+                const T2 Z = zs[(size_t)j * L], Wv = ws[(size_t)(j >> 1) * L];
+                v[0] += Z.x, v[1] += Z.y, v[2] += (j & 1) ? Wv.y : Wv.x;
+            }
+        }
+        warp_sum3(v);
+        if (threadIdx.x == 0) {
+            double* p = fpart + ((size_t)r * (NIpad / NC) + blk) * 3;
+            p[0] = v[0], p[1] = v[1], p[2] = v[2];
+        }
+    }
     // unpack and store six-vectors for k = 0..L/2
     for (int t = threadIdx.x; t < NC * K; t += blockDim.x) {
         const int k = t >> logNC, j = t & (NC - 1);
@@ -204,48 +229,48 @@ __device__ __forceinline__ void fwd_block(const double* __restrict__ f, const in
     }
 }
 
-// Neutral projection in the mode domain: mean_c = sum_b F_c(b, 0) / (n_i L);
-// F_c(b, 0) -= L mean_c for every real column.  One CTA of 256 threads per
-// right-hand side; fixed-order reduction (deterministic).
-__device__ __forceinline__ void project_rhs(double* __restrict__ fh, const int* __restrict__ perm, int n_i, int K,
-                                            int NIpad, int r) {
-    __shared__ double red[3][256];
-    double* row = fh + (size_t)r * K * NIpad * 6;  // k = 0
-    double s0 = 0.0, s1 = 0.0, s2 = 0.0;
-    for (int b = threadIdx.x; b < NIpad; b += blockDim.x) {
-        s0 += row[(size_t)b * 6 + 0];
-        s1 += row[(size_t)b * 6 + 1];
-        s2 -= row[(size_t)b * 6 + 5];
+// The first warp sums the n triples at p, in a fixed order, into the shared out[3].  (One warp, not the CTA: at two FP64
+// lanes a cycle and SM the adds of a wide tree cost more than the loads they wait for.)
+__device__ __forceinline__ void sum_parts(const double* __restrict__ p, int n, double* out) {
+    if (threadIdx.x < 32) {
+        double v[3] = {0.0, 0.0, 0.0};
+#pragma unroll 4
+        for (int t = threadIdx.x; t < n; t += 32) v[0] += p[3 * t], v[1] += p[3 * t + 1], v[2] += p[3 * t + 2];
+        warp_sum3(v);
+        if (threadIdx.x == 0) out[0] = v[0], out[1] = v[1], out[2] = v[2];
     }
-    red[0][threadIdx.x] = s0;
-    red[1][threadIdx.x] = s1;
-    red[2][threadIdx.x] = s2;
     __syncthreads();
-    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-        if ((int)threadIdx.x < w)
-            for (int c = 0; c < 3; c++) red[c][threadIdx.x] += red[c][threadIdx.x + w];
-        __syncthreads();
-    }
-    // L * mean = sum / n_i
-    const double m0 = red[0][0] / (double)n_i, m1 = red[1][0] / (double)n_i, m2 = red[2][0] / (double)n_i;
-    for (int b = threadIdx.x; b < NIpad; b += blockDim.x) {
-        if (perm[b] < 0) continue;
-        row[(size_t)b * 6 + 0] -= m0;
-        row[(size_t)b * 6 + 1] -= m1;
-        row[(size_t)b * 6 + 5] += m2;
-    }
+}
+
+// Neutral projection in the mode domain: mean_c = sum_b F_c(b, 0) / (n_i L);
+// F_c(b, 0) -= L mean_c for every real column.  Each CTA sums the forward transform's per-block sums (the same order
+// in every CTA) and takes a chunk of kProjectChunk columns.  (One CTA for all columns read them twice: 29 us at 4032
+// columns, 10 us now; 11 us at 200, 5 us now.)
+constexpr int kProjectChunk = 128;
+__device__ __forceinline__ void project_chunk(double* __restrict__ fh, const double* __restrict__ fpart, int n_part,
+                                              const int* __restrict__ perm, int n_i, int K, int NIpad, int r, int chunk) {
+    __shared__ double s[3];
+    sum_parts(fpart + (size_t)r * n_part * 3, n_part, s);
+    if (threadIdx.x < 3) s[threadIdx.x] /= (double)n_i;  // L * mean = sum / n_i
+    __syncthreads();
+    const int b = chunk * kProjectChunk + threadIdx.x;
+    if (b >= NIpad || perm[b] < 0) return;
+    double* o = fh + ((size_t)r * K * NIpad + b) * 6;  // k = 0
+    o[0] -= s[0];
+    o[1] -= s[1];
+    o[5] += s[2];
 }
 
 // Inverse transform + epilogue of NC pad columns (block blk of right-hand side
 // r); with want_part the block's per-component sums go to part[r][blk].
 template <typename R>
-__device__ __forceinline__ void inv_block(const double* __restrict__ uh, const int* __restrict__ perm,
+__device__ __forceinline__ void inv_block(const double* uh, const int* __restrict__ perm,
                                           const double2* __restrict__ tw, double* __restrict__ u,
                                           double* __restrict__ part, int n_p, int L, int logL, int K, int NPpad,
                                           int NC, double alpha_over_L, double beta, int want_part, int blk, int n_blk,
                                           int r, void* sraw, const double* __restrict__ alpha_dev = nullptr,
                                           double alpha_dev_scale = 0.0, double* __restrict__ gmax_part = nullptr,
-                                          const float* __restrict__ uh32 = nullptr) {
+                                          const float* __restrict__ uh32 = nullptr, double* keep = nullptr) {
     using T2 = typename Cx<R>::T;
     constexpr bool kF32 = sizeof(R) == 4;
     const int logNC = __ffs(NC) - 1;  // NC and L are powers of two: shifts, no integer division
@@ -394,6 +419,15 @@ __device__ __forceinline__ void inv_block(const double* __restrict__ uh, const i
             double o0 = alpha_over_L * z0, o1 = alpha_over_L * z1, o2 = alpha_over_L * v3;
             if (max_only) {
                 mx64 = fmax(mx64, fmax(fabs(o0), fmax(fabs(o1), fabs(o2))));
+                // over this CTA's own columns of uh (keep), which its transform has read: element 3 p + c at
+                // mode (3 p + c) / 6, entry (3 p + c) % 6
+                if (keep) {
+                    const int m = 3 * p;
+                    double* g = keep + ((size_t)r * K * NPpad + a0 + j) * 6;
+                    g[(size_t)(m / 6) * NPpad * 6 + m % 6] = o0;
+                    g[(size_t)((m + 1) / 6) * NPpad * 6 + (m + 1) % 6] = o1;
+                    g[(size_t)((m + 2) / 6) * NPpad * 6 + (m + 2) % 6] = o2;
+                }
                 continue;
             }
             double* dst = u + (((size_t)r * n_p + oa) * L + p) * 3;
@@ -447,7 +481,8 @@ __device__ __forceinline__ void inv_block(const double* __restrict__ uh, const i
 // transform, k = 0 in FP64.  twl[m] = exp(-2 pi i m / L), m < L, in FP32.
 __device__ __forceinline__ void fwd_block_s(const double* __restrict__ f, const int* __restrict__ perm,
                                             const float2* __restrict__ twl, const Fft1D& F, double* __restrict__ fh,
-                                            int n_i, int L, int K, int NIpad, int NC, int blk, int r, void* sraw) {
+                                            int n_i, int L, int K, int NIpad, int NC, int blk, int r,
+                                            double* __restrict__ fpart, void* sraw) {
     const int nseq = NC + NC / 2, logNC = __ffs(NC) - 1, Lh = L >> 1;
     float2* A = (float2*)sraw;
     float2* B = A + fft::padded(nseq * L);
@@ -490,6 +525,15 @@ __device__ __forceinline__ void fwd_block_s(const double* __restrict__ f, const 
         s0[j][c] = a;
     }
     const float2* Y = fft::fft_smem<false>(A, B, nseq, F, twl);
+    if (warp == 0) {  // the block's sums of the k = 0 entries, for the projection
+        double v[3] = {0.0, 0.0, 0.0};
+        for (int j = lane; j < NC; j += 32) v[0] += s0[j][0], v[1] += s0[j][1], v[2] += s0[j][2];
+        warp_sum3(v);
+        if (lane == 0) {
+            double* p = fpart + ((size_t)r * (NIpad / NC) + blk) * 3;
+            p[0] = v[0], p[1] = v[1], p[2] = v[2];
+        }
+    }
     for (int t = threadIdx.x; t < NC * K; t += blockDim.x) {
         const int k = t >> logNC, j = t & (NC - 1);
         double2* o = (double2*)(fh + (((size_t)r * K + k) * NIpad + b0 + j) * 6);
@@ -693,13 +737,8 @@ __device__ __forceinline__ void inv_block_s(const double* __restrict__ uh, const
 __device__ __forceinline__ void zero_mean_chunk(double* __restrict__ u, const double* __restrict__ part, int n_part,
                                                 int n_p, int L, int r, int c, int n_chunk) {
     __shared__ double mean[3];
-    if (threadIdx.x == 0) {
-        double s0 = 0.0, s1 = 0.0, s2 = 0.0;
-        const double* pp = part + (size_t)r * n_part * 3;
-        for (int t = 0; t < n_part; t++) s0 += pp[3 * t], s1 += pp[3 * t + 1], s2 += pp[3 * t + 2];
-        const double inv = 1.0 / ((double)n_p * (double)L);
-        mean[0] = s0 * inv, mean[1] = s1 * inv, mean[2] = s2 * inv;
-    }
+    sum_parts(part + (size_t)r * n_part * 3, n_part, mean);
+    if (threadIdx.x < 3) mean[threadIdx.x] *= 1.0 / ((double)n_p * (double)L);
     __syncthreads();
     const size_t n = (size_t)n_p * L * 3;
     double* ur = u + (size_t)r * n;
@@ -710,26 +749,63 @@ __device__ __forceinline__ void zero_mean_chunk(double* __restrict__ u, const do
 // ---- one launch per plan ------------------------------------------------------
 template <typename R>
 __global__ void k_forward(const double* __restrict__ f, const int* __restrict__ perm, const double2* __restrict__ tw,
-                          double* __restrict__ fh, int n_i, int L, int logL, int K, int NIpad, int NC) {
+                          double* __restrict__ fh, int n_i, int L, int logL, int K, int NIpad, int NC,
+                          double* __restrict__ fpart) {
     extern __shared__ double2 sbuf[];
-    fwd_block<R>(f, perm, tw, fh, n_i, L, logL, K, NIpad, NC, blockIdx.x, blockIdx.y, sbuf);
+    fwd_block<R>(f, perm, tw, fh, n_i, L, logL, K, NIpad, NC, blockIdx.x, blockIdx.y, fpart, sbuf);
 }
-__global__ void k_project(double* __restrict__ fh, const int* __restrict__ perm, int n_i, int K, int NIpad) {
-    project_rhs(fh, perm, n_i, K, NIpad, blockIdx.y);
+__global__ void __launch_bounds__(kProjectChunk) k_project(double* __restrict__ fh, const double* __restrict__ fpart,
+                                                           int n_part, const int* __restrict__ perm, int n_i, int K,
+                                                           int NIpad) {
+    project_chunk(fh, fpart, n_part, perm, n_i, K, NIpad, blockIdx.y, blockIdx.x);
 }
 template <typename R>
-__global__ void k_inverse(const double* __restrict__ uh, const int* __restrict__ perm, const double2* __restrict__ tw,
+__global__ void k_inverse(const double* uh, const int* __restrict__ perm, const double2* __restrict__ tw,
                           double* __restrict__ u, double* __restrict__ part, int n_p, int L, int logL, int K, int NPpad,
                           int NC, double alpha_over_L, double beta, int want_part, const double* __restrict__ alpha_dev,
-                          double alpha_dev_scale, double* __restrict__ gmax_part, const float* __restrict__ uh32) {
+                          double alpha_dev_scale, double* __restrict__ gmax_part, const float* __restrict__ uh32,
+                          double* keep) {
     extern __shared__ double2 sbuf[];
     inv_block<R>(uh, perm, tw, u, part, n_p, L, logL, K, NPpad, NC, alpha_over_L, beta, want_part, blockIdx.x,
-                 gridDim.x, blockIdx.y, sbuf, alpha_dev, alpha_dev_scale, gmax_part, uh32);
+                 gridDim.x, blockIdx.y, sbuf, alpha_dev, alpha_dev_scale, gmax_part, uh32, keep);
+}
+// u -= alpha g with the g = G f that the maximum's pass kept in uh; with want_part the block's sums as k_inverse's.
+// (A second inverse transform took 40 us at 1500 columns, L = 64, this 10 us: three passes over u, bound by latency.)
+__global__ void k_update(const double* __restrict__ g, const int* __restrict__ perm, double* __restrict__ u,
+                         double* __restrict__ part, int n_p, int L, int K, int NPpad, int NC,
+                         const double* __restrict__ alpha_dev, int want_part) {
+    const int r = blockIdx.y, a0 = blockIdx.x * NC;
+    const double na = -alpha_dev[r];
+    double s[3] = {0.0, 0.0, 0.0};
+    for (int t = threadIdx.x; t < NC * (L / 2); t += blockDim.x) {  // a column's mode slot: two repeats
+        const int k = t / NC, j = t - k * NC;
+        const int oa = perm[a0 + j];
+        if (oa < 0) continue;
+        const double* src = g + (((size_t)r * K + k) * NPpad + a0 + j) * 6;
+        double* dst = u + (((size_t)r * n_p + oa) * L + 2 * k) * 3;
+#pragma unroll
+        for (int c = 0; c < 6; c++) {
+            const double o = fma(na, src[c], dst[c]);
+            dst[c] = o;
+            s[c % 3] += o;
+        }
+    }
+    if (!want_part) return;
+    __shared__ double red[8][3];
+    warp_sum3(s);
+    if (threadIdx.x % 32 == 0) red[threadIdx.x / 32][0] = s[0], red[threadIdx.x / 32][1] = s[1], red[threadIdx.x / 32][2] = s[2];
+    __syncthreads();
+    if (threadIdx.x < 3) {
+        double v = 0.0;
+        for (int w = 0; w < (int)blockDim.x / 32; w++) v += red[w][threadIdx.x];
+        part[((size_t)r * gridDim.x + blockIdx.x) * 3 + threadIdx.x] = v;
+    }
 }
 __global__ void k_forward_s(const double* __restrict__ f, const int* __restrict__ perm, const float2* __restrict__ twl,
-                            Fft1D F, double* __restrict__ fh, int n_i, int L, int K, int NIpad, int NC) {
+                            Fft1D F, double* __restrict__ fh, int n_i, int L, int K, int NIpad, int NC,
+                            double* __restrict__ fpart) {
     extern __shared__ double2 sbuf[];
-    fwd_block_s(f, perm, twl, F, fh, n_i, L, K, NIpad, NC, blockIdx.x, blockIdx.y, sbuf);
+    fwd_block_s(f, perm, twl, F, fh, n_i, L, K, NIpad, NC, blockIdx.x, blockIdx.y, fpart, sbuf);
 }
 __global__ void k_inverse_s(const double* __restrict__ uh, const int* __restrict__ perm, const float2* __restrict__ twl,
                             Fft1D F, double* __restrict__ u, double* __restrict__ part, int n_p, int L, int K, int NPpad,
@@ -750,14 +826,15 @@ __global__ void k_batch_forward(const LineArgs* __restrict__ la, const int4* __r
     const int4 w = items[blockIdx.x];
     const LineArgs A = la[w.x];
     if (sizeof(R) == 4 && A.stockham)
-        fwd_block_s(A.f, A.perm_i, A.twl, A.F, A.fh, A.n_i, A.L, A.K, A.NIpad, A.NC, w.y, w.z, sbuf);
+        fwd_block_s(A.f, A.perm_i, A.twl, A.F, A.fh, A.n_i, A.L, A.K, A.NIpad, A.NC, w.y, w.z, A.fpart, sbuf);
     else
-        fwd_block<R>(A.f, A.perm_i, A.tw, A.fh, A.n_i, A.L, A.logL, A.K, A.NIpad, A.NC, w.y, w.z, sbuf);
+        fwd_block<R>(A.f, A.perm_i, A.tw, A.fh, A.n_i, A.L, A.logL, A.K, A.NIpad, A.NC, w.y, w.z, A.fpart, sbuf);
 }
-__global__ void k_batch_project(const LineArgs* __restrict__ la, const int4* __restrict__ items) {
-    const int4 w = items[blockIdx.x];
+__global__ void __launch_bounds__(kProjectChunk) k_batch_project(const LineArgs* __restrict__ la,
+                                                                 const int4* __restrict__ items) {
+    const int4 w = items[blockIdx.x];  // (instance, chunk, r, 0)
     const LineArgs A = la[w.x];
-    project_rhs(A.fh, A.perm_i, A.n_i, A.K, A.NIpad, w.z);
+    project_chunk(A.fh, A.fpart, A.NIpad / A.NC, A.perm_i, A.n_i, A.K, A.NIpad, w.z, w.y);
 }
 template <typename R>
 __global__ void k_batch_inverse(const LineArgs* __restrict__ la, const int4* __restrict__ items, double alpha,
@@ -791,7 +868,7 @@ bool line_stockham(int L, const void* a, const void* b) {
 }
 
 cudaError_t launch_forward(Plan& P, const double* f, int n_rhs, bool project, cudaStream_t st) {
-    const int NC = line_cols(P.L);
+    const int NC = line_nc(P, P.precision);
     const size_t smem = line_smem(P.L, NC);
     cudaError_t e;
     // opt in above the default dynamic limit (the kernel's static arrays count towards 48 KB)
@@ -799,25 +876,37 @@ cudaError_t launch_forward(Plan& P, const double* f, int n_rhs, bool project, cu
     if (line_fp32(P.precision) && line_stockham(P.L, f, P.d_fh)) {
         const size_t ss = line_smem_s(P.L, NC);
         if ((e = cudaFuncSetAttribute(k_forward_s, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ss))) return e;
-        k_forward_s<<<grid, 256, ss, st>>>(f, P.d_perm_i, P.d_twl, P.line_fft, P.d_fh, P.n_i, P.L, P.K, P.NIpad, NC);
+        k_forward_s<<<grid, 256, ss, st>>>(f, P.d_perm_i, P.d_twl, P.line_fft, P.d_fh, P.n_i, P.L, P.K, P.NIpad, NC,
+                                           P.d_fpart);
     } else if (line_fp32(P.precision)) {
         if ((e = cudaFuncSetAttribute(k_forward<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem))) return e;
-        k_forward<float><<<grid, 256, smem / 2, st>>>(f, P.d_perm_i, P.d_tw, P.d_fh, P.n_i, P.L, P.logL, P.K, P.NIpad, NC);
+        k_forward<float><<<grid, 256, smem / 2, st>>>(f, P.d_perm_i, P.d_tw, P.d_fh, P.n_i, P.L, P.logL, P.K, P.NIpad, NC,
+                                                     P.d_fpart);
     } else {
         if ((e = cudaFuncSetAttribute(k_forward<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem))) return e;
-        k_forward<double><<<grid, 256, smem, st>>>(f, P.d_perm_i, P.d_tw, P.d_fh, P.n_i, P.L, P.logL, P.K, P.NIpad, NC);
+        k_forward<double><<<grid, 256, smem, st>>>(f, P.d_perm_i, P.d_tw, P.d_fh, P.n_i, P.L, P.logL, P.K, P.NIpad, NC,
+                                                     P.d_fpart);
     }
     if ((e = cudaGetLastError())) return e;
     if (project) {
-        k_project<<<dim3(1, n_rhs), 256, 0, st>>>(P.d_fh, P.d_perm_i, P.n_i, P.K, P.NIpad);
+        k_project<<<dim3(line_project_chunks(P.NIpad), n_rhs), kProjectChunk, 0, st>>>(
+            P.d_fh, P.d_fpart, P.NIpad / NC, P.d_perm_i, P.n_i, P.K, P.NIpad);
         if ((e = cudaGetLastError())) return e;
     }
     return cudaSuccess;
 }
 
+static cudaError_t launch_zero_mean(Plan& P, double* u, int n_part, int n_rhs, cudaStream_t st) {
+    const size_t n = (size_t)P.n_p * P.L * 3;
+    const int blocks = (int)std::min<size_t>((n + 255) / 256, 2 * 152);  // each sums the partials again
+    k_zero_mean<<<dim3(blocks, n_rhs), 256, 0, st>>>(u, P.d_part, n_part, P.n_p, P.L);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_inverse(Plan& P, double* u, int n_rhs, double alpha, double beta, bool zero_mean,
-                           cudaStream_t st, const double* alpha_dev, double alpha_dev_scale, double* gmax_part) {
-    const int NC = line_cols(P.L);
+                           cudaStream_t st, const double* alpha_dev, double alpha_dev_scale, double* gmax_part,
+                           bool keep_g) {
+    const int NC = line_nc(P, P.precision);
     const size_t smem = line_smem(P.L, NC);
     cudaError_t e;
     const int nb = P.NPpad / NC;
@@ -834,29 +923,35 @@ cudaError_t launch_inverse(Plan& P, double* u, int n_rhs, double alpha, double b
         if ((e = cudaFuncSetAttribute(k_inverse<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem))) return e;
         k_inverse<float><<<grid, 256, smem / 2, st>>>(P.d_uh, P.d_perm_p, P.d_tw, u, P.d_part, P.n_p, P.L, P.logL, P.K,
                                                       P.NPpad, NC, alpha / (double)P.L, beta, zero_mean ? 1 : 0,
-                                                      alpha_dev, alpha_dev_scale, gmax_part, uh32);
+                                                      alpha_dev, alpha_dev_scale, gmax_part, uh32, nullptr);
     } else {
         if ((e = cudaFuncSetAttribute(k_inverse<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem))) return e;
         k_inverse<double><<<grid, 256, smem, st>>>(P.d_uh, P.d_perm_p, P.d_tw, u, P.d_part, P.n_p, P.L, P.logL, P.K,
                                                    P.NPpad, NC, alpha / (double)P.L, beta, zero_mean ? 1 : 0,
-                                                   alpha_dev, alpha_dev_scale, gmax_part, nullptr);
+                                                   alpha_dev, alpha_dev_scale, gmax_part, nullptr,
+                                                   keep_g ? P.d_uh : nullptr);
     }
     if ((e = cudaGetLastError())) return e;
-    if (zero_mean && !gmax_part) {
-        const size_t n = (size_t)P.n_p * P.L * 3;
-        int blocks = (int)std::min<size_t>((n + 255) / 256, 4 * 152);
-        k_zero_mean<<<dim3(blocks, n_rhs), 256, 0, st>>>(u, P.d_part, nb, P.n_p, P.L);
-        if ((e = cudaGetLastError())) return e;
-    }
-    return cudaSuccess;
+    return zero_mean && !gmax_part ? launch_zero_mean(P, u, nb, n_rhs, st) : cudaSuccess;
 }
+
+cudaError_t launch_kept_update(Plan& P, double* u, int n_rhs, const double* alpha_dev, bool zero_mean, cudaStream_t st) {
+    const int NC = line_nc(P, P.precision), nb = P.NPpad / NC;
+    const int threads = std::min(256, std::max(32, (NC * P.L / 2 + 31) / 32 * 32));
+    k_update<<<dim3(nb, n_rhs), threads, 0, st>>>(P.d_uh, P.d_perm_p, u, P.d_part, P.n_p, P.L, P.K, P.NPpad, NC, alpha_dev,
+                                              zero_mean ? 1 : 0);
+    if (cudaError_t e = cudaGetLastError()) return e;
+    return zero_mean ? launch_zero_mean(P, u, nb, n_rhs, st) : cudaSuccess;
+}
+
+int line_project_chunks(int NIpad) { return (NIpad + kProjectChunk - 1) / kProjectChunk; }
 
 LineArgs make_line_args(const Plan& P, const double* f, double* u) {
     LineArgs A;
     A.f = f, A.u = u, A.fh = P.d_fh, A.uh = P.d_uh, A.perm_i = P.d_perm_i, A.perm_p = P.d_perm_p, A.tw = P.d_tw;
-    A.part = P.d_part;
+    A.part = P.d_part, A.fpart = P.d_fpart;
     A.n_i = P.n_i, A.n_p = P.n_p, A.L = P.L, A.logL = P.logL, A.K = P.K, A.NIpad = P.NIpad, A.NPpad = P.NPpad;
-    A.NC = line_cols(P.L);
+    A.NC = line_nc(P, P.precision);
     A.F = P.line_fft;
     A.twl = P.d_twl;
     A.uh32 = is_tensor_precision(P.precision) ? P.d_uh32 : nullptr;
@@ -889,7 +984,7 @@ cudaError_t launch_batch_line(int stage, const LineArgs* d_args, const int4* d_i
             }
             break;
         case 1:
-            k_batch_project<<<n_items, 256, 0, st>>>(d_args, d_items);
+            k_batch_project<<<n_items, kProjectChunk, 0, st>>>(d_args, d_items);
             break;
         case 2:
             if (fp32) {

@@ -193,7 +193,7 @@ int dev_alloc(T** p, size_t count, size_t& acc, const char* what) {
 void free_plan(fbc::Plan& P) {
     void* bufs[] = {P.d_xy_p,  P.d_off_i,    P.d_bbox_a, P.d_bbox_b, P.d_perm_i, P.d_perm_p,
                     P.d_used,  P.d_rep,      P.d_tw,       P.d_twL,    P.d_twl,    P.d_table,  P.d_table32, P.d_table_x2, P.d_table_x2_k0,
-                    P.d_fh,    P.d_uh,       P.d_part,   P.d_stage_f, P.d_stage_u, P.d_status, P.d_bprep,
+                    P.d_fh,    P.d_uh,       P.d_part,   P.d_fpart, P.d_stage_f, P.d_stage_u, P.d_status, P.d_bprep,
                     P.d_relax, P.d_uh32, P.d_off_oz, P.d_seg_part, P.d_seg_cnt};
     for (void* b : bufs)
         if (b) cudaFree(b);
@@ -472,7 +472,7 @@ int fbc_plan_create(const fbc_geometry* geom, const fbc_material* mat, const fbc
     std::vector<int> off_i(P.NIpad);
     for (int s = 0; s < P.NIpad; s++) off_i[s] = tb.xy[s].x + P.W * tb.xy[s].y;
     const size_t cells = (size_t)P.K * P.Dy * P.Dx;
-    const int nlb = P.NPpad / fbc::line_cols(L);
+    const int nlb = P.NPpad / fbc::line_nc64(L, P.NIpad, opt.max_rhs);  // at least the FP32 form's
 #define ALLOC(ptr, n, what)                                  \
     do {                                                     \
         int s_ = dev_alloc(&(ptr), (n), acc, what);          \
@@ -499,6 +499,7 @@ int fbc_plan_create(const fbc_geometry* geom, const fbc_material* mat, const fbc
     ALLOC(P.d_fh, (size_t)opt.max_rhs * P.K * P.NIpad * 6, "fh");
     ALLOC(P.d_uh, (size_t)opt.max_rhs * P.K * P.NPpad * 6, "uh");
     ALLOC(P.d_part, (size_t)opt.max_rhs * nlb * 3, "partials");
+    ALLOC(P.d_fpart, (size_t)opt.max_rhs * (P.NIpad / fbc::line_nc64(L, P.NIpad, opt.max_rhs)) * 3, "net forces");
     ALLOC(P.d_relax, (size_t)opt.max_rhs * (fbc::kRelaxBlocks * 2 + nlb), "relaxation");
     ALLOC(P.d_status, 1, "status");
     size_t n_cnt = 0;
@@ -686,7 +687,7 @@ int fbc_apply_relaxed(fbc_plan* plan, const double* f_new, const double* f_old, 
         if (int s = apply_checks(P, f_old, u, n_rhs, flags)) return s;
     }
     cudaStream_t st = (cudaStream_t)stream;
-    const int nlb = P.NPpad / fbc::line_cols(P.L);
+    const int nlb = P.NPpad / fbc::line_nc(P, P.precision);
     double* dots = P.d_relax;
     double* gmax = P.d_relax + (size_t)P.opt.max_rhs * fbc::kRelaxBlocks * 2;
     cudaError_t e = cudaSuccess;
@@ -694,12 +695,16 @@ int fbc_apply_relaxed(fbc_plan* plan, const double* f_new, const double* f_old, 
     if (e != cudaSuccess) return cuda_fail(e, "relaxation dot products");
     if (int s = apply_modes(P, f_new, n_rhs, flags, st)) return s;
     // ||G f_new||_inf per right-hand side (a pass of the inverse transform that writes nothing)
-    if (du_max > 0.0) e = fbc::launch_inverse(P, u, n_rhs, 1.0, 0.0, false, st, nullptr, 0.0, gmax);
+    // with FP64 line transforms that pass keeps g in the mode buffer (FP32 ones scale by alpha before they round:
+    // theirs transforms again)
+    const bool keep = du_max > 0.0 && !fbc::line_fp32(P.precision);
+    if (du_max > 0.0) e = fbc::launch_inverse(P, u, n_rhs, 1.0, 0.0, false, st, nullptr, 0.0, gmax, keep);
     if (e == cudaSuccess) e = fbc::launch_relax_alpha(dots, f_old ? 1 : 0, gmax, nlb, n_rhs, du_max, alpha_io, st);
     if (e != cudaSuccess) return cuda_fail(e, "relaxation parameter");
     // u <- u - alpha_{k+1} G f_new, then the optional zero mean
-    e = fbc::launch_inverse(P, u, n_rhs, 0.0, 1.0, (flags & FBC_APPLY_ZERO_MEAN_U) != 0, st, alpha_io,
-                            -1.0 / (double)P.L, nullptr);
+    const bool zm = (flags & FBC_APPLY_ZERO_MEAN_U) != 0;
+    e = keep ? fbc::launch_kept_update(P, u, n_rhs, alpha_io, zm, st)
+             : fbc::launch_inverse(P, u, n_rhs, 0.0, 1.0, zm, st, alpha_io, -1.0 / (double)P.L, nullptr);
     if (e != cudaSuccess) return cuda_fail(e, "inverse transform");
     return FBC_OK;
 }

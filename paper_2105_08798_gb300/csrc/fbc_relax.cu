@@ -4,7 +4,7 @@
 //   alpha_{k+1} = 1 where that is negative,
 //   alpha_{k+1} = du_max / ||G f_{k+1}||_inf where ||alpha_{k+1} G f_{k+1}||_inf > du_max.
 // One value per right-hand side (each is its own relaxation sequence).  The dot
-// products are summed in a fixed order (per-block partials, then one thread),
+// products are summed in a fixed order (per-block partials, then one warp's tree),
 // so the result does not depend on scheduling.
 #include "fbc_internal.cuh"
 
@@ -37,28 +37,31 @@ __global__ void k_relax_dots(const double* __restrict__ f_new, const double* __r
     }
 }
 
-// One thread per right-hand side: Algorithm 2.  With equal f_new and f_old (a zero
-// denominator) alpha_k is kept.
+// One warp per right-hand side: Algorithm 2.  With equal f_new and f_old (a zero denominator) alpha_k is kept.
+// (One thread walking the partials took 19 us at 128 + 48 of them.)
 __global__ void k_relax_alpha(const double* __restrict__ dot_part, int has_old, const double* __restrict__ gmax_part,
                               int n_gblk, int n_rhs, double du_max, double* __restrict__ alpha_io) {
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= n_rhs) return;
-    double alpha = alpha_io[r];
-    if (has_old) {
-        double d = 0.0, q = 0.0;
-        for (int b = 0; b < kRelaxBlocks; b++) {
-            d += dot_part[((size_t)r * kRelaxBlocks + b) * 2];
-            q += dot_part[((size_t)r * kRelaxBlocks + b) * 2 + 1];
+    const int r = blockIdx.x, lane = threadIdx.x;
+    double alpha = alpha_io[r], d = 0.0, q = 0.0, gmax = 0.0;
+    if (has_old)
+#pragma unroll
+        for (int b = 0; b < kRelaxBlocks / 32; b++) {
+            const double2 v = ((const double2*)dot_part)[(size_t)r * kRelaxBlocks + lane + 32 * b];
+            d += v.x, q += v.y;
         }
+    if (du_max > 0.0)
+        for (int b = lane; b < n_gblk; b += 32) gmax = fmax(gmax, gmax_part[(size_t)r * n_gblk + b]);
+    for (int o = 16; o > 0; o >>= 1) {
+        d += __shfl_xor_sync(0xffffffffu, d, o);
+        q += __shfl_xor_sync(0xffffffffu, q, o);
+        gmax = fmax(gmax, __shfl_xor_sync(0xffffffffu, gmax, o));
+    }
+    if (has_old) {
         if (q > 0.0) alpha = -alpha * d / q;
         if (alpha < 0.0) alpha = 1.0;
     }
-    if (du_max > 0.0) {
-        double gmax = 0.0;
-        for (int b = 0; b < n_gblk; b++) gmax = fmax(gmax, gmax_part[(size_t)r * n_gblk + b]);
-        if (gmax > 0.0 && alpha * gmax > du_max) alpha = du_max / gmax;
-    }
-    alpha_io[r] = alpha;
+    if (du_max > 0.0 && gmax > 0.0 && alpha * gmax > du_max) alpha = du_max / gmax;
+    if (lane == 0) alpha_io[r] = alpha;
 }
 
 }  // namespace
@@ -71,7 +74,7 @@ cudaError_t launch_relax_dots(const double* f_new, const double* f_old, size_t n
 
 cudaError_t launch_relax_alpha(const double* dot_part, int has_old, const double* gmax_part, int n_gblk, int n_rhs,
                                double du_max, double* alpha_io, cudaStream_t st) {
-    k_relax_alpha<<<(n_rhs + 63) / 64, 64, 0, st>>>(dot_part, has_old, gmax_part, n_gblk, n_rhs, du_max, alpha_io);
+    k_relax_alpha<<<n_rhs, 32, 0, st>>>(dot_part, has_old, gmax_part, n_gblk, n_rhs, du_max, alpha_io);
     return cudaGetLastError();
 }
 

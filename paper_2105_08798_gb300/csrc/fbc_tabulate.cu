@@ -267,25 +267,27 @@ __device__ void green_cubic(const CubicDir& D, double rx, double ry, double rz, 
 // H-matrix's FP32 table keep the node-by-node form's bits.
 enum { kGreenIso = 0, kGreenNodes = 1, kGreenPoly = 2 };
 
-// G(0, 0, m l3) + G(0, 0, -m l3) for the images m = 1 .. n + N: the same for every difference and offset.
+// G(0, 0, m l3) + G(0, 0, -m l3) for the images m = 1 .. n + N (one block each, a thread per sign): the same for every
+// difference and offset.
 template <int KIND>
 __global__ void k_reference(double* __restrict__ ref) {
-    const int m = threadIdx.x + 1;
-    if (m > c_tp.rich_n + c_tp.rich_N) return;
-    const double zm = (double)m * ((double)c_tp.L * c_tp.c);
-    double g[6], h[6];
+    const int m = blockIdx.x + 1;
+    __shared__ double h[6];
+    const double zm = (threadIdx.x ? -1.0 : 1.0) * ((double)m * ((double)c_tp.L * c_tp.c));
+    double g[6];
     if (KIND == kGreenIso) {
         green_isotropic(0.0, 0.0, zm, g);
-        green_isotropic(0.0, 0.0, -zm, h);
     } else if (KIND == kGreenNodes) {
         green_nodes(0.0, 0.0, zm, g);
-        green_nodes(0.0, 0.0, -zm, h);
     } else {
         const CubicDir D = cubic_dir(0.0, 0.0);
         green_cubic(D, 0.0, 0.0, zm, g);
-        green_cubic(D, 0.0, 0.0, -zm, h);
     }
-    for (int t = 0; t < 6; t++) ref[(m - 1) * 6 + t] = g[t] + h[t];
+    if (threadIdx.x == 1)
+        for (int t = 0; t < 6; t++) h[t] = g[t];
+    __syncthreads();
+    if (threadIdx.x == 0)
+        for (int t = 0; t < 6; t++) ref[(m - 1) * 6 + t] = g[t] + h[t];
 }
 
 // Stage 1: one thread per (listed difference, s in [0, L/2]).  Of a pair of used differences d and -d only one
@@ -466,7 +468,7 @@ static cudaError_t upload_tabulate_constants(Plan& P, int kind, cudaStream_t st)
 // Stage 1 of nd listed differences from d0 on (ref: the images' reference sums).
 template <int KIND>
 static cudaError_t launch_periodic(Plan& P, int d0, int nd, double* ref, double* gs, cudaStream_t st) {
-    if (d0 == 0) k_reference<KIND><<<1, 64, 0, st>>>(ref);
+    if (d0 == 0) k_reference<KIND><<<P.tp.rich_n + P.tp.rich_N, 2, 0, st>>>(ref);
     const long long threads = (long long)nd * (P.L / 2 + 1);
     k_periodic<KIND><<<(unsigned)((threads + 127) / 128), 128, 0, st>>>(P.d_rep + d0, nd, ref, gs);
     return cudaGetLastError();
