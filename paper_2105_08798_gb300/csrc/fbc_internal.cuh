@@ -285,9 +285,12 @@ constexpr double kQrCut = 16.0;
 
 // Network inputs of difference d (d != 0) at mode k >= 1:
 // (ln(q r) / 4, d_x / r, d_y / r, ln(r) / 5) with q = 2 pi k / (L c); returns q r.
+__host__ __device__ inline double surrogate_qr(int dx, int dy, int k, int L, double c) {
+    return 2.0 * 3.14159265358979323846 * k / (L * c) * sqrt((double)dx * dx + (double)dy * dy);
+}
 __host__ __device__ inline double surrogate_features(int dx, int dy, int k, int L, double c, float* x) {
     const double r = sqrt((double)dx * dx + (double)dy * dy);
-    const double qr = 2.0 * 3.14159265358979323846 * k / (L * c) * r;
+    const double qr = surrogate_qr(dx, dy, k, L, c);
     x[0] = (float)(log(qr) * 0.25);
     x[1] = (float)(dx / r);
     x[2] = (float)(dy / r);
