@@ -128,10 +128,9 @@ void build_tc_items(fbc_batch* b) {
     b->smem_tc = 0;
     for (int i = 0; i < b->n; i++) {
         const fbc::Plan& P = b->plans[i]->p;
-        const int rpc = inst_rpc(b, i), R = b->n_rhs[i], HW = P.H * P.W;
-        const int nbuf = fbc::contract_tc_nbuf_smem(b->precision, HW, 2) <= 227 * 1024 ? 2 : 1;
-        b->smem_tc = std::max(b->smem_tc, fbc::contract_tc_nbuf_smem(b->precision, HW, nbuf));
-        b->tc_jobs[i] = fbc::contract_tc_job(P, R, rpc, nbuf);
+        const int rpc = inst_rpc(b, i), R = b->n_rhs[i];
+        b->smem_tc = std::max(b->smem_tc, fbc::contract_tc_smem(b->precision, P));
+        b->tc_jobs[i] = fbc::contract_tc_job(P, R, rpc);
         for (int k = 1; k < P.K; k++)
             for (int tA = 0; tA < P.n_ta; tA++)
                 for (int g = 0; g < (R + rpc - 1) / rpc; g++) {
@@ -220,7 +219,7 @@ int fbc_batch_create(fbc_plan* const* plans, int32_t n_plans, const double* cons
             return bfail(FBC_ERR_UNSUPPORTED, "batches run the dense per-mode contraction, not the in-plane FFT form");
         if (prec == FBC_PREC_BF16X6)
             return bfail(FBC_ERR_UNSUPPORTED, "BF16X6 plans run on their own, not in a batch");
-        if (fbc::is_tensor_precision(prec) && fbc::contract_tc_smem(prec, P.W * P.H) > 227 * 1024)
+        if (fbc::is_tensor_precision(prec) && fbc::contract_tc_smem(prec, P) > 227 * 1024)
             return bfail(FBC_ERR_UNSUPPORTED, "tensor-core contraction: an instance's sub-box exceeds shared memory");
         if (n_rhs[i] < 1 || n_rhs[i] > P.opt.max_rhs) return bfail(FBC_ERR_INVALID_ARG, "n_rhs outside [1, max_rhs]");
         if (!f[i] || !u[i]) return bfail(FBC_ERR_INVALID_ARG, "f or u of an instance is NULL");

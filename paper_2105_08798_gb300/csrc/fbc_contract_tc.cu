@@ -10,18 +10,29 @@
 // table reals.  A CTA owns 128 pad columns (GEMM rows) at one k and up to 64
 // right-hand sides (N = 2 R columns) and walks the interface columns in
 // stages of 16, through a ring of shared-memory stages:
-//   * eight builder warps gather the six 128 x 16 blocks A_e(a, b) =
-//     T_e(x_a - x_b) from the staged table sub-box, split them into bf16
-//     pieces (h, m, l) or round them to tf32, and store them in the K-major
-//     no-swizzle canonical layout (8-row x 16-byte core matrices);
+//   * a warp stages the table sub-box of each interface tile, a bulk copy per
+//     row, a tile ahead where two fit;
+//   * twelve builder warps gather the six 128 x 16 blocks A_e(a, b) =
+//     T_e(x_a - x_b) from it, a row and two entries a thread, and split them
+//     into bf16 pieces (h, m, l) or round them to tf32.  A thread's 32 words are
+//     one tcgen05.st into the A operand in tensor memory (TF32, BF16X2: up to
+//     four operands of 96 columns above the accumulators, so a stage is built
+//     while others are multiplied), or go to shared memory in the K-major
+//     no-swizzle canonical layout (BF16X3);
 //   * the force operand X_0, X_1, X_2 was split once per apply by k_prep_b
 //     into the same layout, one contiguous chunk per (k, rhs group, stage);
 //     one thread streams each chunk in with a bulk copy (cp.async.bulk);
-//   * one warp (an elected lane) issues the 9 block products per split-product pair with
-//     tcgen05.mma (M = 128, N = 2 R, K = 16 bf16 / 8 tf32) into three TMEM
-//     accumulators (one per output component); the -B13, -B23 entries use
-//     the instruction's negate-A bit; a commit to the stage's "empty" barrier
-//     hands the stage back to the builders and the copy thread.
+//   * one warp (an elected lane) issues the 9 block products per split-product
+//     pair as seven tcgen05.mma (M = 128, N = 2 R or 4 R, K = 16 bf16 / 8 tf32)
+//     into three TMEM accumulators (one per output component); commits hand the
+//     stage back to the builders and the copy thread.
+// What bounds it: at 16 right-hand sides the gathers (a stage's 192 shared
+// loads take about 900 cycles with their bank conflicts) and the issue of the
+// products (21 of some 36 cycles) about equally; from N = 128 the tensor pipe.
+// 4502 + 3001 columns, L = 512, 16 right-hand sides, BF16X2: 11.9 ms with eight
+// builder warps (12 tcgen05.st a stage each), one A operand and sub-boxes
+// copied by the builders, 8.3 ms now; 64 right-hand sides, L = 64: 4.3 and
+// 4.2 ms.
 // Split products: TF32 (1), BF16X2 (hh + hm + mh), BF16X3 (+ hl + lh + mm),
 // pieces h = bf16(x), m = bf16(x - h), l = bf16(x - h - m), all rounded to
 // nearest.  The logarithmic k = 0 mode is left to the double-float kernel.
@@ -38,6 +49,7 @@
 
 #include <algorithm>
 
+#include "fbc_f32x2.cuh"
 #include "fbc_internal.cuh"
 #include "fbc_tc.cuh"
 
@@ -49,13 +61,16 @@ constexpr int kRows = kTileA;    // GEMM rows (pad columns) per CTA
 constexpr int kRhsPerCta = 64;
 constexpr int kNPB = 128;        // force-operand rows per CTA (64 rhs x (x, y'))
 constexpr int kKC = 16;          // interface columns per stage
-constexpr int kBuilderWarps = 8;
+constexpr int kBuilderWarps = 12;
 constexpr int kBuilders = kBuilderWarps * 32;
-constexpr int kMmaWarp = 8, kCopyWarp = 9;
-constexpr int kThreads = 10 * 32;
+constexpr int kMmaWarp = kBuilderWarps, kCopyWarp = kBuilderWarps + 1, kTabWarp = kBuilderWarps + 2;
+constexpr int kThreads = (kBuilderWarps + 3) * 32;
 constexpr int kStagesPerTile = kTileB / kKC;
 constexpr int kDrainTiles = 16;  // interface tiles per tensor-memory accumulation group
-constexpr uint32_t kAcol = 384;  // first TMEM column of the A operand (after 3 x 128 accumulator columns)
+constexpr int kMaxABuf = 4;      // A operands in tensor memory: 96 columns each from the top, 3 NP columns of accumulators below
+constexpr int kACols = 96;
+__device__ __forceinline__ uint32_t a_col(int j) { return (uint32_t)(kTmemCols - kACols * (j + 1)); }
+__device__ __forceinline__ int a_bufs(int NP) { return min(kMaxABuf, (kTmemCols - 3 * NP) / kACols); }
 
 using tc::idesc;
 using tc::mbar_expect_tx;
@@ -89,14 +104,20 @@ struct TcLayout {
     static constexpr size_t ABLK = (size_t)kRows * kKC * C::ES;
     static constexpr size_t A_STAGE = C::ATM ? 0 : 6 * C::NS * ABLK;  // shared-memory A stage
     static constexpr uint32_t ACOLS = (uint32_t)(kKC * C::ES / 4);         // TMEM columns of one A block
+    static_assert(!C::ATM || 6 * C::NS * ACOLS == kACols, "six entries of NS pieces");
     static constexpr size_t B_STAGE = 3 * C::NS * (size_t)kNPB * kKC * C::ES;  // allocated for 128 rows
 };
 
-// Products issued per stage, fully unrolled: for output component co and
-// input component ci the table entry kEnt[co][ci] of M (the (0, 2) and (1, 2)
-// entries negated through the instruction descriptor), and for split product
-// pr the pieces (kPa[pr], kPb[pr]) of the A and B operands, by decreasing
-// magnitude: hh, hm, mh, hl, lh, mm.
+// Products of a stage, in the order in which each accumulator takes them: table entry, force block (X_2 stored
+// negated, first in a chunk: [-X_2, X_1, X_0]), accumulator.  M is symmetric up to the sign of its (0, 2) and (1, 2)
+// entries, so A12 multiplies X_1 into U_0 and X_0 into U_1, and B23 multiplies -X_2 into U_1 and X_1 into U_2: with the
+// blocks and the accumulators in this order each pair is one instruction of 2 NP columns (seven per split product, not
+// nine; at NP = 32 an instruction costs its issue, some 33 cycles, whatever its width).  U_2's A33 term negates A.
+struct Prod {
+    int ent, blk, acc, wide, neg;
+};
+// Split product pr takes the pieces (kPa[pr], kPb[pr]) of the A and B operands, by decreasing magnitude: hh, hm, mh,
+// hl, lh, mm.
 
 // Split x into NS pieces of the operand type; returned as raw bits (bf16 in
 // the low 16 bits, or the tf32 bit pattern).  FP32 arithmetic throughout: each
@@ -144,9 +165,16 @@ __host__ __device__ __forceinline__ size_t bchunk_index(int k, int g, int tB, in
     return (((size_t)k * G + g) * n_tb + tB) * kStagesPerTile + st;
 }
 
+// Rows of a group's blocks: two per right-hand side, in whole steps of 16 (an instruction's N).
+__host__ __device__ __forceinline__ int group_rows(int rpc, int n_rhs, int g) {
+    const int RG = rpc < n_rhs - g * rpc ? rpc : n_rhs - g * rpc;
+    return RG > 0 ? (2 * RG + 15) / 16 * 16 : 0;
+}
+
 // One thread per 16-byte core row (block c, row n, core column kc) of a chunk:
 // X_c(b, n = 2 r + h) = fh[g rpc + r][k][b][3 h + c], zero for r beyond the group
-// (rpc right-hand sides per group, G groups, npb >= 2 rpc rows per chunk).
+// (rpc right-hand sides per group, G groups, chunks of npb >= 2 rpc rows per block).
+// A chunk holds, piece by piece, the blocks -X_2, X_1, X_0 of the group's rows.
 template <int PREC>
 __global__ void k_prep_b(const double* __restrict__ fh, int K, int NIpad, int n_tb, int G, int npb, int rpc,
                          int n_rhs, int k0, int n_modes, unsigned char* __restrict__ out) {
@@ -166,7 +194,8 @@ __global__ void k_prep_b(const double* __restrict__ fh, int K, int NIpad, int n_
         q /= n_tb;
         const int g = (int)(q % G);
         const int k = k0 + (int)(q / G);
-        const int RG = min(rpc, n_rhs - g * rpc);
+        const int RG = min(rpc, n_rhs - g * rpc), NP = group_rows(rpc, n_rhs, g);
+        if (n >= NP) continue;
         const int r = n >> 1, h = n & 1;
         const int b0 = tB * kTileB + st * kKC + kc * KPC;
         uint32_t w[C::NS][KPC];
@@ -175,7 +204,7 @@ __global__ void k_prep_b(const double* __restrict__ fh, int K, int NIpad, int n_
             float v = 0.f;
             if (r < RG) v = (float)fh[(((size_t)(g * rpc + r) * K + k) * NIpad + b0 + i) * 6 + h * 3 + c];
             uint32_t sp[C::NS];
-            split<PREC>(v, sp);
+            split<PREC>(c == 2 ? -v : v, sp);
 #pragma unroll
             for (int p = 0; p < C::NS; p++) w[p][i] = sp[p];
         }
@@ -183,24 +212,62 @@ __global__ void k_prep_b(const double* __restrict__ fh, int K, int NIpad, int n_
         const uint32_t off = (uint32_t)(n / 8) * Lt::SBO + kc * 128 + (n % 8) * 16;
 #pragma unroll
         for (int p = 0; p < C::NS; p++)
-            *(uint4*)(base + (size_t)(c * C::NS + p) * npb * kKC * C::ES + off) = pack16<C::ES, KPC>(w[p]);
+            *(uint4*)(base + (size_t)(p * 3 + 2 - c) * NP * kKC * C::ES + off) = pack16<C::ES, KPC>(w[p]);
     }
 }
 
 // Shared-memory barriers and flags of the contraction CTA.
 template <int S>
 struct TcSync {
-    uint64_t full[S], bfull[S], empty[S], done, afull, aempty;
+    uint64_t full[S], bfull[S], empty[S], done, afull[kMaxABuf], aempty[kMaxABuf], tfull[2], tempty[2];
     uint32_t tbase;
     volatile int abort;
 };
 
+// The products of one stage.  FIRST: they overwrite the accumulators; accumulator 1's first split product then cannot
+// share an instruction with accumulator 0's.
+template <int PREC, bool FIRST>
+__device__ __forceinline__ void issue_stage(uint32_t tmem, uint32_t ta, uint64_t dAs, uint64_t dBs, uint32_t bblk16, int NP,
+                                            uint32_t id, uint32_t idw, uint32_t idn, uint32_t el) {
+    using C = TcCfg<PREC>;
+    using Lt = TcLayout<PREC>;
+#pragma unroll
+    for (int q = 0; q < 7; q++)
+#pragma unroll
+        for (int pr = 0; pr < C::NPROD; pr++)
+#pragma unroll
+            for (int ks = 0; ks < kKC / C::KMMA; ks++) {
+                constexpr int kPa[6] = {0, 0, 1, 0, 2, 1}, kPb[6] = {0, 1, 0, 2, 0, 1};
+                constexpr Prod P[7] = {{0, 2, 0, 0, 0}, {1, 1, 0, 1, 0}, {2, 1, 1, 0, 0}, {4, 2, 2, 0, 0},
+                                       {4, 0, 0, 0, 0}, {5, 0, 1, 1, 0}, {3, 0, 2, 0, 1}};
+                const int ablk = P[q].ent * C::NS + kPa[pr];
+                auto mma = [&](int blk, int acc, uint32_t idd, uint32_t en) {
+                    const uint64_t db = dBs + (uint64_t)((kPb[pr] * 3 + blk) * bblk16 + 16 * ks);
+                    const uint32_t dt = tmem + (uint32_t)(acc * NP);
+                    if (C::ATM)  // A from tensor memory: block ablk, K step ks (8 columns per MMA)
+                        tc::mma_ts<C::FMT == 2>(dt, ta + (uint32_t)ablk * Lt::ACOLS + 8u * ks, db, idd, en, el);
+                    else
+                        tc::mma_ss(dt, dAs + (uint64_t)((ablk * Lt::ABLK + 256 * ks) >> 4), db, idd, en, el);
+                };
+                const bool start = FIRST && pr == 0 && ks == 0;
+                if (P[q].wide && !(start && q == 1)) {
+                    mma(P[q].blk, P[q].acc, idw, 1u);
+                } else if (P[q].wide) {
+                    mma(P[q].blk, P[q].acc, id, 1u);
+                    mma(P[q].blk + 1, P[q].acc + 1, id, 0u);
+                } else {
+                    mma(P[q].blk, P[q].acc, P[q].neg ? idn : id, start && (q == 0 || q == 3) ? 0u : 1u);
+                }
+            }
+}
+
 // One work item (job J, mode k = wk.y, pad tile tA = wk.z, rhs group g = wk.w) on the whole CTA.  it_base:
 // stages this CTA has run before the item (every role counts alike, so stage s = it % S and the barrier
-// phases run on across items); n_done: items run before it (the parity of `done`).
+// phases run on across items); n_done: items run before it (the parity of `done`); aph: the parities of this role's
+// next wait on each A buffer (bits 0..3) and table buffer (bits 8, 9), which run on likewise.
 template <int PREC>
 __device__ __forceinline__ void tc_item(const TcJob& J, const int4 wk, const uint32_t it_base, const uint32_t n_done,
-                                        TcSync<TcCfg<PREC>::S>& sy, unsigned char* smem, const int wl) {
+                                        TcSync<TcCfg<PREC>::S>& sy, unsigned char* smem, const int wl, uint32_t& aph) {
     using C = TcCfg<PREC>;
     using Lt = TcLayout<PREC>;
     constexpr int S = C::S;
@@ -208,8 +275,10 @@ __device__ __forceinline__ void tc_item(const TcJob& J, const int4 wk, const uin
     uint64_t* bfull = sy.bfull;
     uint64_t* empty = sy.empty;
     uint64_t& done = sy.done;
-    uint64_t& afull = sy.afull;
-    uint64_t& aempty = sy.aempty;
+    uint64_t* afull = sy.afull;
+    uint64_t* aempty = sy.aempty;
+    uint64_t* tfull = sy.tfull;
+    uint64_t* tempty = sy.tempty;
     volatile int& s_abort = sy.abort;
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
     const ContractArgs& A = J.A;
@@ -219,15 +288,16 @@ __device__ __forceinline__ void tc_item(const TcJob& J, const int4 wk, const uin
         unsigned char* sA = smem;                                   // [S][6][NS][128][16]
         unsigned char* sB = sA + S * Lt::A_STAGE;                   // [S][3][NS][npb][16]
         int* s_off = (int*)(sB + S * Lt::B_STAGE);                  // [nbuf][TB]
-        float* s_tab = (float*)(s_off + J.nbuf * kTileB);           // [nbuf][HW][6]
+        unsigned char* s_tab = (unsigned char*)(s_off + J.nbuf * kTileB);  // [nbuf][tab_bytes]
         const int nbuf = J.nbuf, gs = J.gs;
         const int k = wk.y, tA = wk.z, g = wk.w;
         const int r0 = g * J.rpc;
         const int RG = min(J.rpc, J.n_rhs - r0);
-        const int NP = ((2 * RG + 15) / 16) * 16;
+        const int NP = group_rows(J.rpc, J.n_rhs, g);
+        const int n_abuf = a_bufs(NP);
         const int n_it = A.n_tb * kStagesPerTile;
         const uint32_t chunk_bytes = (uint32_t)(3 * C::NS * J.npb * kKC * C::ES);
-        const size_t bblk = (size_t)J.npb * kKC * C::ES;              // one (block, piece) of a chunk
+        const uint32_t bblk = (uint32_t)(NP * kKC * C::ES);          // one (block, piece) of a chunk
 
         if (warp == kCopyWarp) {
             // ---- force operand: one bulk copy per stage ----
@@ -242,9 +312,9 @@ __device__ __forceinline__ void tc_item(const TcJob& J, const int4 wk, const uin
                         break;
                     }
                     const int tB = il / kStagesPerTile, st = il % kStagesPerTile;
-                    mbar_expect_tx(&bfull[s], chunk_bytes);
+                    mbar_expect_tx(&bfull[s], 3 * C::NS * bblk);
                     bulk_g2s(sB + s * Lt::B_STAGE, J.bprep + bchunk_index(k, g, tB, st, J.G, A.n_tb) * chunk_bytes,
-                             chunk_bytes, &bfull[s]);
+                             3 * C::NS * bblk, &bfull[s]);
                 }
                 // copies still in flight land before the CTA may go on or exit: the full bound, whatever the
                 // stop flag says
@@ -253,22 +323,67 @@ __device__ __forceinline__ void tc_item(const TcJob& J, const int4 wk, const uin
                     tc::mbar_wait(&bfull[it % S], (it / S) & 1u);
                 }
             }
+        } else if (warp == kTabWarp) {
+            // ---- table sub-boxes: a bulk copy per row ----
+            // A row's 24 W bytes start on an 8-byte boundary, a copy on a 16-byte one: it takes the bytes around them
+            // too.  The shared pitch leaves room for them and equals the table's modulo 16, so that the rows stay a
+            // pitch apart behind the same offset of 0 or 8.  Cells outside the box are left as they are: nobody reads
+            // them (every difference of a pair of tiles lies in it).
+            if (J.bulk) {
+                const int4 bA = A.bbox_a[tA];
+                const unsigned char* tk = (const unsigned char*)(A.tab32 + (size_t)(k - A.kbase) * A.Dy * A.Dx * 6);
+                int b = 0;
+                uint32_t used = 0;
+                for (int tB = 0; tB < A.n_tb; tB++) {
+                    const int4 bB = A.bbox_b[tB];
+                    const int gx0 = bA.x - bB.y - A.box_x0, gy0 = bA.z - bB.w - A.box_y0;
+                    const int rows = min(A.H, A.Dy - gy0), bytes = 24 * min(A.W, A.Dx - gx0);
+                    const unsigned char* src = tk + ((size_t)gy0 * A.Dx + gx0) * 24;
+                    uint32_t sum = 0;
+                    for (int iy = lane; iy < rows; iy += 32) {
+                        const size_t p = (size_t)src + (size_t)iy * A.Dx * 24;
+                        sum += (uint32_t)(((p + bytes + 15) & ~(size_t)15) - (p & ~(size_t)15));
+                    }
+                    sum = __reduce_add_sync(0xffffffffu, sum) + kTileB * 4;
+                    if (!__all_sync(0xffffffffu, wait_or_abort(&tempty[b], aph >> (8 + b) & 1u, &s_abort, wl))) {
+                        s_abort = 1;
+                        break;
+                    }
+                    aph ^= 0x100u << b, used |= 1u << b;
+                    if (lane == 0) {
+                        mbar_expect_tx(&tfull[b], sum);
+                        bulk_g2s(s_off + b * kTileB, J.off + tB * kTileB, kTileB * 4, &tfull[b]);
+                    }
+                    __syncwarp();
+                    unsigned char* dst = s_tab + (size_t)b * J.tab_bytes + ((size_t)src & 15);
+                    for (int iy = lane; iy < rows; iy += 32) {
+                        const size_t p = (size_t)src + (size_t)iy * A.Dx * 24;
+                        bulk_g2s(dst + (size_t)iy * J.pitch - (p & 15), (const void*)(p & ~(size_t)15),
+                                 (uint32_t)(((p + bytes + 15) & ~(size_t)15) - (p & ~(size_t)15)), &tfull[b]);
+                    }
+                    if (++b == J.nbuf) b = 0;
+                }
+                // copies still in flight land before the CTA may go on or exit: the full bound
+                for (b = 0; b < 2; b++)
+                    if (used >> b & 1u) tc::mbar_wait(&tfull[b], aph >> (8 + b) & 1u);
+            }
         } else if (warp == kMmaWarp) {
             // ---- tensor-core issue, from the whole warp (one elected lane issues) ----
             const uint32_t el = tc::elect_one();
-            const uint32_t id = idesc(C::FMT, kRows, NP), idn = id | (1u << 13);  // bit 13: negate A
+            const uint32_t id = idesc(C::FMT, kRows, NP), idw = idesc(C::FMT, kRows, 2 * NP), idn = id | (1u << 13);  // bit 13: negate A
             // descriptor of B block 0 of stage 0; the others differ by (byte offset >> 4) in the address field
             const uint64_t dB0 = sdesc(smem_u32(sB), 128, Lt::SBO);
             const uint64_t dA0 = sdesc(smem_u32(sA), 128, Lt::SBO);
-            const uint32_t bblk16 = (uint32_t)(bblk >> 4);
+            const uint32_t bblk16 = bblk >> 4;
+            int j = 0;     // A buffer
             int gpos = 0;  // position of the stage in its accumulation group
             bool stop = false;
             for (int il = 0; il < n_it; il++) {
                 const uint32_t it = it_base + il;
                 const int s = it % S;
                 const uint32_t par = (it / S) & 1u;
-                uint64_t* af = C::ATM ? &afull : &full[s];
-                const uint32_t apar = C::ATM ? (it & 1u) : par;
+                uint64_t* af = C::ATM ? &afull[j] : &full[s];
+                const uint32_t apar = C::ATM ? (aph >> j & 1u) : par;
                 stop = !__all_sync(0xffffffffu, wait_or_abort(af, apar, &s_abort, wl) &&
                                                     wait_or_abort(&bfull[s], par, &s_abort, wl));
                 if (stop) break;
@@ -276,56 +391,48 @@ __device__ __forceinline__ void tc_item(const TcJob& J, const int4 wk, const uin
                 const uint64_t dBs = dB0 + (uint64_t)((s * Lt::B_STAGE) >> 4);
                 const uint64_t dAs = dA0 + (uint64_t)((s * Lt::A_STAGE) >> 4);
                 // a new accumulation group starts by overwriting the accumulators
-                const uint32_t first = gpos == 0 ? 0u : 1u;
+                const bool first = gpos == 0;
                 if (++gpos == gs) gpos = 0;
-#pragma unroll
-                for (int co = 0; co < 3; co++)
-#pragma unroll
-                    for (int ci = 0; ci < 3; ci++)
-#pragma unroll
-                        for (int pr = 0; pr < C::NPROD; pr++)
-#pragma unroll
-                            for (int ks = 0; ks < kKC / C::KMMA; ks++) {
-                                constexpr int kEnt[3][3] = {{0, 1, 4}, {1, 2, 5}, {4, 5, 3}};
-                                constexpr int kPa[6] = {0, 0, 1, 0, 2, 1}, kPb[6] = {0, 1, 0, 2, 0, 1};
-                                const int ablk = kEnt[co][ci] * C::NS + kPa[pr];
-                                const uint64_t db = dBs + (uint64_t)((ci * C::NS + kPb[pr]) * bblk16 + 16 * ks);
-                                const uint32_t idd = (ci == 2 && co < 2) ? idn : id;
-                                const uint32_t dt = tmem + (uint32_t)(co * NP);
-                                // the first product into each accumulator overwrites it
-                                const uint32_t en = (ci | pr | ks) ? 1u : first;
-                                if (C::ATM)  // A from tensor memory: block ablk, K step ks (8 columns per MMA)
-                                    tc::mma_ts<C::FMT == 2>(dt, tmem + kAcol + (uint32_t)ablk * Lt::ACOLS + 8u * ks, db, idd,
-                                                            en, el);
-                                else
-                                    tc::mma_ss(dt, dAs + (uint64_t)((ablk * Lt::ABLK + 256 * ks) >> 4), db, idd, en, el);
-                            }
-                if (C::ATM) tc::commit_elected(&aempty, el);
+                const uint32_t ta = tmem + a_col(j);
+                if (first)
+                    issue_stage<PREC, true>(tmem, ta, dAs, dBs, bblk16, NP, id, idw, idn, el);
+                else
+                    issue_stage<PREC, false>(tmem, ta, dAs, dBs, bblk16, NP, id, idw, idn, el);
+                if (C::ATM) {
+                    tc::commit_elected(&aempty[j], el);
+                    aph ^= 1u << j;
+                    if (++j == n_abuf) j = 0;
+                }
                 tc::commit_elected(&empty[s], el);
             }
             if (stop) s_abort = 1;
             tc::commit_elected(&done, el);  // also after a stop: fires once the issued products are complete
         } else {
-            // ---- builders (warps 0..7) ----
-            const int tid = threadIdx.x;                  // 0 .. 255
+            // ---- builders (warps 0..11) ----
+            const int tid = threadIdx.x;                  // 0 .. 383
             const int a_loc = (warp & 3) * 32 + lane;     // TMEM lane = GEMM row
-            const int hb = warp >> 2;                     // which 8 of the stage's 16 columns
+            const int pl = warp >> 2;                     // which two of the six entries
             const int a = tA * kRows + a_loc;
             const int2 xa = A.xy_p[a];
             const int4 bA = A.bbox_a[tA];
             const float* tk = A.tab32 + (size_t)(k - A.kbase) * A.Dy * A.Dx * 6;
+            // (a table buffer too small for padded rows: the builders copy it themselves)
+            const int sy0 = tid / (3 * A.W), sx0 = tid % (3 * A.W), dsy = kBuilders / (3 * A.W), dsx = kBuilders % (3 * A.W);
             // table sub-box and interface offsets of tile tB into buffer buf, by asynchronous copies
             auto stage_async = [&](int buf, int tB) {
                 const int4 bB = A.bbox_b[tB];
                 const int ox = bA.x - bB.y, oy = bA.z - bB.w;
-                float* dt = s_tab + (size_t)buf * HW * 6;
-                for (int e = tid; e < HW; e += kBuilders) {
-                    const int iy = e / A.W, ix = e - iy * A.W;
-                    const int gx = ox + ix - A.box_x0, gy = oy + iy - A.box_y0;
-                    const bool in = gx < A.Dx && gy < A.Dy;
-                    const float* src = in ? tk + ((size_t)gy * A.Dx + gx) * 6 : tk;  // zero fill outside the box
-#pragma unroll
-                    for (int h = 0; h < 3; h++) cp_async8(dt + (size_t)e * 6 + 2 * h, src + 2 * h, in ? 8 : 0);
+                const int gx0 = ox - A.box_x0, gy0 = oy - A.box_y0;
+                float2* dt = (float2*)(s_tab + (size_t)buf * J.tab_bytes);
+                // eight bytes a thread, neighbouring threads neighbouring ones: row iy, 8-byte word cx of it
+                const float2* t0 = (const float2*)tk + ((ptrdiff_t)gy0 * A.Dx + gx0) * 3;
+                const int cx_in = 3 * (A.Dx - gx0);
+                int iy = sy0, cx = sx0;
+                for (int e = tid; e < 3 * HW; e += kBuilders) {
+                    const bool in = cx < cx_in && gy0 + iy < A.Dy;  // zero fill outside the box
+                    cp_async8(dt + e, in ? t0 + ((ptrdiff_t)iy * A.Dx * 3 + cx) : (const float2*)tk, in ? 8 : 0);
+                    iy += dsy, cx += dsx;
+                    if (cx >= 3 * A.W) cx -= 3 * A.W, iy++;
                 }
                 if (tid < kTileB / 4) cp_async16(s_off + buf * kTileB + 4 * tid, A.off_i + tB * kTileB + 4 * tid);
                 asm volatile("cp.async.commit_group;" ::: "memory");
@@ -336,7 +443,7 @@ __device__ __forceinline__ void tc_item(const TcJob& J, const int4 wk, const uin
             // group writes, the later ones add.  The sums are FP32 values, kept in FP32.
             const uint32_t tacc = tmem + ((uint32_t)((warp & 3) * 32) << 16);
             auto drain = [&](bool add) {
-                for (int c0 = hb * 16; c0 < NP; c0 += 32) {
+                for (int c0 = pl * 16; c0 < NP; c0 += 48) {
                     float v0[16], v1[16], v2[16];
                     tc::ld16(tacc + (uint32_t)c0, v0);
                     tc::ld16(tacc + (uint32_t)(NP + c0), v1);
@@ -369,23 +476,35 @@ __device__ __forceinline__ void tc_item(const TcJob& J, const int4 wk, const uin
                 }
             };
             int il = 0, gpos = 0;  // stage of the item and its position in the accumulation group
-            if (nbuf == 2) stage_async(0, 0);
-            for (int tB = 0; tB < A.n_tb; tB++) {
-                if (nbuf == 1) {
-                    if (builders_sync_any(s_abort)) break;  // everyone is done with the previous tile
-                    stage_async(0, tB);
-                }
-                asm volatile("cp.async.wait_all;" ::: "memory");
-                // this tile's copies are visible to every builder, the previous tile is done;
-                // the same stop decision in every builder
-                if (builders_sync_any(s_abort)) break;
-                if (nbuf == 2 && tB + 1 < A.n_tb) stage_async((tB + 1) & 1, tB + 1);
-                const int buf = nbuf == 2 ? (tB & 1) : 0;
-                const float* tab_b = s_tab + (size_t)buf * HW * 6;
-                const int* off_b = s_off + buf * kTileB;
+            int j = 0;             // A buffer
+            const bool bulk = J.bulk;
+            const int pitch = J.pitch, om = bulk ? 1 : 24;  // bytes of a sub-box row, of a unit of s_off
+            if (!bulk && nbuf == 2) stage_async(0, 0);
+            for (int tB = 0, buf = 0; tB < A.n_tb; tB++, buf = buf + 1 == nbuf ? 0 : buf + 1) {
                 const int4 bB = A.bbox_b[tB];
+                if (bulk) {
+                    if (s_abort || !wait_or_abort(&tfull[buf], aph >> (8 + buf) & 1u, &s_abort, wl)) {
+                        s_abort = 1;
+                        break;
+                    }
+                    aph ^= 0x100u << buf;
+                } else {
+                    if (nbuf == 1) {
+                        if (builders_sync_any<kBuilders>(s_abort)) break;  // everyone is done with the previous tile
+                        stage_async(0, tB);
+                    }
+                    asm volatile("cp.async.wait_all;" ::: "memory");
+                    // this tile's copies are visible to every builder, the previous tile is done;
+                    // the same stop decision in every builder
+                    if (builders_sync_any<kBuilders>(s_abort)) break;
+                    if (nbuf == 2 && tB + 1 < A.n_tb) stage_async(buf ^ 1, tB + 1);
+                }
+                const unsigned char* tab_b = s_tab + (size_t)buf * J.tab_bytes;
+                const int* off_b = s_off + buf * kTileB;
                 const int ox = bA.x - bB.y, oy = bA.z - bB.w;
-                const int base = (xa.x - ox) + A.W * (xa.y - oy);
+                // byte offset of entries 2 pl of this row's difference to the origin; behind a shift of 0 or 8
+                const int odd = (((k - A.kbase) * A.Dy + oy - A.box_y0) * A.Dx + ox - A.box_x0) & 1;
+                const int base = 24 * (xa.x - ox) + (int)((unsigned)pitch * (unsigned)(xa.y - oy)) + 8 * pl + (bulk ? 8 * odd : 0);
                 for (int st = 0; st < kStagesPerTile; st++, il++) {
                     const uint32_t it = it_base + il;
                     const int s = it % S;
@@ -395,115 +514,89 @@ __device__ __forceinline__ void tc_item(const TcJob& J, const int4 wk, const uin
                         continue;  // keep the barrier count of the other builders
                     }
                     // At a group boundary, wait for the previous stage's products first (A in tensor
-                    // memory: the A buffer's release; otherwise the single stage's release above)
+                    // memory: its buffer's release; otherwise the single stage's release above)
                     // and drain the accumulators before gathering, where few registers are live.
-                    bool drained = false;
                     const bool boundary = il > 0 && gpos == 0;
                     if (++gpos == gs) gpos = 0;
                     if (boundary) {
-                        if (C::ATM && (s_abort || !wait_or_abort(&aempty, (it & 1u) ^ 1u, &s_abort, wl))) {
+                        const int jp = j == 0 ? n_abuf - 1 : j - 1;
+                        if (C::ATM && (s_abort || !wait_or_abort(&aempty[jp], aph >> jp & 1u, &s_abort, wl))) {
                             s_abort = 1;
                             continue;
                         }
                         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                         drain(il > gs);
                         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-                        drained = true;
                     }
-                    // row a_loc, columns st*16 + hb*8 .. + 7 of this tile: six entries, NS pieces each
-                    float v[8][6];
+                    // row a_loc, the stage's 16 columns: entries 2 pl and 2 pl + 1
+                    float2 v[kKC];
 #pragma unroll
-                    for (int i = 0; i < 8; i++) {
-                        const int idx = base - off_b[st * kKC + hb * 8 + i];
-                        const float2* src = (const float2*)(tab_b + (size_t)idx * 6);
-                        const float2 p0 = src[0], p1 = src[1], p2 = src[2];
-                        v[i][0] = p0.x, v[i][1] = p0.y, v[i][2] = p1.x, v[i][3] = p1.y, v[i][4] = p2.x, v[i][5] = p2.y;
+                    for (int i = 0; i < kKC; i += 4) {
+                        const int4 o = *(const int4*)(off_b + st * kKC + i);
+                        v[i] = *(const float2*)(tab_b + (base - om * o.x));
+                        v[i + 1] = *(const float2*)(tab_b + (base - om * o.y));
+                        v[i + 2] = *(const float2*)(tab_b + (base - om * o.z));
+                        v[i + 3] = *(const float2*)(tab_b + (base - om * o.w));
                     }
-                    // split into NS pieces: four 32-bit words (eight bf16, or four tf32 twice) per entry and piece
-                    uint32_t wq[6][C::NS][4], wt[6][2][4];
+                    // split into NS pieces: w[(entry, piece)][32-bit words of 16 elements], packed round-to-nearest
+                    // conversions with exact FP32 remainders (bf16), or one tf32 word per element
+                    constexpr int NW = kKC * C::ES / 4;
+                    uint32_t w[2 * C::NS * NW];
 #pragma unroll
-                    for (int e = 0; e < 6; e++) {
-                        float x[8];
-#pragma unroll
-                        for (int i = 0; i < 8; i++) x[i] = v[i][e];
+                    for (int p = 0; p < C::NS; p++) {
                         if (C::ES == 2) {
-                            // bf16 pieces two at a time: packed round-to-nearest conversion, exact FP32 remainders
 #pragma unroll
-                            for (int p = 0; p < C::NS; p++)
-#pragma unroll
-                                for (int i = 0; i < 4; i++) {
-                                    uint32_t w;
-                                    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(w) : "f"(x[2 * i + 1]), "f"(x[2 * i]));
-                                    wq[e][p][i] = w;
-                                    if (p + 1 < C::NS) {
-                                        x[2 * i] = __fsub_rn(x[2 * i], __uint_as_float(w << 16));
-                                        x[2 * i + 1] = __fsub_rn(x[2 * i + 1], __uint_as_float(w & 0xffff0000u));
-                                    }
+                            for (int i = 0; i < kKC; i += 2) {
+                                uint32_t h0, h1;
+                                asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(h0) : "f"(v[i + 1].x), "f"(v[i].x));
+                                asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(h1) : "f"(v[i + 1].y), "f"(v[i].y));
+                                w[p * NW + i / 2] = h0, w[(C::NS + p) * NW + i / 2] = h1;
+                                if (p + 1 < C::NS) {  // exact remainders, of a column's two entries at a time
+                                    upk2(sub2(pk2(v[i].x, v[i].y), pk2(__uint_as_float(h0 << 16), __uint_as_float(h1 << 16))),
+                                         v[i].x, v[i].y);
+                                    upk2(sub2(pk2(v[i + 1].x, v[i + 1].y), pk2(__uint_as_float(h0 & 0xffff0000u),
+                                                                               __uint_as_float(h1 & 0xffff0000u))),
+                                         v[i + 1].x, v[i + 1].y);
                                 }
+                            }
                         } else {
 #pragma unroll
-                            for (int q = 0; q < 2; q++)
-#pragma unroll
-                                for (int i = 0; i < 4; i++) asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(wt[e][q][i]) : "f"(x[4 * q + i]));
+                            for (int i = 0; i < kKC; i++) {
+                                asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(w[i]) : "f"(v[i].x));
+                                asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(w[NW + i]) : "f"(v[i].y));
+                            }
                         }
                     }
                     if (C::ATM) {
-                        // the tensor-memory A buffer is free once the previous stage's products are complete
-                        if (!drained && (s_abort || !wait_or_abort(&aempty, (it & 1u) ^ 1u, &s_abort, wl))) {
+                        // free once the products of the stage that had the buffer before are complete
+                        if (s_abort || !wait_or_abort(&aempty[j], aph >> j & 1u, &s_abort, wl)) {
                             s_abort = 1;
                             continue;
                         }
+                        aph ^= 1u << j;
                         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                        // lane = row a_loc; columns: block * ACOLS + this thread's K half
-                        const uint32_t trow = tmem + ((uint32_t)((warp & 3) * 32) << 16) + kAcol;
-#pragma unroll
-                        for (int e = 0; e < 6; e++) {
-                            if (C::ES == 2) {
-#pragma unroll
-                                for (int p = 0; p < C::NS; p++)
-                                    asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};" ::"r"(
-                                                     trow + (uint32_t)(e * C::NS + p) * Lt::ACOLS + 4u * hb),
-                                                 "r"(wq[e][p][0]), "r"(wq[e][p][1]), "r"(wq[e][p][2]), "r"(wq[e][p][3])
-                                                 : "memory");
-                            } else {
-                                asm volatile(
-                                    "tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(
-                                        trow + (uint32_t)e * Lt::ACOLS + 8u * hb),
-                                    "r"(wt[e][0][0]), "r"(wt[e][0][1]), "r"(wt[e][0][2]), "r"(wt[e][0][3]), "r"(wt[e][1][0]),
-                                    "r"(wt[e][1][1]), "r"(wt[e][1][2]), "r"(wt[e][1][3])
-                                    : "memory");
-                            }
-                        }
+                        // lane = row a_loc; this warp's entries and pieces: 32 columns in a row
+                        tc::st32(tmem + ((uint32_t)((warp & 3) * 32) << 16) + a_col(j) + 32u * pl, w);
                         asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
                         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
                         __syncwarp();
-                        if (lane == 0) mbar_arrive(&afull);
+                        if (lane == 0) mbar_arrive(&afull[j]);
+                        if (++j == n_abuf) j = 0;
                     } else {
-                        unsigned char* dstA = sA + s * Lt::A_STAGE;
+                        unsigned char* dstA = sA + s * Lt::A_STAGE + (size_t)(a_loc / 8) * Lt::SBO + (a_loc % 8) * 16;
 #pragma unroll
-                        for (int e = 0; e < 6; e++) {
-                            if (C::ES == 2) {
+                        for (int q = 0; q < 2 * C::NS; q++)
 #pragma unroll
-                                for (int p = 0; p < C::NS; p++) {
-                                    const uint32_t off = (uint32_t)(a_loc / 8) * Lt::SBO + hb * 128 + (a_loc % 8) * 16;
-                                    *(uint4*)(dstA + (size_t)(e * C::NS + p) * Lt::ABLK + off) =
-                                        make_uint4(wq[e][p][0], wq[e][p][1], wq[e][p][2], wq[e][p][3]);
-                                }
-                            } else {
-#pragma unroll
-                                for (int q = 0; q < 2; q++) {
-                                    const int kc = hb * 2 + q;
-                                    const uint32_t off = (uint32_t)(a_loc / 8) * Lt::SBO + kc * 128 + (a_loc % 8) * 16;
-                                    *(uint4*)(dstA + (size_t)e * Lt::ABLK + off) =
-                                        make_uint4(wt[e][q][0], wt[e][q][1], wt[e][q][2], wt[e][q][3]);
-                                }
-                            }
-                        }
+                            for (int i = 0; i < NW; i += 4)
+                                *(uint4*)(dstA + (size_t)(2 * pl * C::NS + q) * Lt::ABLK + 32 * i) =
+                                    make_uint4(w[q * NW + i], w[q * NW + i + 1], w[q * NW + i + 2], w[q * NW + i + 3]);
                         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                         __syncwarp();
                         if (lane == 0) mbar_arrive(&full[s]);
                     }
                 }
+                __syncwarp();
+                if (bulk && lane == 0) mbar_arrive(&tempty[buf]);
             }
             asm volatile("cp.async.wait_all;" ::: "memory");  // a prefetch still in flight after a stop
             // ---- epilogue: accumulators -> uh (FP64) ----
@@ -517,6 +610,12 @@ __device__ __forceinline__ void tc_item(const TcJob& J, const int4 wk, const uin
     }
 }
 
+// a filling role's first wait on a buffer passes, a reading role's does not
+__device__ __forceinline__ uint32_t first_parities() {
+    const int warp = threadIdx.x / 32;
+    return warp < kBuilderWarps ? 0xfu : warp == kTabWarp ? 0x300u : 0u;
+}
+
 template <int PREC>
 __device__ __forceinline__ void tc_setup(TcSync<TcCfg<PREC>::S>& sy) {
     constexpr int S = TcCfg<PREC>::S;
@@ -524,7 +623,8 @@ __device__ __forceinline__ void tc_setup(TcSync<TcCfg<PREC>::S>& sy) {
         sy.abort = 0;
         for (int s = 0; s < S; s++) mbar_init(&sy.full[s], kBuilderWarps), mbar_init(&sy.bfull[s], 1), mbar_init(&sy.empty[s], 1);
         mbar_init(&sy.done, 1);
-        mbar_init(&sy.afull, kBuilderWarps), mbar_init(&sy.aempty, 1);
+        for (int j = 0; j < kMaxABuf; j++) mbar_init(&sy.afull[j], kBuilderWarps), mbar_init(&sy.aempty[j], 1);
+        for (int j = 0; j < 2; j++) mbar_init(&sy.tfull[j], 1), mbar_init(&sy.tempty[j], kBuilderWarps);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (threadIdx.x / 32 == 0) {
@@ -553,7 +653,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_contract_tc(TcJob J, int wl, in
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ TcSync<TcCfg<PREC>::S> sy;
     tc_setup<PREC>(sy);
-    tc_item<PREC>(J, make_int4(0, J.A.k0 + (int)blockIdx.y, (int)blockIdx.x, (int)blockIdx.z), 0u, 0u, sy, smem, wl);
+    uint32_t aph = first_parities();
+    tc_item<PREC>(J, make_int4(0, J.A.k0 + (int)blockIdx.y, (int)blockIdx.x, (int)blockIdx.z), 0u, 0u, sy, smem, wl, aph);
     tc_teardown<PREC>(sy, status);
 }
 
@@ -571,7 +672,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     __shared__ int4 s_wk;
     __shared__ TcJob s_job;  // the current item's job
     tc_setup<PREC>(sy);
-    uint32_t it_base = 0, n_done = 0;
+    uint32_t it_base = 0, n_done = 0, aph = first_parities();
     for (;;) {
         if (threadIdx.x == 0) {
             const int ii = atomicAdd(counter, 1);
@@ -582,7 +683,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         __syncthreads();
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         if (s_item >= n_items || sy.abort) break;
-        tc_item<PREC>(s_job, s_wk, it_base, n_done, sy, smem, wl);
+        tc_item<PREC>(s_job, s_wk, it_base, n_done, sy, smem, wl, aph);
         it_base += (uint32_t)(s_job.A.n_tb * kStagesPerTile);
         n_done++;
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -593,15 +694,29 @@ __global__ void __launch_bounds__(kThreads, 1)
 }
 
 template <int PREC>
-size_t tc_smem(int HW, int nbuf) {
+size_t tc_smem(size_t tab_bytes, int nbuf) {
     using Lt = TcLayout<PREC>;
-    return TcCfg<PREC>::S * (Lt::A_STAGE + Lt::B_STAGE) + nbuf * ((size_t)6 * HW * 4 + (size_t)kTileB * 4) + 1024;
+    return TcCfg<PREC>::S * (Lt::A_STAGE + Lt::B_STAGE) + nbuf * (tab_bytes + (size_t)kTileB * 4) + 1024;
 }
-// two table buffers (the next tile prefetched) when they fit, else one
+// How a plan's table sub-boxes are staged: two buffers (the next tile prefetched) when they fit, else one; rows by bulk
+// copies with the pitch these need, unless that costs a buffer or does not fit: then the builders copy them with
+// cp.async, in 8-byte pieces without padding (4502 + 3001 columns, BF16X2, 16 right-hand sides: 11.3 ms, of which the
+// builders spent 40 % issuing these, against 8.3 ms by bulk copies).
+struct TcStaging {
+    int nbuf, bulk, pitch;
+    size_t tab_bytes, smem;
+};
 template <int PREC>
-int tc_nbuf(int HW) { return tc_smem<PREC>(HW, 2) <= 227 * 1024 ? 2 : 1; }
-template <int PREC>
-size_t tc_smem(int HW) { return tc_smem<PREC>(HW, tc_nbuf<PREC>(HW)); }
+TcStaging tc_staging(const Plan& P) {
+    const size_t flat = ((size_t)24 * P.W * P.H + 15) / 16 * 16, rows = ((size_t)contract_tc_pitch(P) * P.H + 47) / 16 * 16;
+    TcStaging t;
+    t.nbuf = tc_smem<PREC>(flat, 2) <= 227 * 1024 ? 2 : 1;
+    t.bulk = tc_smem<PREC>(rows, t.nbuf) <= 227 * 1024;
+    t.pitch = t.bulk ? contract_tc_pitch(P) : 24 * P.W;
+    t.tab_bytes = t.bulk ? rows : flat;
+    t.smem = tc_smem<PREC>(t.tab_bytes, t.nbuf);
+    return t;
+}
 
 int prep_groups(const Plan& P) { return (P.opt.max_rhs + kRhsPerCta - 1) / kRhsPerCta; }
 int prep_rows(const Plan& P) { return ((2 * std::min(kRhsPerCta, P.opt.max_rhs) + 15) / 16) * 16; }
@@ -626,7 +741,8 @@ cudaError_t prep_tc(const Plan& P, const double* fh, int rpc, int n_rhs, int k0,
 }
 
 template <int PREC>
-TcJob make_job(const ContractArgs& A, const Plan& P, int n_rhs, int rpc, int nbuf) {
+TcJob make_job(const ContractArgs& A, const Plan& P, int n_rhs, int rpc) {
+    const TcStaging t = tc_staging<PREC>(P);
     TcJob J;
     J.A = A;
     J.bprep = (const unsigned char*)P.d_bprep;
@@ -637,20 +753,21 @@ TcJob make_job(const ContractArgs& A, const Plan& P, int n_rhs, int rpc, int nbu
     // accumulation groups of kDrainTiles interface tiles (1024 columns), or one group
     const int n_it = P.n_tb * kStagesPerTile;
     J.gs = (P.opt.flags & FBC_PLAN_TC_FAST_ACCUMULATE) ? n_it : std::min(n_it, kDrainTiles * kStagesPerTile);
-    J.nbuf = nbuf;
+    J.nbuf = t.nbuf, J.bulk = t.bulk, J.pitch = t.pitch, J.tab_bytes = (int)t.tab_bytes;
+    J.off = P.d_off_tc;
     return J;
 }
 
 template <int PREC>
 cudaError_t launch_tc(const ContractArgs& A, const Plan& P, int n_rhs, cudaStream_t st, int n_modes) {
-    const size_t smem = tc_smem<PREC>(P.H * P.W);
-    if (smem > 227 * 1024) return cudaErrorInvalidConfiguration;
+    const size_t smem = tc_staging<PREC>(P).smem;
+    if (smem > 227 * 1024 || !P.d_off_tc) return cudaErrorInvalidConfiguration;
     if (!P.d_bprep || P.bprep_prec != PREC || n_rhs > P.opt.max_rhs) return cudaErrorInvalidValue;
     const int rpc = std::min(kRhsPerCta, P.opt.max_rhs);
     if (cudaError_t e = prep_tc<PREC>(P, A.fh, rpc, n_rhs, A.k0, n_modes, st)) return e;
     cudaError_t e = cudaFuncSetAttribute(k_contract_tc<PREC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e) return e;
-    const TcJob J = make_job<PREC>(A, P, n_rhs, rpc, tc_nbuf<PREC>(P.H * P.W));
+    const TcJob J = make_job<PREC>(A, P, n_rhs, rpc);
     dim3 grid(P.n_ta, n_modes, (n_rhs + rpc - 1) / rpc);
     const int wl = P.wait_limit > 0 ? P.wait_limit : tc::kWaitLimit;
     k_contract_tc<PREC><<<grid, kThreads, smem, st>>>(J, wl, P.d_status);
@@ -669,10 +786,17 @@ cudaError_t launch_tc_batch(const TcJob* d_jobs, const int4* d_items, int n_item
 
 }  // namespace
 
-size_t contract_tc_smem(int precision, int HW) {
-    if (precision == FBC_PREC_TF32) return tc_smem<FBC_PREC_TF32>(HW);
-    if (precision == FBC_PREC_BF16X2) return tc_smem<FBC_PREC_BF16X2>(HW);
-    return tc_smem<FBC_PREC_BF16X3>(HW);
+size_t contract_tc_smem(int precision, const Plan& P) {
+    if (precision == FBC_PREC_TF32) return tc_staging<FBC_PREC_TF32>(P).smem;
+    if (precision == FBC_PREC_BF16X2) return tc_staging<FBC_PREC_BF16X2>(P).smem;
+    return tc_staging<FBC_PREC_BF16X3>(P).smem;
+}
+// Bytes from row to row of a sub-box staged by bulk copies: room for 8 bytes on either side of a row's 24 W, and the
+// table's own pitch modulo 16.
+int contract_tc_pitch(const Plan& P) {
+    int p = 24 * P.W + 16;
+    if ((p & 15) != 8 * (P.Dx & 1)) p += 8;
+    return p;
 }
 
 size_t contract_tc_prep_bytes(const Plan& P, int precision) {
@@ -690,12 +814,6 @@ bool contract_tc_rpc_fits(const Plan& P, int rpc) {
     return want <= (long long)prep_groups(P) * prep_rows(P);
 }
 
-size_t contract_tc_nbuf_smem(int precision, int HW, int nbuf) {
-    if (precision == FBC_PREC_TF32) return tc_smem<FBC_PREC_TF32>(HW, nbuf);
-    if (precision == FBC_PREC_BF16X2) return tc_smem<FBC_PREC_BF16X2>(HW, nbuf);
-    return tc_smem<FBC_PREC_BF16X3>(HW, nbuf);
-}
-
 cudaError_t contract_tc_prep(const Plan& P, const double* fh, int rpc, int n_rhs, int k0, int n_modes, cudaStream_t st) {
     if (!P.d_bprep || P.bprep_prec != P.precision || !contract_tc_rpc_fits(P, rpc)) return cudaErrorInvalidValue;
     if (P.precision == FBC_PREC_TF32) return prep_tc<FBC_PREC_TF32>(P, fh, rpc, n_rhs, k0, n_modes, st);
@@ -704,11 +822,11 @@ cudaError_t contract_tc_prep(const Plan& P, const double* fh, int rpc, int n_rhs
     return cudaErrorInvalidValue;
 }
 
-TcJob contract_tc_job(const Plan& P, int n_rhs, int rpc, int nbuf) {
+TcJob contract_tc_job(const Plan& P, int n_rhs, int rpc) {
     const ContractArgs A = make_contract_args(P);
-    if (P.precision == FBC_PREC_TF32) return make_job<FBC_PREC_TF32>(A, P, n_rhs, rpc, nbuf);
-    if (P.precision == FBC_PREC_BF16X2) return make_job<FBC_PREC_BF16X2>(A, P, n_rhs, rpc, nbuf);
-    return make_job<FBC_PREC_BF16X3>(A, P, n_rhs, rpc, nbuf);
+    if (P.precision == FBC_PREC_TF32) return make_job<FBC_PREC_TF32>(A, P, n_rhs, rpc);
+    if (P.precision == FBC_PREC_BF16X2) return make_job<FBC_PREC_BF16X2>(A, P, n_rhs, rpc);
+    return make_job<FBC_PREC_BF16X3>(A, P, n_rhs, rpc);
 }
 
 cudaError_t launch_contract_tc_batch(int precision, const TcJob* d_jobs, const int4* d_items, int n_items,

@@ -103,7 +103,7 @@ struct Plan {
     float2* d_twl = nullptr;     // [L] exp(-2 pi i t / L) in FP32: the Stockham FP32 line transforms
     Fft1D line_fft;              // their passes (length L)
     double* d_table = nullptr;   // [K][Dy][Dx][6] FP64
-    float* d_table32 = nullptr;  // [K][Dy][Dx][6] FP32 (FBC_PREC_FP32)
+    float* d_table32 = nullptr;  // [K][Dy][Dx][6] FP32 (FBC_PREC_FP32), kTableTail floats more
     float* d_table_x2 = nullptr; // [K][Dy][Dx][12] hi/lo pairs (FBC_PREC_F32X2)
     float* d_table_x2_k0 = nullptr; // [Dy][Dx][12]: the k = 0 slice as hi/lo pairs (FP32 and tensor-core plans)
     double* d_fh = nullptr;      // [max_rhs][K][NIpad][6]
@@ -128,13 +128,14 @@ struct Plan {
     int2* d_far = nullptr;
     int2* d_near = nullptr;
     float* d_near32 = nullptr;   // [K][n_near][6] exact entries of the near field
-    float* d_slice = nullptr;    // [sur_chunk][Dy][Dx][6] streamed mode slices (FP32)
+    float* d_slice = nullptr;    // [sur_chunk][Dy][Dx][6] streamed mode slices (FP32), kTableTail floats more
     int sur_chunk = 0;           // modes per streamed chunk
     // tensor-core forms: the force operand split once per apply (fbc_contract_tc.cu)
     void* d_bprep = nullptr;
     size_t bprep_bytes = 0;
     int bprep_prec = -1;
     int* d_off_oz = nullptr;  // FBC_PREC_BF16X6: [NIpad] x_b + oz_pitch * y_b of the sorted interface sites, [NPpad] row order
+    int* d_off_tc = nullptr;  // tensor forms: [NIpad] 24 x_b + contract_tc_pitch y_b of the sorted interface sites
     int oz_pitch = 0;         // row pitch of its cut sub-boxes
     Seg seg64, segx2, seg0;        // segments of the interface sum (small plans)
     double* d_seg_part = nullptr;  // their partial sums and counters
@@ -144,6 +145,8 @@ struct Plan {
     size_t table_bytes = 0, workspace_bytes = 0;
     FftGrid* fft = nullptr;  // in-plane FFT form: grid, transformed kernel, workspace
 };
+
+constexpr int kTableTail = 4;  // floats after an FP32 table: a 16-byte copy of its last row may reach 8 bytes past it
 
 // Everything a contraction tile needs about one plan (one instance of a batch).
 struct ContractArgs {
@@ -177,6 +180,8 @@ struct TcJob {
     int npb;                     // force-operand rows per chunk: 2 rpc rounded up to 16
     int gs;                      // stages per tensor-memory accumulation group
     int nbuf;                    // table sub-box buffers in shared memory (2: the next tile prefetched)
+    int bulk, pitch, tab_bytes;  // rows staged by bulk copies, bytes from row to row, of a buffer
+    const int* off;              // [NIpad] byte offsets 24 x_b + pitch y_b (bulk)
 };
 
 // Everything the line transforms need about one plan (one instance of a batch).
@@ -237,15 +242,15 @@ cudaError_t launch_contract_x2_k0(Plan& P, const ContractArgs& A, int n_rhs, cud
 // streamed contraction of a plan with an attached surrogate (modes k >= 1)
 cudaError_t launch_contract_streamed(Plan& P, int n_rhs, cudaStream_t st);
 void release_surrogate_buffers(Plan& P);
-size_t contract_tc_smem(int precision, int HW);
-size_t contract_tc_nbuf_smem(int precision, int HW, int nbuf);
+size_t contract_tc_smem(int precision, const Plan& P);
+int contract_tc_pitch(const Plan& P);
 size_t contract_tc_prep_bytes(const Plan& P, int precision);
 // tensor-core batches: rhs groups a plan's operand buffer holds, the split of one instance's forces, its job
 // record, and the persistent launch over a queue of items (job, k, pad tile, rhs group)
 int contract_tc_max_rpc(const Plan& P);
 bool contract_tc_rpc_fits(const Plan& P, int rpc);
 cudaError_t contract_tc_prep(const Plan& P, const double* fh, int rpc, int n_rhs, int k0, int n_modes, cudaStream_t st);
-TcJob contract_tc_job(const Plan& P, int n_rhs, int rpc, int nbuf);
+TcJob contract_tc_job(const Plan& P, int n_rhs, int rpc);
 cudaError_t launch_contract_tc_batch(int precision, const TcJob* d_jobs, const int4* d_items, int n_items,
                                      int* d_counter, int grid, size_t smem, int wl, int* status, cudaStream_t st);
 // FBC_PREC_BF16X6 (fbc_contract_oz.cu): shared memory of the contraction, bytes of the sliced force

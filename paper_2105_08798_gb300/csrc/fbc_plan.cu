@@ -194,7 +194,7 @@ void free_plan(fbc::Plan& P) {
     void* bufs[] = {P.d_xy_p,  P.d_off_i,    P.d_bbox_a, P.d_bbox_b, P.d_perm_i, P.d_perm_p,
                     P.d_used,  P.d_rep,      P.d_tw,       P.d_twL,    P.d_twl,    P.d_table,  P.d_table32, P.d_table_x2, P.d_table_x2_k0,
                     P.d_fh,    P.d_uh,       P.d_part,   P.d_fpart, P.d_stage_f, P.d_stage_u, P.d_status, P.d_bprep,
-                    P.d_relax, P.d_uh32, P.d_off_oz, P.d_seg_part, P.d_seg_cnt};
+                    P.d_relax, P.d_uh32, P.d_off_oz, P.d_off_tc, P.d_seg_part, P.d_seg_cnt};
     for (void* b : bufs)
         if (b) cudaFree(b);
     for (auto& e : P.ev)
@@ -212,7 +212,7 @@ int ensure_derived(fbc::Plan& P, int precision) {
     const size_t cells = (size_t)P.K * P.Dy * P.Dx;
     size_t acc = 0;
     if ((precision == FBC_PREC_FP32 || fbc::is_tensor_precision(precision)) && !P.d_table32) {
-        int s = dev_alloc(&P.d_table32, cells * 6, acc, "table32");
+        int s = dev_alloc(&P.d_table32, cells * 6 + fbc::kTableTail, acc, "table32");
         if (s) return s;
     }
     // the tensor forms' split force operand, sized for this precision's pieces
@@ -235,6 +235,20 @@ int ensure_derived(fbc::Plan& P, int precision) {
     if (fbc::is_tensor_precision(precision) && !P.d_uh32) {
         int s = dev_alloc(&P.d_uh32, (size_t)P.opt.max_rhs * P.K * P.NPpad * 6, acc, "uh32");
         if (s) return s;
+    }
+    if (fbc::is_tensor_precision(precision) && !P.d_off_tc) {
+        int s = dev_alloc(&P.d_off_tc, P.NIpad, acc, "off_tc");
+        if (s) return s;
+        std::vector<int> off(P.NIpad);
+        const int pitch = fbc::contract_tc_pitch(P);
+        for (int t = 0; t < P.NIpad; t++) // (modulo 2^32: the kernel takes differences)
+            off[t] = (int)(24u * (unsigned)P.xy_i_sorted[t].x + (unsigned)pitch * (unsigned)P.xy_i_sorted[t].y);
+        cudaError_t e = cudaMemcpy(P.d_off_tc, off.data(), sizeof(int) * off.size(), cudaMemcpyHostToDevice);
+        if (e != cudaSuccess) {
+            cudaFree(P.d_off_tc);
+            P.d_off_tc = nullptr;
+            return cuda_fail(e, "off_tc");
+        }
     }
     // FBC_PREC_BF16X6: the double-float table and the sliced force operand with its scales
     if (precision == FBC_PREC_BF16X6 && P.bprep_prec != precision) {
@@ -623,7 +637,7 @@ static int apply_checks(fbc::Plan& P, const double* f, const double* u, int32_t 
     if (fc < uc + ub && uc < fc + fb) return fail(FBC_ERR_INVALID_ARG, "f and u overlap");
     if ((P.precision == FBC_PREC_FP32 || fbc::is_tensor_precision(P.precision)) && !P.d_table32 && !P.sur)
         return fail(FBC_ERR_INVALID_ARG, "FP32 table missing");
-    if (fbc::is_tensor_precision(P.precision) && fbc::contract_tc_smem(P.precision, P.W * P.H) > 227 * 1024)
+    if (fbc::is_tensor_precision(P.precision) && fbc::contract_tc_smem(P.precision, P) > 227 * 1024)
         return fail(FBC_ERR_UNSUPPORTED, "tensor-core contraction: staged sub-box too large for shared memory");
     if ((P.precision == FBC_PREC_F32X2 || P.precision == FBC_PREC_BF16X6) && !P.d_table_x2)
         return fail(FBC_ERR_INVALID_ARG, "double-float table missing");

@@ -718,7 +718,7 @@ int fbc_plan_attach_surrogate(fbc_plan* plan, fbc_surrogate* S, double r_min, in
     A((void**)&P.d_far, sizeof(int2) * far.size());
     A((void**)&P.d_near, sizeof(int2) * near.size());
     A((void**)&P.d_near32, sizeof(float) * 6 * near.size() * P.K);
-    A((void**)&P.d_slice, slice_bytes * chunk);
+    A((void**)&P.d_slice, slice_bytes * chunk + fbc::kTableTail * sizeof(float));
     if (!e && !far.empty()) e = cudaMemcpy(P.d_far, far.data(), sizeof(int2) * far.size(), cudaMemcpyHostToDevice);
     if (!e && !near.empty()) e = cudaMemcpy(P.d_near, near.data(), sizeof(int2) * near.size(), cudaMemcpyHostToDevice);
     // cells no pair reads stay zero (padding columns multiply them by zero forces)
@@ -746,7 +746,7 @@ int fbc_plan_attach_surrogate(fbc_plan* plan, fbc_surrogate* S, double r_min, in
         // the k = 0 double-float slice stays; the K-slice tables go
         const size_t kcells = (size_t)P.K * cells;
         if (P.d_table) cudaFree(P.d_table), P.d_table = nullptr;
-        if (P.d_table32) cudaFree(P.d_table32), P.d_table32 = nullptr, P.workspace_bytes -= kcells * 6 * sizeof(float);
+        if (P.d_table32) cudaFree(P.d_table32), P.d_table32 = nullptr, P.workspace_bytes -= (kcells * 6 + fbc::kTableTail) * sizeof(float);
         if (P.d_table_x2) cudaFree(P.d_table_x2), P.d_table_x2 = nullptr, P.workspace_bytes -= kcells * 12 * sizeof(float);
         P.tables_released = true;
         P.table_bytes = 0;
