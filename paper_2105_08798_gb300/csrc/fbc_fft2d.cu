@@ -32,7 +32,10 @@
 // out, two buffers used in turn): each pass gives every thread one
 // sub-transform of radix 8, 6, 5, 4, 3 or 2 in registers; the lengths are
 // chosen for the fewest passes (216 = 6 x 6 x 6, 320 = 5 x 8 x 8: three
-// passes through shared memory each).
+// passes through shared memory each).  The FP64 pipe bounds the FP64 ones: with
+// the butterflies of fbc_fft.cuh that fold the twiddles in, and first passes
+// that leave out the empty half of the grid, P1, P2 and P3 of 4000 + 6000 sites
+// at 129 modes take 0.32, 1.70 and 0.52 ms (0.46, 2.27 and 0.65 before).
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
@@ -68,6 +71,7 @@ struct FftGrid {
     int2* d_used = nullptr;        // [n_used] differences placed on the grid (table entries)
     unsigned char* d_mirror = nullptr;  // [n_used] 1: also place the mirror -d (it is not a table entry)
     int n_used = 0;
+    bool half_x = false, half_y = false;  // every interface site lies in the grid's lower half in x, in y
     size_t bytes = 0;
 };
 
@@ -75,7 +79,9 @@ namespace {
 
 using namespace fft;
 
-constexpr int kFftThreads = 384;  // one radix-8 work item per thread when a block holds 3 x 1024 points
+// FP32: one radix-8 work item per thread when a block holds 3 x 1024 points.  FP64: two such blocks an SM, with the
+// registers for their butterflies and twiddles (384 threads, 80 registers: the columns of 4000 + 6000 sites, 129 modes, took 1.80 ms, 1.70 so).
+template <typename R> constexpr int fft_threads() { return sizeof(R) == 4 ? 384 : 256; }
 constexpr int kSetupThreads = 256;
 constexpr int kRowElems = 1024;  // complex elements per component a block of P1 / P3 transforms
 
@@ -126,6 +132,7 @@ struct FftArgs {
     Fft1D fx, fy;
     int Mx, My, ny_i, ny_p, R, K, NIpad, NPpad, item0;
     double scale;
+    bool half_x, half_y;  // every interface site lies in the grid's lower half in x, in y
     // divisions of the index decodes: by the rows per block of P1 / P3, ny_i, ny_p and My
     unsigned mG, mNyi, mNyp, mMy;
     int lG, lNyi, lNyp, lMy;
@@ -133,7 +140,7 @@ struct FftArgs {
 
 // P1: rows of interface sites, forward FFT along x.  Block: G rows of one item.
 template <typename R>
-__global__ void __launch_bounds__(kFftThreads, sizeof(R) == 4 ? 3 : 2) k_fft_rows_fwd(FftArgs A, int G) {
+__global__ void __launch_bounds__(fft_threads<R>(), sizeof(R) == 4 ? 3 : 2) k_fft_rows_fwd(FftArgs A, int G) {
     using C = Cx<R>;
     extern __shared__ __align__(16) unsigned char smraw[];
     C* s = (C*)smraw;  // [G][3][Mx] (padded index), then the same again as scratch
@@ -151,7 +158,7 @@ __global__ void __launch_bounds__(kFftThreads, sizeof(R) == 4 ? 3 : 2) k_fft_row
         for (int c = 0; c < 3; c++) s[sx((g * 3 + c) * A.Mx + xp)] = mkc<C>((R)v[c], (R)v[3 + c]);
     }
     __syncthreads();
-    const C* res = fft_smem<false>(s, s + n, G * 3, A.fx, (const C*)A.twx);
+    const C* res = fft_smem<false, sizeof(R) == 8>(s, s + n, G * 3, A.fx, (const C*)A.twx, A.half_x);
     const int gr = min(G, A.ny_i - row0);
     C* out = (C*)A.T1 + (size_t)iq * A.Mx * A.ny_i * 3;
     for (int t = threadIdx.x; t < A.Mx * G * 3; t += blockDim.x) {
@@ -162,7 +169,7 @@ __global__ void __launch_bounds__(kFftThreads, sizeof(R) == 4 ? 3 : 2) k_fft_row
 
 // P2: G grid columns of one item: forward FFT along y, Mhat, inverse FFT along y, pad rows out.
 template <typename R>
-__global__ void __launch_bounds__(kFftThreads, sizeof(R) == 4 ? 3 : 2) k_fft_cols(FftArgs A, int G) {
+__global__ void __launch_bounds__(fft_threads<R>(), sizeof(R) == 4 ? 3 : 2) k_fft_cols(FftArgs A, int G) {
     using C = Cx<R>;
     extern __shared__ __align__(16) unsigned char smraw[];
     C* s = (C*)smraw;  // [G][3][My] (padded index), then the same again as scratch
@@ -176,7 +183,7 @@ __global__ void __launch_bounds__(kFftThreads, sizeof(R) == 4 ? 3 : 2) k_fft_col
         s[sx((g * 3 + c) * A.My + A.ypos_i[row])] = in[((size_t)(xi0 + g) * A.ny_i + row) * 3 + c];
     }
     __syncthreads();
-    C* z0p = fft_smem<false>(s, s + n, G * 3, A.fy, (const C*)A.twy);
+    C* z0p = fft_smem<false, sizeof(R) == 8>(s, s + n, G * 3, A.fy, (const C*)A.twy, A.half_y);
     for (int t = threadIdx.x; t < gc * A.My; t += blockDim.x) {
         const int g = fdiv(t, A.mMy, A.lMy), et = t - g * A.My;
         const R* m = (const R*)A.mhat + (((size_t)k * A.Mx + xi0 + g) * A.My + et) * 6;
@@ -189,7 +196,7 @@ __global__ void __launch_bounds__(kFftThreads, sizeof(R) == 4 ? 3 : 2) k_fft_col
         z0p[i2] = mkc<C>(fmx(a33, z2.x, -fmx(b13, z0.y, b23 * z1.y)), fmx(a33, z2.y, fmx(b13, z0.x, b23 * z1.x)));
     }
     __syncthreads();
-    const C* res = fft_smem<true>(z0p, z0p == s ? s + n : s, G * 3, A.fy, (const C*)A.twy);
+    const C* res = fft_smem<true, sizeof(R) == 8>(z0p, z0p == s ? s + n : s, G * 3, A.fy, (const C*)A.twy);
     C* out = (C*)A.T2 + (size_t)iq * A.Mx * A.ny_p * 3;
     for (int t = threadIdx.x; t < gc * A.ny_p * 3; t += blockDim.x) {
         const int q = t / 3, c = t - 3 * q, g = fdiv(q, A.mNyp, A.lNyp), row = q - g * A.ny_p;
@@ -199,7 +206,7 @@ __global__ void __launch_bounds__(kFftThreads, sizeof(R) == 4 ? 3 : 2) k_fft_col
 
 // P3: G pad rows of one item: inverse FFT along x, scale, scatter the pad sites into uh.
 template <typename R>
-__global__ void __launch_bounds__(kFftThreads, sizeof(R) == 4 ? 3 : 2) k_fft_rows_inv(FftArgs A, int G) {
+__global__ void __launch_bounds__(fft_threads<R>(), sizeof(R) == 4 ? 3 : 2) k_fft_rows_inv(FftArgs A, int G) {
     using C = Cx<R>;
     extern __shared__ __align__(16) unsigned char smraw[];
     C* s = (C*)smraw;  // [G][3][Mx] (padded index), then the same again as scratch
@@ -211,7 +218,7 @@ __global__ void __launch_bounds__(kFftThreads, sizeof(R) == 4 ? 3 : 2) k_fft_row
         s[sx((g * 3 + c) * A.Mx + xi)] = g < gr ? in[((size_t)xi * A.ny_p + row0 + g) * 3 + c] : mkc<C>(0, 0);
     }
     __syncthreads();
-    const C* res = fft_smem<true>(s, s + n, G * 3, A.fx, (const C*)A.twx);
+    const C* res = fft_smem<true, sizeof(R) == 8>(s, s + n, G * 3, A.fx, (const C*)A.twx);
     double* uk = A.uh + ((size_t)r * A.K + k) * A.NPpad * 6;
     const int e1 = A.row_p[row0 + gr];
     for (int e = A.row_p[row0] + threadIdx.x; e < e1; e += blockDim.x) {
@@ -391,6 +398,9 @@ int fft_prepare(Plan& P, int precision) {
         return report_error(FBC_ERR_UNSUPPORTED, "in-plane FFT: two sites share a grid residue");
     }
     F->ny_i = (int)ypos_i.size(), F->ny_p = (int)ypos_p.size();
+    F->half_x = F->half_y = true;
+    for (const int2& en : ent_i) F->half_x = F->half_x && 2 * (en.x & 4095) < Mx;
+    for (int y : ypos_i) F->half_y = F->half_y && 2 * y < My;
     std::vector<unsigned char> mirror(used.size());
     for (size_t u = 0; u < used.size(); u++) mirror[u] = uset.count({-used[u].x, -used[u].y}) ? 0 : 1;
     // workspace for Q (rhs, mode) items at a time, at most about 1 GiB
@@ -505,12 +515,12 @@ static cudaError_t run_fft_items(FftArgs A, const FftGrid* F, int i_begin, int i
     for (int i0 = i_begin; i0 < i_end; i0 += q_max) {
         const int q = std::min(q_max, i_end - i0);
         A.item0 = i0;
-        k_fft_rows_fwd<R><<<dim3((F->ny_i + Gr - 1) / Gr, q), kFftThreads, smem_r, st>>>(A, Gr);
+        k_fft_rows_fwd<R><<<dim3((F->ny_i + Gr - 1) / Gr, q), fft_threads<R>(), smem_r, st>>>(A, Gr);
         cudaError_t e = cudaGetLastError();
         if (e) return e;
-        k_fft_cols<R><<<dim3((F->Mx + Gc - 1) / Gc, q), kFftThreads, smem_c, st>>>(A, Gc);
+        k_fft_cols<R><<<dim3((F->Mx + Gc - 1) / Gc, q), fft_threads<R>(), smem_c, st>>>(A, Gc);
         if ((e = cudaGetLastError())) return e;
-        k_fft_rows_inv<R><<<dim3((F->ny_p + Gr - 1) / Gr, q), kFftThreads, smem_r, st>>>(A, Gr);
+        k_fft_rows_inv<R><<<dim3((F->ny_p + Gr - 1) / Gr, q), fft_threads<R>(), smem_r, st>>>(A, Gr);
         if ((e = cudaGetLastError())) return e;
     }
     return cudaSuccess;
@@ -522,7 +532,7 @@ cudaError_t launch_contract_fft(Plan& P, int n_rhs, cudaStream_t st) {
     FftArgs A{};
     A.fh = P.d_fh, A.uh = P.d_uh, A.T1 = F->d_T1, A.T2 = F->d_T2;
     A.row_i = F->d_row_i, A.ent_i = F->d_ent_i, A.row_p = F->d_row_p, A.ent_p = F->d_ent_p;
-    A.ypos_i = F->d_ypos_i, A.ypos_p = F->d_ypos_p;
+    A.ypos_i = F->d_ypos_i, A.ypos_p = F->d_ypos_p, A.half_x = F->half_x, A.half_y = F->half_y;
     A.fx = F->fx, A.fy = F->fy;
     A.Mx = F->Mx, A.My = F->My, A.ny_i = F->ny_i, A.ny_p = F->ny_p;
     A.R = n_rhs, A.K = P.K, A.NIpad = P.NIpad, A.NPpad = P.NPpad;
