@@ -667,8 +667,13 @@ __global__ void __launch_bounds__(kThreads, 1) k_contract_oz(OzArgs O, int wl, i
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(sy.tbase), "r"(kTmemCols));
 }
 
-// dynamic shared memory: the force ring, offsets, two cut sub-boxes of `cells` cells and the cells' magnitudes
-size_t oz_smem(int cells, int slots) { return (size_t)slots * kSlot + 2 * kTileB * 4 + (size_t)cells * (2 * 36 + 4) + 1024; }
+// shared memory: the force ring, offsets, two cut sub-boxes of `cells` cells and the cells' magnitudes (dynamic), and the
+// static part, which the dynamic one's alignment rounds up to 1024
+constexpr size_t kStaticSmem = 1024;
+static_assert(sizeof(OzSync) <= kStaticSmem, "the barriers fit");
+size_t oz_smem(int cells, int slots) {
+    return (size_t)slots * kSlot + 2 * kTileB * 4 + (size_t)cells * (2 * 36 + 4) + kStaticSmem;
+}
 constexpr size_t kMaxSmem = 227 * 1024;
 int oz_ring(int cells) {
     int n = kSlots;
@@ -752,7 +757,7 @@ size_t contract_oz_prep_bytes(const Plan& P) {
 }
 
 // Modes A.k0 .. K - 1 (A.k0 >= 1) of an FBC_PREC_BF16X6 plan: scales and slices of the forces, then the
-// contraction, one CTA per (pad tile, output component) x mode x group of 16 right-hand sides.
+// contraction, one CTA per (pad tile, output component) x mode x group of kRhs right-hand sides.
 cudaError_t launch_contract_oz(const ContractArgs& A, const Plan& P, int n_rhs, cudaStream_t st) {
     const int n_modes = P.K - A.k0;
     if (n_modes <= 0 || n_rhs < 1) return cudaSuccess;
@@ -784,8 +789,8 @@ cudaError_t launch_contract_oz(const ContractArgs& A, const Plan& P, int n_rhs, 
     const int wl = P.wait_limit > 0 ? P.wait_limit : tc::kWaitLimit;
     const dim3 grid3(3 * P.n_ta, n_modes, gu);
     auto launch = [&](auto kernel) -> cudaError_t {
-        if (cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) return e;
-        kernel<<<grid3, kThreads, smem, st>>>(O, wl, P.d_status);
+        if (cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(smem - kStaticSmem))) return e;
+        kernel<<<grid3, kThreads, smem - kStaticSmem, st>>>(O, wl, P.d_status);
         return cudaGetLastError();
     };
     // cells in registers: 12 a slicer thread cover the sub-boxes of compact tiles (36 x 42 at 8000 x 12000

@@ -693,10 +693,13 @@ __global__ void __launch_bounds__(kThreads, 1)
     tc_teardown<PREC>(sy, status);
 }
 
+// with the static part, which the dynamic one's alignment rounds up to 1024
+constexpr size_t kStaticSmem = 1024;
+static_assert(sizeof(TcSync<3>) + sizeof(TcJob) + 32 <= kStaticSmem, "the barriers and the queue's job fit");
 template <int PREC>
 size_t tc_smem(size_t tab_bytes, int nbuf) {
     using Lt = TcLayout<PREC>;
-    return TcCfg<PREC>::S * (Lt::A_STAGE + Lt::B_STAGE) + nbuf * (tab_bytes + (size_t)kTileB * 4) + 1024;
+    return TcCfg<PREC>::S * (Lt::A_STAGE + Lt::B_STAGE) + nbuf * (tab_bytes + (size_t)kTileB * 4) + kStaticSmem;
 }
 // How a plan's table sub-boxes are staged: two buffers (the next tile prefetched) when they fit, else one; rows by bulk
 // copies with the pitch these need, unless that costs a buffer or does not fit: then the builders copy them with
@@ -760,8 +763,8 @@ TcJob make_job(const ContractArgs& A, const Plan& P, int n_rhs, int rpc) {
 
 template <int PREC>
 cudaError_t launch_tc(const ContractArgs& A, const Plan& P, int n_rhs, cudaStream_t st, int n_modes) {
-    const size_t smem = tc_staging<PREC>(P).smem;
-    if (smem > 227 * 1024 || !P.d_off_tc) return cudaErrorInvalidConfiguration;
+    const size_t all = tc_staging<PREC>(P).smem, smem = all - kStaticSmem;
+    if (all > 227 * 1024 || !P.d_off_tc) return cudaErrorInvalidConfiguration;
     if (!P.d_bprep || P.bprep_prec != PREC || n_rhs > P.opt.max_rhs) return cudaErrorInvalidValue;
     const int rpc = std::min(kRhsPerCta, P.opt.max_rhs);
     if (cudaError_t e = prep_tc<PREC>(P, A.fh, rpc, n_rhs, A.k0, n_modes, st)) return e;
@@ -776,7 +779,8 @@ cudaError_t launch_tc(const ContractArgs& A, const Plan& P, int n_rhs, cudaStrea
 
 template <int PREC>
 cudaError_t launch_tc_batch(const TcJob* d_jobs, const int4* d_items, int n_items, int* d_counter, int grid,
-                            size_t smem, int wl, int* status, cudaStream_t st) {
+                            size_t all, int wl, int* status, cudaStream_t st) {
+    const size_t smem = all - kStaticSmem;
     cudaError_t e =
         cudaFuncSetAttribute(k_contract_tc_queue<PREC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e) return e;
