@@ -26,9 +26,11 @@
 //     pair as seven tcgen05.mma (M = 128, N = 2 R or 4 R, K = 16 bf16 / 8 tf32)
 //     into three TMEM accumulators (one per output component); commits hand the
 //     stage back to the builders and the copy thread.
-// What bounds it: at 16 right-hand sides the gathers (a stage's 192 shared
-// loads take about 900 cycles with their bank conflicts) and the issue of the
-// products (21 of some 36 cycles) about equally; from N = 128 the tensor pipe.
+// What bounds it: at 16 right-hand sides the issue of a stage's products (21 of
+// some 36 cycles) and the hand-overs around it (a wait on a completed barrier
+// takes 100 to 160 cycles); from N = 128 the tensor pipe.  (The gathers' bank
+// conflicts are not it: rows dealt to the warps by bank, 3.7 wavefronts a gather
+// for 4.5, made it slower, 10.8 ms an update for 10.4.)
 // 4502 + 3001 columns, L = 512, 16 right-hand sides, BF16X2: 11.9 ms with eight
 // builder warps (12 tcgen05.st a stage each), one A operand and sub-boxes
 // copied by the builders, 8.3 ms now; 64 right-hand sides, L = 64: 4.3 and
