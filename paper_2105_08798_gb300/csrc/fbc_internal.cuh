@@ -77,7 +77,9 @@ struct Plan {
     fbc_options opt{};
     MaterialDev mat{};
     TabulateParams tp{};
-    // cubic medium: quadrature nodes and scaled constants of the tabulation (made on first use)
+    // cubic medium: whether the FP64-type tables take the polynomial form (cubic_poly_form), quadrature nodes and
+    // scaled constants of the tabulation (made on first use)
+    bool tab_poly = false;
     MaterialDev tab_mat{};
     double tab_pre = 0.0;
     std::vector<double> tab_nodes;
@@ -203,6 +205,7 @@ struct LineArgs {
 };
 
 // ---- launchers (each returns the launch's cudaError_t) ---------------------
+bool cubic_poly_form(const fbc_material& m, int nquad);
 cudaError_t launch_tabulate(Plan& P, cudaStream_t st);
 // The periodic kernel in real space, G~(d, s) for s = 0..L/2 (the stage before the line DFT), as
 // FP32 six-entry records at every cell of the difference box: out[Dy * Dx][L/2 + 1][6] (11, 12, 22,

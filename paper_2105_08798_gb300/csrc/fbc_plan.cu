@@ -470,6 +470,7 @@ int fbc_plan_create(const fbc_geometry* geom, const fbc_material* mat, const fbc
         P.mat.kelvin_a = 3.0 - 4.0 * mat->nu;
     } else {
         christoffel_form(*mat, Q, P.mat.K);
+        P.tab_poly = fbc::cubic_poly_form(*mat, opt.quad);
     }
     P.tp.L = L, P.tp.K = P.K, P.tp.Lh = L / 2, P.tp.c = P.c;
     P.tp.rich_n = opt.rich_n, P.tp.rich_N = opt.rich_N;

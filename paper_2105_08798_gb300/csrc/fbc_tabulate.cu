@@ -155,8 +155,8 @@ __device__ __forceinline__ CubicDir cubic_dir(double rx, double ry) {
 // part E and odd part O of the determinant serve both, 1/(E+O) +- 1/(E-O) = (2 E, -2 O) / ((E+O)(E-O)), and
 // one division serves two such pairs.  About 11 FP64 operations a node and 400 a point.  The coefficients' rounding is
 // the same at every node and does not average out, so the directions enter as quotients of exact squares, the
-// products are fused and the sums are taken in groups of eight pairs: emulated against 64-bit mantissas over a
-// slab's points the entries' error is then that of the node-by-node form (3.11e-16 and 3.12e-16 of |G|).
+// products are fused and the sums are taken in groups of eight pairs.  That rounding is relative to the largest
+// products of the entries of M, not to the determinant at a node: the form serves the media cubic_poly_form lets through.
 // The 1000 x 1500, L = 64 cubic slab's table: 112.3 ms with its first update before, 6.9 ms now;
 // 4000 x 6000, L = 256: 1676 ms before, 97 ms now (433 ms with the node-by-node form).
 __device__ void green_cubic(const CubicDir& D, double rx, double ry, double rz, double g[6]) {
@@ -261,7 +261,8 @@ __device__ void green_cubic(const CubicDir& D, double rx, double ry, double rz, 
     g[5] = entry(A[3]);
 }
 
-// Which Green function a launch evaluates.  The polynomial form serves the plans of the FP64-accurate precisions.
+// Which Green function a launch evaluates.  The polynomial form serves the plans of the FP64-accurate precisions whose
+// medium and node count cubic_poly_form lets through.
 // The others round the table to 32 bits or fewer, where a last-bit change of a few FP64 entries moves the
 // rounding of some (1e-9 to 4e-9 of an update, more than those forms differ by from run to run): they and the
 // H-matrix's FP32 table keep the node-by-node form's bits.
@@ -425,6 +426,31 @@ __global__ void k_derive_x2(const double* __restrict__ t64, float* __restrict__ 
 
 }  // namespace
 
+// Whether the polynomial form is as exact as the node-by-node one for a cubic medium: the cube of the mean eigenvalue of
+// M(z) (its trace is C11 + 2 C44 for every unit z) over the smallest determinant at most 3, from 48 nodes on.  The
+// determinant is linear in the elementary symmetric functions p, q of the squared components of z, so its minimum lies
+// on the border of the range of (p, q), which the directions with squares (t, t, 1 - 2 t) reach.
+// Errors against 64-bit mantissas (both forms emulated, 64 nodes, points of a slab), polynomial over node by node: 1500
+// random media below 3, of |G| 0.71 to 0.89 on average and 1.03 at most, of the image sum 0.80 to 0.95 on average
+// (single media scatter, 0.6 to 1.5).  Beyond, media of every bulk modulus: 1.2 at 4, 2 at 10, and without bound:
+//     C11, C12, C44           quantity    rms error of |G|, nodes / poly     of the image sum
+//     1.5, 1.0, 0.9              2.8        3.0e-16 / 3.0e-16              1.3e-13 / 1.4e-13
+//     1.0, 0.9, 0.45             8.1        3.3e-16 / 6.3e-16              1.2e-13 / 2.7e-13
+//     1.0, 0.2, 0.01           390          3.0e-16 / 5.8e-15              2.7e-14 / 1.3e-13
+//     1.0, 0.99, 0.005        1500          6.6e-15 / 1.1e-13              6.9e-13 / 9.4e-12
+// With fewer nodes the coefficients' rounding weighs more: below 3, 0.92 to 1.06 and 1.02 to 1.28 on average at 16 nodes,
+// 0.75 to 0.86 and 0.88 to 1.04 at 48.
+bool cubic_poly_form(const fbc_material& m, int nquad) {
+    const double tr = m.C11 + 2.0 * m.C44, c11 = m.C11 / tr, c12 = m.C12 / tr, c44 = m.C44 / tr;  // any unit of stress
+    const double h = c11 - c12 - 2.0 * c44;  // zero: isotropic
+    double det = HUGE_VAL;
+    for (int j = 0; j <= 96; j++) {  // (t = 0, 1/3, 1/2: the axes <100>, <111>, <110>)
+        const double t = j / 192.0, r = 1.0 - 2.0 * t, p = t * (t + 2.0 * r), q = t * t * r;
+        det = std::min(det, c11 * c44 * c44 + h * ((c11 + c12) * c44 * p + h * (c11 + 2.0 * c12 + c44) * q));
+    }
+    return nquad >= 48 && 1.0 <= 3.0 * 27.0 * det;
+}
+
 // The plan's medium and tabulation parameters into this file's constant memory (shared by every
 // plan: uploaded again before each use).  The copies' sources live in the plan.
 static cudaError_t upload_tabulate_constants(Plan& P, int kind, cudaStream_t st) {
@@ -504,7 +530,9 @@ cudaError_t launch_tabulate(Plan& P, cudaStream_t st) {
         cudaError_t e = cudaFuncSetAttribute(k_line_dft, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e) return e;
     }
-    const int kind = P.mat.kind == FBC_MATERIAL_ISOTROPIC ? kGreenIso : line_fp32(P.precision) ? kGreenNodes : kGreenPoly;
+    const int kind = P.mat.kind == FBC_MATERIAL_ISOTROPIC          ? kGreenIso
+                     : line_fp32(P.precision) || !P.tab_poly ? kGreenNodes
+                                                             : kGreenPoly;
     return tabulate_chunks(P, kind, st, [&](int d0, int nd, const double* gs) {
         const int bt = std::min(256, std::max(32, ((P.K + 31) / 32) * 32));
         k_line_dft<<<nd, bt, smem, st>>>(P.d_rep + d0, gs, P.d_twL, P.d_table);
