@@ -130,7 +130,7 @@ struct FftArgs {
     const void* twx;
     const void* twy;
     Fft1D fx, fy;
-    int Mx, My, ny_i, ny_p, R, K, NIpad, NPpad, item0;
+    int Mx, My, ny_i, ny_p, R, K, NIpad, NPpad, n_p, item0;
     double scale;
     bool half_x, half_y;  // every interface site lies in the grid's lower half in x, in y
     // divisions of the index decodes: by the rows per block of P1 / P3, ny_i, ny_p and My
@@ -204,7 +204,10 @@ __global__ void __launch_bounds__(fft_threads<R>(), sizeof(R) == 4 ? 3 : 2) k_ff
     }
 }
 
-// P3: G pad rows of one item: inverse FFT along x, scale, scatter the pad sites into uh.
+// P3: G pad rows of one item: inverse FFT along x, scale, scatter the pad sites into uh.  Of the padding slots behind the
+// n_p sites only the first is read to any effect: the inverse line transform carries the third components of two
+// neighbouring slots in one complex sequence, so with n_p odd the last site shares one with it, and it has to be zero (the
+// dense forms leave a repeated site's values there).
 template <typename R>
 __global__ void __launch_bounds__(fft_threads<R>(), sizeof(R) == 4 ? 3 : 2) k_fft_rows_inv(FftArgs A, int G) {
     using C = Cx<R>;
@@ -220,6 +223,7 @@ __global__ void __launch_bounds__(fft_threads<R>(), sizeof(R) == 4 ? 3 : 2) k_ff
     __syncthreads();
     const C* res = fft_smem<true, sizeof(R) == 8>(s, s + n, G * 3, A.fx, (const C*)A.twx);
     double* uk = A.uh + ((size_t)r * A.K + k) * A.NPpad * 6;
+    if (blockIdx.x == 0 && (A.n_p & 1) && threadIdx.x < 6) uk[(size_t)A.n_p * 6 + threadIdx.x] = 0.0;
     const int e1 = A.row_p[row0 + gr];
     for (int e = A.row_p[row0] + threadIdx.x; e < e1; e += blockDim.x) {
         const int2 en = A.ent_p[e];
@@ -535,7 +539,7 @@ cudaError_t launch_contract_fft(Plan& P, int n_rhs, cudaStream_t st) {
     A.ypos_i = F->d_ypos_i, A.ypos_p = F->d_ypos_p, A.half_x = F->half_x, A.half_y = F->half_y;
     A.fx = F->fx, A.fy = F->fy;
     A.Mx = F->Mx, A.My = F->My, A.ny_i = F->ny_i, A.ny_p = F->ny_p;
-    A.R = n_rhs, A.K = P.K, A.NIpad = P.NIpad, A.NPpad = P.NPpad;
+    A.R = n_rhs, A.K = P.K, A.NIpad = P.NIpad, A.NPpad = P.NPpad, A.n_p = P.n_p;
     A.scale = 1.0 / ((double)F->Mx * (double)F->My);
     const int items = n_rhs * P.K;
     // FP64: every mode; FP32 form: the logarithmic k = 0 mode (items 0 .. n_rhs - 1) stays FP64
