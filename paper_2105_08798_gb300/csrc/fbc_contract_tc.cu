@@ -44,9 +44,10 @@
 // given up; on a timeout the CTA records the status word, stops, waits for its
 // own bulk copies and tensor-core work -- those two waits ignore the stop and
 // keep the full bound, since the CTA may not exit or free its tensor memory
-// while either is in flight -- frees its tensor memory and returns.  Warps that
-// synchronise on a named barrier decide to stop only right after it, so none
-// is left waiting there.
+// while either is in flight -- frees its tensor memory and returns.  A warp
+// decides to stop as a whole (its tensor-memory accesses take every lane), and
+// warps that synchronise on a named barrier leave only right after it, so none
+// is left waiting.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -477,6 +478,13 @@ __device__ __forceinline__ void tc_item(const TcJob& J, const int4 wk, const uin
                     }
                 }
             };
+            // A pipeline wait of a builder warp, and its stop decision: one for all lanes, since what follows (tensor-memory
+            // loads and stores, __syncwarp) takes the whole warp and lanes that left it would be waited for without a bound.
+            auto wait_warp = [&](uint64_t* m, uint32_t parity) {
+                const bool go = __all_sync(0xffffffffu, !s_abort && wait_or_abort(m, parity, &s_abort, wl));
+                if (!go) s_abort = 1;
+                return go;
+            };
             int il = 0, gpos = 0;  // stage of the item and its position in the accumulation group
             int j = 0;             // A buffer
             const bool bulk = J.bulk;
@@ -485,10 +493,7 @@ __device__ __forceinline__ void tc_item(const TcJob& J, const int4 wk, const uin
             for (int tB = 0, buf = 0; tB < A.n_tb; tB++, buf = buf + 1 == nbuf ? 0 : buf + 1) {
                 const int4 bB = A.bbox_b[tB];
                 if (bulk) {
-                    if (s_abort || !wait_or_abort(&tfull[buf], aph >> (8 + buf) & 1u, &s_abort, wl)) {
-                        s_abort = 1;
-                        break;
-                    }
+                    if (!wait_warp(&tfull[buf], aph >> (8 + buf) & 1u)) break;
                     aph ^= 0x100u << buf;
                 } else {
                     if (nbuf == 1) {
@@ -511,10 +516,8 @@ __device__ __forceinline__ void tc_item(const TcJob& J, const int4 wk, const uin
                     const uint32_t it = it_base + il;
                     const int s = it % S;
                     const uint32_t u = it / S;
-                    if (!C::ATM && (s_abort || !wait_or_abort(&empty[s], (u & 1u) ^ 1u, &s_abort, wl))) {
-                        s_abort = 1;
-                        continue;  // keep the barrier count of the other builders
-                    }
+                    // (a stop ends the tile; the next one's start ends the item, on the barrier where the builders have one)
+                    if (!C::ATM && !wait_warp(&empty[s], (u & 1u) ^ 1u)) break;
                     // At a group boundary, wait for the previous stage's products first (A in tensor
                     // memory: its buffer's release; otherwise the single stage's release above)
                     // and drain the accumulators before gathering, where few registers are live.
@@ -522,10 +525,7 @@ __device__ __forceinline__ void tc_item(const TcJob& J, const int4 wk, const uin
                     if (++gpos == gs) gpos = 0;
                     if (boundary) {
                         const int jp = j == 0 ? n_abuf - 1 : j - 1;
-                        if (C::ATM && (s_abort || !wait_or_abort(&aempty[jp], aph >> jp & 1u, &s_abort, wl))) {
-                            s_abort = 1;
-                            continue;
-                        }
+                        if (C::ATM && !wait_warp(&aempty[jp], aph >> jp & 1u)) break;
                         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                         drain(il > gs);
                         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -571,10 +571,7 @@ __device__ __forceinline__ void tc_item(const TcJob& J, const int4 wk, const uin
                     }
                     if (C::ATM) {
                         // free once the products of the stage that had the buffer before are complete
-                        if (s_abort || !wait_or_abort(&aempty[j], aph >> j & 1u, &s_abort, wl)) {
-                            s_abort = 1;
-                            continue;
-                        }
+                        if (!wait_warp(&aempty[j], aph >> j & 1u)) break;
                         aph ^= 1u << j;
                         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                         // lane = row a_loc; this warp's entries and pieces: 32 columns in a row
@@ -605,7 +602,7 @@ __device__ __forceinline__ void tc_item(const TcJob& J, const int4 wk, const uin
             // the MMA thread commits `done` once per item on every path, also after a stop; every product it
             // issued is complete once `done` fires, so this wait keeps the full bound whatever the stop flag says
             const bool done_ok = tc::mbar_wait(&done, n_done & 1u);
-            const bool ok = done_ok && !s_abort;
+            const bool ok = __all_sync(0xffffffffu, done_ok && !s_abort);
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             if (ok) drain(n_it > gs);  // the last group; earlier groups were drained in the loop
         }
