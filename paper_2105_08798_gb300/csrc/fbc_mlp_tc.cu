@@ -71,18 +71,21 @@ __device__ __forceinline__ uint32_t bf16_pair(float lo, float hi) {
     return r;
 }
 
-// SiLU of z0 and z1, z / (1 + 2^(-z log2 e)), split into bf16 pieces hi + lo.  One reciprocal serves both (the exponents
-// are held below 60: beyond, where |SiLU| < 1e-16, the product of the two would overflow).  The approximate instructions
-// are good to about 2^-22, the pieces to 2^-17.
+// SiLU of z0 and z1, z / (1 + 2^(-z log2 e)), split into bf16 pieces hi + lo.  One reciprocal serves both: each z is held at
+// -41.5 from below (a NaN stays one), so that the product of the two denominators stays below 2^120; there and beyond the
+// result is -4e-17 where |SiLU| is at most that.  The factors that multiply z are at most 1: a large z passes through
+// whatever its neighbour is.  The approximate instructions are good to about 2^-22, the pieces to 2^-17.
 __device__ __forceinline__ void silu_split2(float z0, float z1, uint32_t& hi, uint32_t& lo) {
     float t0, t1, e0, e1, a0, a1, r, v0, v1;
+    asm("max.NaN.f32 %0, %1, %2;" : "=f"(z0) : "f"(z0), "f"(-41.5f));
+    asm("max.NaN.f32 %0, %1, %2;" : "=f"(z1) : "f"(z1), "f"(-41.5f));
     const uint64_t z = pk2(z0, z1);
     upk2(mul2(z, pk2(-1.4426950408889634f, -1.4426950408889634f)), t0, t1);
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e0) : "f"(fminf(t0, 60.f)));
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e1) : "f"(fminf(t1, 60.f)));
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e0) : "f"(t0));
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e1) : "f"(t1));
     upk2(add2(pk2(e0, e1), pk2(1.f, 1.f)), a0, a1);
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a0 * a1));
-    const uint64_t v = mul2(mul2(z, pk2(a1, a0)), pk2(r, r));
+    const uint64_t v = mul2(z, mul2(pk2(a1, a0), pk2(r, r)));
     upk2(v, v0, v1);
     hi = bf16_pair(v0, v1);
     upk2(sub2(v, pk2(__uint_as_float(hi << 16), __uint_as_float(hi & 0xffff0000u))), v0, v1);
