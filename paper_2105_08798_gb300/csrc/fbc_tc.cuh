@@ -76,17 +76,6 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* m, uint32_t phase) {
     return false;
 }
 
-__device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint64_t da, uint64_t db, uint32_t id, uint32_t accum) {
-    asm volatile(
-        "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem_d),
-        "l"(da), "l"(db), "r"(id), "r"(accum));
-}
-
-__device__ __forceinline__ void commit(uint64_t* m) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(m)));
-}
-
 // Issue of products from a whole, converged warp: the warp runs the loop, and one elected lane's predicate
 // guards each instruction.  Issued from a branch that only one thread takes, a product cost 45 to 83 cycles
 // whatever its size (its operands then pass through per-thread registers); issued this way M = 128, K = 16
@@ -175,7 +164,7 @@ __device__ __forceinline__ bool wait_or_abort_sleep(uint64_t* m, uint32_t parity
 // Named barrier 1 among the NT threads of the builder warps that also returns,
 // to every one of them, whether any passed flag != 0: a decision all of them
 // take alike.
-template <int NT = 256>
+template <int NT>
 __device__ __forceinline__ bool builders_sync_any(int flag) {
     uint32_t r;
     asm volatile(
@@ -204,17 +193,6 @@ __device__ __forceinline__ void cp_async8(void* dst, const void* src, int src_by
 }
 __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
-}
-
-// 4 bytes, or zero when src_bytes is 0
-__device__ __forceinline__ void cp_async4(void* dst, const void* src, int src_bytes) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(src_bytes)
-                 : "memory");
-}
-// 16 bytes, of which the first src_bytes (0 or 16) come from global memory and the rest are zero
-__device__ __forceinline__ void cp_async16z(void* dst, const void* src, int src_bytes) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(src_bytes)
-                 : "memory");
 }
 
 // 4 consecutive FP32 accumulator columns of this thread's TMEM lane (no wait: follow with tcgen05.wait::ld)
