@@ -23,7 +23,7 @@
 // isotropic medium and Barnett's integral over the unit circle normal to r,
 //     G(r) = 1/(8 pi^2 |r|) int_0^{2 pi} (zz)^{-1} dpsi,
 // for a cubic one, evaluated by the trapezoid rule on [0, pi) (the integrand
-// has period pi) with the nodes' cosines and sines in constant memory.
+// has period pi) with the nodes' cosines and sines among the kernel's parameters.
 //
 // The reference terms G(0, 0, +-m l3) depend on m alone and are computed once; of each pair d, -d only one is
 // evaluated.  Together four times fewer Green functions than one thread per (d, s) evaluating all of
@@ -37,20 +37,33 @@
 namespace fbc {
 namespace {
 
-__constant__ MaterialDev c_mat;
-__constant__ TabulateParams c_tp;
-__constant__ double c_qcos[kMaxQuad];     // the quadrature nodes psi
-__constant__ double c_qsin[kMaxQuad];
-__constant__ double c_node[kMaxQuad][6];  // cos and sin of 2 psi, 4 psi and 6 psi at the quadrature nodes
-__constant__ double c_pre;                // cubic medium: (scale of the constants) / (pi nquad)
+// Which Green function a launch evaluates.  The polynomial form serves the plans of the FP64-accurate precisions whose
+// medium and node count cubic_poly_form lets through.
+// The others round the table to 32 bits or fewer, where a last-bit change of a few FP64 entries moves the
+// rounding of some (1e-9 to 4e-9 of an update, more than those forms differ by from run to run): they and the
+// H-matrix's FP32 table keep the node-by-node form's bits.
+enum { kGreenIso = 0, kGreenNodes = 1, kGreenPoly = 2 };
+
+// A launch's medium and quadrature nodes: kernel parameters, so that plans tabulated on different streams at the same
+// time keep their own.
+struct Medium {
+    MaterialDev m;
+    double pre;  // polynomial form: (scale of the constants) / (pi nquad)
+};
+// cos and sin of psi at the nodes (node by node), or of 2 psi, 4 psi and 6 psi
+template <int KIND>
+struct QuadNodes {
+    double v[KIND == kGreenIso ? 1 : kMaxQuad][KIND == kGreenPoly ? 6 : 2];
+};
+static_assert(sizeof(Medium) + sizeof(QuadNodes<kGreenPoly>) + sizeof(TabulateParams) + 64 <= 32764, "kernel parameters");
 
 // G as six entries (11, 12, 22, 33, 13, 23) of the symmetric tensor: Kelvin's closed form.
-__device__ void green_isotropic(double rx, double ry, double rz, double g[6]) {
+__device__ __forceinline__ void green_isotropic(const MaterialDev& mat, double rx, double ry, double rz, double g[6]) {
     const double R2 = rx * rx + ry * ry + rz * rz;
     const double R = sqrt(R2);
-    const double pre = c_mat.kelvin_pre / R;
+    const double pre = mat.kelvin_pre / R;
     const double iR2 = 1.0 / R2;
-    const double a = c_mat.kelvin_a;
+    const double a = mat.kelvin_a;
     g[0] = pre * (a + rx * rx * iR2);
     g[1] = pre * (rx * ry * iR2);
     g[2] = pre * (a + ry * ry * iR2);
@@ -61,7 +74,8 @@ __device__ void green_isotropic(double rx, double ry, double rz, double g[6]) {
 
 // Barnett's integral for a cubic medium node by node: the Christoffel matrix M of z = cos(psi) e1 + sin(psi) e2,
 // its cofactors and a division at every node, about 88 FP64 operations each.
-__device__ void green_nodes(double rx, double ry, double rz, double g[6]) {
+__device__ __forceinline__ void green_nodes(const MaterialDev& mat, const QuadNodes<kGreenNodes>& N, double rx, double ry,
+                                            double rz, double g[6]) {
     const double R2 = rx * rx + ry * ry + rz * rz;
     const double R = sqrt(R2);
     // unit direction and an orthonormal pair spanning the plane normal to it
@@ -79,9 +93,9 @@ __device__ void green_nodes(double rx, double ry, double rz, double g[6]) {
     const double e2y = hz * e1x - hx * e1z;
     const double e2z = hx * e1y - hy * e1x;
     double s0 = 0, s1 = 0, s2 = 0, s3 = 0, s4 = 0, s5 = 0;  // 11 22 33 23 13 12
-    const int nq = c_mat.nquad;
+    const int nq = mat.nquad;
     for (int q = 0; q < nq; q++) {
-        const double cq = c_qcos[q], sq = c_qsin[q];
+        const double cq = N.v[q][0], sq = N.v[q][1];
         const double zx = cq * e1x + sq * e2x;
         const double zy = cq * e1y + sq * e2y;
         const double zz = cq * e1z + sq * e2z;
@@ -91,7 +105,7 @@ __device__ void green_nodes(double rx, double ry, double rz, double g[6]) {
         for (int I = 0; I < 6; I++) {
             double v = 0.0;
 #pragma unroll
-            for (int J = 0; J < 6; J++) v = fma(c_mat.K[6 * I + J], p[J], v);
+            for (int J = 0; J < 6; J++) v = fma(mat.K[6 * I + J], p[J], v);
             m[I] = v;
         }
         // symmetric 3x3 inverse by the adjugate; m = (a, b, c, d, e, f) = (00, 11, 22, 12, 02, 01)
@@ -121,17 +135,17 @@ struct CubicDir {
     double rho2, rho, e1x, e1y, p[6], k11[6];
 };
 
-__device__ __forceinline__ void christoffel(const double (&p)[6], double (&m)[6]) {
+__device__ __forceinline__ void christoffel(const MaterialDev& mat, const double (&p)[6], double (&m)[6]) {
 #pragma unroll
     for (int I = 0; I < 6; I++) {
         double v = 0.0;
 #pragma unroll
-        for (int J = 0; J < 6; J++) v = fma(c_mat.K[6 * I + J], p[J], v);
+        for (int J = 0; J < 6; J++) v = fma(mat.K[6 * I + J], p[J], v);
         m[I] = v;
     }
 }
 
-__device__ __forceinline__ CubicDir cubic_dir(double rx, double ry) {
+__device__ __forceinline__ CubicDir cubic_dir(const MaterialDev& mat, double rx, double ry) {
     CubicDir D;
     const bool line = rx == 0.0 && ry == 0.0;  // r along the line: any in-plane direction
     D.rho2 = fma(rx, rx, ry * ry);
@@ -143,7 +157,7 @@ __device__ __forceinline__ CubicDir cubic_dir(double rx, double ry) {
     D.p[1] = rx * rx * i;
     D.p[2] = D.p[3] = D.p[4] = 0.0;
     D.p[5] = -(rx * ry) * i;
-    christoffel(D.p, D.k11);
+    christoffel(mat, D.p, D.k11);
     return D;
 }
 
@@ -159,7 +173,9 @@ __device__ __forceinline__ CubicDir cubic_dir(double rx, double ry) {
 // products of the entries of M, not to the determinant at a node: the form serves the media cubic_poly_form lets through.
 // The 1000 x 1500, L = 64 cubic slab's table: 112.3 ms with its first update before, 6.9 ms now;
 // 4000 x 6000, L = 256: 1676 ms before, 97 ms now (433 ms with the node-by-node form).
-__device__ void green_cubic(const CubicDir& D, double rx, double ry, double rz, double g[6]) {
+__device__ __forceinline__ void green_cubic(const Medium& M, const QuadNodes<kGreenPoly>& N, const CubicDir& D, double rx,
+                                            double ry, double rz, double g[6]) {
+    const MaterialDev& mat = M.m;
     const double R2 = fma(rz, rz, D.rho2), R = sqrt(R2), iR = 1.0 / R, i2 = 1.0 / R2;
     const double hz = rz * iR, hr = D.rho * iR, zz = rz * rz * i2;
     double u[6], v[6], w[6];  // 2 M = u + v cos 2psi + w sin 2psi, entries (00, 11, 22, 12, 02, 01)
@@ -167,10 +183,10 @@ __device__ void green_cubic(const CubicDir& D, double rx, double ry, double rz, 
         // e2 = (-hz e1y, hz e1x, hr)
         const double p22[6] = {zz * D.p[1], zz * D.p[0], D.rho2 * i2, -(rz * ry) * i2, -(rz * rx) * i2, -zz * D.p[5]};
         double k22[6];
-        christoffel(p22, k22);
+        christoffel(mat, p22, k22);
         const double x = 2.0 * hz * D.p[5];
         const double p12[6] = {-x, x, 0.0, D.e1y * hr, D.e1x * hr, hz * (D.p[0] - D.p[1])};
-        christoffel(p12, w);
+        christoffel(mat, p12, w);
 #pragma unroll
         for (int t = 0; t < 6; t++) u[t] = D.k11[t] + k22[t], v[t] = D.k11[t] - k22[t];
     }
@@ -207,12 +223,12 @@ __device__ void green_cubic(const CubicDir& D, double rx, double ry, double rz, 
     det(0, A[0]);
     double s0 = 0, s1 = 0, s2 = 0, s3 = 0, s4 = 0, t0 = 0, t1 = 0, t2 = 0, t3 = 0, t4 = 0;
     auto parts = [&](int q, double& E, double& O) {
-        const double* n = c_node[q];
+        const double* n = N.v[q];
         E = fma(n[3], d4, fma(n[2], d3, d0));
         O = fma(n[5], d6, fma(n[4], d5, fma(n[1], d2, n[0] * d1)));
     };
     auto add = [&](int q, double e, double o) {  // e, o: the even and odd parts of the node's 1 / det
-        const double* n = c_node[q];
+        const double* n = N.v[q];
         t0 += e;
         t1 = fma(n[0], o, t1);
         t2 = fma(n[1], o, t2);
@@ -223,7 +239,7 @@ __device__ void green_cubic(const CubicDir& D, double rx, double ry, double rz, 
         s0 += t0, s1 += t1, s2 += t2, s3 += t3, s4 += t4;
         t0 = t1 = t2 = t3 = t4 = 0.0;
     };
-    const int nq = c_mat.nquad;
+    const int nq = mat.nquad;
     double scale;
     if (nq % 4 == 0) {
         for (int q = 0; q < nq / 2; q += 2) {
@@ -249,7 +265,7 @@ __device__ void green_cubic(const CubicDir& D, double rx, double ry, double rz, 
         scale = 1.0;
     }
     join();
-    const double pre = scale * c_pre * iR;
+    const double pre = scale * M.pre * iR;
     auto entry = [&](const double (&q)[5]) {
         return pre * fma(q[0], s0, fma(q[1], s1, fma(q[2], s2, fma(q[3], s3, q[4] * s4))));
     };
@@ -261,28 +277,22 @@ __device__ void green_cubic(const CubicDir& D, double rx, double ry, double rz, 
     g[5] = entry(A[3]);
 }
 
-// Which Green function a launch evaluates.  The polynomial form serves the plans of the FP64-accurate precisions whose
-// medium and node count cubic_poly_form lets through.
-// The others round the table to 32 bits or fewer, where a last-bit change of a few FP64 entries moves the
-// rounding of some (1e-9 to 4e-9 of an update, more than those forms differ by from run to run): they and the
-// H-matrix's FP32 table keep the node-by-node form's bits.
-enum { kGreenIso = 0, kGreenNodes = 1, kGreenPoly = 2 };
-
 // G(0, 0, m l3) + G(0, 0, -m l3) for the images m = 1 .. n + N (one block each, a thread per sign): the same for every
 // difference and offset.
 template <int KIND>
-__global__ void k_reference(double* __restrict__ ref) {
+__global__ void k_reference(const __grid_constant__ Medium M, const __grid_constant__ QuadNodes<KIND> Q,
+                            const __grid_constant__ TabulateParams T, double* __restrict__ ref) {
     const int m = blockIdx.x + 1;
     __shared__ double h[6];
-    const double zm = (threadIdx.x ? -1.0 : 1.0) * ((double)m * ((double)c_tp.L * c_tp.c));
+    const double zm = (threadIdx.x ? -1.0 : 1.0) * ((double)m * ((double)T.L * T.c));
     double g[6];
-    if (KIND == kGreenIso) {
-        green_isotropic(0.0, 0.0, zm, g);
-    } else if (KIND == kGreenNodes) {
-        green_nodes(0.0, 0.0, zm, g);
+    if constexpr (KIND == kGreenIso) {
+        green_isotropic(M.m, 0.0, 0.0, zm, g);
+    } else if constexpr (KIND == kGreenNodes) {
+        green_nodes(M.m, Q, 0.0, 0.0, zm, g);
     } else {
-        const CubicDir D = cubic_dir(0.0, 0.0);
-        green_cubic(D, 0.0, 0.0, zm, g);
+        const CubicDir D = cubic_dir(M.m, 0.0, 0.0);
+        green_cubic(M, Q, D, 0.0, 0.0, zm, g);
     }
     if (threadIdx.x == 1)
         for (int t = 0; t < 6; t++) h[t] = g[t];
@@ -294,9 +304,10 @@ __global__ void k_reference(double* __restrict__ ref) {
 // Stage 1: one thread per (listed difference, s in [0, L/2]).  Of a pair of used differences d and -d only one
 // is listed: G(-d, s) is G(d, s) with the odd entries (13, 23) negated, bit for bit, so stage 2 writes both.
 template <int KIND>
-__global__ void __launch_bounds__(128) k_periodic(const int4* __restrict__ rep, int n_rep,
-                                                  const double* __restrict__ ref, double* __restrict__ gs) {
-    const int Lh = c_tp.Lh;
+__global__ void __launch_bounds__(128) k_periodic(const __grid_constant__ Medium M, const __grid_constant__ QuadNodes<KIND> Q,
+                                                  const __grid_constant__ TabulateParams T, const int4* __restrict__ rep,
+                                                  int n_rep, const double* __restrict__ ref, double* __restrict__ gs) {
+    const int Lh = T.Lh;
     const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const long long total = (long long)n_rep * (Lh + 1);
     if (tid >= total) return;
@@ -309,18 +320,18 @@ __global__ void __launch_bounds__(128) k_periodic(const int4* __restrict__ rep, 
         return;
     }
     const double rx = (double)d.x, ry = (double)d.y;
-    const double l3 = (double)c_tp.L * c_tp.c;
-    const double z0 = (double)s * c_tp.c;  // centred representative: s <= L/2
+    const double l3 = (double)T.L * T.c;
+    const double z0 = (double)s * T.c;  // centred representative: s <= L/2
     CubicDir D;
-    if (KIND == kGreenPoly) D = cubic_dir(rx, ry);
+    if (KIND == kGreenPoly) D = cubic_dir(M.m, rx, ry);
     auto green = [&](double z, double (&g)[6]) {
-        if (KIND == kGreenIso) green_isotropic(rx, ry, z, g);
-        else if (KIND == kGreenNodes) green_nodes(rx, ry, z, g);
-        else green_cubic(D, rx, ry, z, g);
+        if constexpr (KIND == kGreenIso) green_isotropic(M.m, rx, ry, z, g);
+        else if constexpr (KIND == kGreenNodes) green_nodes(M.m, Q, rx, ry, z, g);
+        else green_cubic(M, Q, D, rx, ry, z, g);
     };
     double acc[6], g[6], h[6];
     green(z0, acc);
-    const int n = c_tp.rich_n, N = c_tp.rich_N;
+    const int n = T.rich_n, N = T.rich_N;
     double tail[6] = {0, 0, 0, 0, 0, 0};
     for (int m = 1; m <= n + N; m++) {
         const double zm = (double)m * l3;
@@ -331,7 +342,7 @@ __global__ void __launch_bounds__(128) k_periodic(const int4* __restrict__ rep, 
 #pragma unroll
             for (int t = 0; t < 6; t++) acc[t] += ((g[t] + h[t]) - rf[t]);
         } else {
-            const double w = c_tp.W[m - n - 1];
+            const double w = T.W[m - n - 1];
 #pragma unroll
             for (int t = 0; t < 6; t++) tail[t] = fma(w, (g[t] + h[t]) - rf[t], tail[t]);
         }
@@ -351,17 +362,17 @@ __global__ void __launch_bounds__(128) k_periodic(const int4* __restrict__ rep, 
 
 // Stage 2: one CTA per listed difference; threads over k.  The table entry of -d is that of d with the odd
 // entries negated.
-__global__ void k_line_dft(const int4* __restrict__ rep, const double* __restrict__ gs,
-                           const double2* __restrict__ twL, double* __restrict__ table) {
+__global__ void k_line_dft(const __grid_constant__ TabulateParams T, const int4* __restrict__ rep,
+                           const double* __restrict__ gs, const double2* __restrict__ twL, double* __restrict__ table) {
     extern __shared__ double sg[];  // [Lh+1][6]
-    const int Lh = c_tp.Lh, L = c_tp.L, K = c_tp.K;
+    const int Lh = T.Lh, L = T.L, K = T.K;
     const int di = blockIdx.x;
     const double* src = gs + (size_t)di * (Lh + 1) * 6;
     for (int t = threadIdx.x; t < (Lh + 1) * 6; t += blockDim.x) sg[t] = src[t];
     __syncthreads();
     const int4 d = rep[di];
-    const int ix = d.x - c_tp.box_x0, iy = d.y - c_tp.box_y0;
-    const int mx = -d.x - c_tp.box_x0, my = -d.y - c_tp.box_y0;  // -d, in the box where it is used
+    const int ix = d.x - T.box_x0, iy = d.y - T.box_y0;
+    const int mx = -d.x - T.box_x0, my = -d.y - T.box_y0;  // -d, in the box where it is used
     for (int k = threadIdx.x; k < K; k += blockDim.x) {
         const double sgn = (k & 1) ? -1.0 : 1.0;
         double A0 = 0, A1 = 0, A2 = 0, A3 = 0, B4 = 0, B5 = 0;
@@ -387,11 +398,11 @@ __global__ void k_line_dft(const int4* __restrict__ rep, const double* __restric
         v[3] = g0[3] + sgn * gh[3] + 2.0 * A3;
         v[4] = -2.0 * B4;
         v[5] = -2.0 * B5;
-        double* o = table + (((size_t)k * c_tp.Dy + iy) * c_tp.Dx + ix) * 6;
+        double* o = table + (((size_t)k * T.Dy + iy) * T.Dx + ix) * 6;
 #pragma unroll
         for (int t = 0; t < 6; t++) o[t] = v[t];
         if (d.z) {
-            double* q = table + (((size_t)k * c_tp.Dy + my) * c_tp.Dx + mx) * 6;
+            double* q = table + (((size_t)k * T.Dy + my) * T.Dx + mx) * 6;
 #pragma unroll
             for (int t = 0; t < 6; t++) q[t] = t < 4 ? v[t] : -v[t];
         }
@@ -451,62 +462,56 @@ bool cubic_poly_form(const fbc_material& m, int nquad) {
     return nquad >= 48 && 1.0 <= 3.0 * 27.0 * det;
 }
 
-// The plan's medium and tabulation parameters into this file's constant memory (shared by every
-// plan: uploaded again before each use).  The copies' sources live in the plan.
-static cudaError_t upload_tabulate_constants(Plan& P, int kind, cudaStream_t st) {
-    auto put = [&](const auto& symbol, const void* src, size_t bytes) {
-        return cudaMemcpyToSymbolAsync(symbol, src, bytes, 0, cudaMemcpyHostToDevice, st);
-    };
-    cudaError_t e;
+// A cubic plan's quadrature nodes and scaled constants, once.
+static void make_tabulate_constants(Plan& P) {
     const int nq = P.mat.nquad;
-    if (kind != kGreenIso && P.tab_nodes.empty()) {
-        P.tab_nodes.assign((size_t)nq * 8, 0.0);  // [nq] cos, [nq] sin of psi, then [nq][6]
-        for (int q = 0; q < nq; q++) {
-            const double psi = M_PI * (double)q / (double)nq;
-            P.tab_nodes[q] = cos(psi), P.tab_nodes[nq + q] = sin(psi);
-            for (int j = 0; j < 3; j++) {
-                const double a = M_PI * (double)((2LL * (j + 1) * q) % (2LL * nq)) / (double)nq;
-                P.tab_nodes[(size_t)2 * nq + q * 6 + 2 * j] = cos(a);
-                P.tab_nodes[(size_t)2 * nq + q * 6 + 2 * j + 1] = sin(a);
-            }
+    P.tab_nodes.assign((size_t)nq * 8, 0.0);  // [nq] cos, [nq] sin of psi, then [nq][6]
+    for (int q = 0; q < nq; q++) {
+        const double psi = M_PI * (double)q / (double)nq;
+        P.tab_nodes[q] = cos(psi), P.tab_nodes[nq + q] = sin(psi);
+        for (int j = 0; j < 3; j++) {
+            const double a = M_PI * (double)((2LL * (j + 1) * q) % (2LL * nq)) / (double)nq;
+            P.tab_nodes[(size_t)2 * nq + q * 6 + 2 * j] = cos(a);
+            P.tab_nodes[(size_t)2 * nq + q * 6 + 2 * j + 1] = sin(a);
         }
-        // the constants scaled by a power of two to a largest magnitude in [1, 2): products of four
-        // determinants stay in range whatever the unit of stress
-        double top = 0.0;
-        for (int t = 0; t < 36; t++) top = std::max(top, std::fabs(P.mat.K[t]));
-        const double sc = std::ldexp(1.0, -std::ilogb(top));
-        P.tab_mat = P.mat;
-        for (int t = 0; t < 36; t++) P.tab_mat.K[t] = P.mat.K[t] * sc;
-        P.tab_pre = sc / (M_PI * (double)nq);
     }
-    if (kind == kGreenNodes) {
-        if ((e = put(c_qcos, P.tab_nodes.data(), sizeof(double) * nq))) return e;
-        if ((e = put(c_qsin, P.tab_nodes.data() + nq, sizeof(double) * nq))) return e;
-    }
-    if (kind == kGreenPoly) {
-        if ((e = put(c_node, P.tab_nodes.data() + 2 * (size_t)nq, sizeof(double) * 6 * nq))) return e;
-        if ((e = put(c_pre, &P.tab_pre, sizeof(double)))) return e;
-    }
-    if ((e = put(c_mat, kind == kGreenPoly ? &P.tab_mat : &P.mat, sizeof(MaterialDev)))) return e;
-    return put(c_tp, &P.tp, sizeof(TabulateParams));
+    // the constants scaled by a power of two to a largest magnitude in [1, 2): products of four
+    // determinants stay in range whatever the unit of stress
+    double top = 0.0;
+    for (int t = 0; t < 36; t++) top = std::max(top, std::fabs(P.mat.K[t]));
+    const double sc = std::ldexp(1.0, -std::ilogb(top));
+    P.tab_mat = P.mat;
+    for (int t = 0; t < 36; t++) P.tab_mat.K[t] = P.mat.K[t] * sc;
+    P.tab_pre = sc / (M_PI * (double)nq);
 }
 
 // Stage 1 of nd listed differences from d0 on (ref: the images' reference sums).
 template <int KIND>
 static cudaError_t launch_periodic(Plan& P, int d0, int nd, double* ref, double* gs, cudaStream_t st) {
-    if (d0 == 0) k_reference<KIND><<<P.tp.rich_n + P.tp.rich_N, 2, 0, st>>>(ref);
+    if (KIND != kGreenIso && P.tab_nodes.empty()) make_tabulate_constants(P);
+    Medium M;
+    M.m = KIND == kGreenPoly ? P.tab_mat : P.mat, M.pre = P.tab_pre;
+    QuadNodes<KIND> N{};
+    if constexpr (KIND != kGreenIso) {
+        const int nq = P.mat.nquad;
+        const double* v = P.tab_nodes.data();
+        for (int q = 0; q < nq; q++) {
+            if constexpr (KIND == kGreenPoly) std::copy(v + 2 * nq + 6 * q, v + 2 * nq + 6 * q + 6, N.v[q]);
+            else N.v[q][0] = v[q], N.v[q][1] = v[nq + q];
+        }
+    }
+    if (d0 == 0) k_reference<KIND><<<P.tp.rich_n + P.tp.rich_N, 2, 0, st>>>(M, N, P.tp, ref);
     const long long threads = (long long)nd * (P.L / 2 + 1);
-    k_periodic<KIND><<<(unsigned)((threads + 127) / 128), 128, 0, st>>>(P.d_rep + d0, nd, ref, gs);
+    k_periodic<KIND><<<(unsigned)((threads + 127) / 128), 128, 0, st>>>(M, N, P.tp, P.d_rep + d0, nd, ref, gs);
     return cudaGetLastError();
 }
 
-// Constants, the stage-1 buffer (differences in chunks of at most 256 MB) after the reference sums, and
+// The stage-1 buffer (differences in chunks of at most 256 MB) after the reference sums, and
 // `stage2(d0, nd, gs)` for every chunk.
 template <class F>
 static cudaError_t tabulate_chunks(Plan& P, int kind, cudaStream_t st, F stage2) {
-    cudaError_t e;
-    if ((e = upload_tabulate_constants(P, kind, st))) return e;
     if (P.n_rep == 0) return cudaSuccess;
+    cudaError_t e;
     const size_t per_d = (size_t)(P.L / 2 + 1) * 6 * sizeof(double);
     const size_t n_ref = kMaxRichImages * 6;
     const int chunk = (int)std::min<size_t>((size_t)P.n_rep, std::max<size_t>(1, ((size_t)256 << 20) / per_d));
@@ -535,16 +540,16 @@ cudaError_t launch_tabulate(Plan& P, cudaStream_t st) {
                                                              : kGreenPoly;
     return tabulate_chunks(P, kind, st, [&](int d0, int nd, const double* gs) {
         const int bt = std::min(256, std::max(32, ((P.K + 31) / 32) * 32));
-        k_line_dft<<<nd, bt, smem, st>>>(P.d_rep + d0, gs, P.d_twL, P.d_table);
+        k_line_dft<<<nd, bt, smem, st>>>(P.tp, P.d_rep + d0, gs, P.d_twL, P.d_table);
         return cudaGetLastError();
     });
 }
 
 // Stage-1 output of a chunk of listed differences, rounded to FP32 and placed at each difference's
 // cell of the box (and its mirror's, the odd entries negated): out[cell][s][6] for s = 0..L/2.
-__global__ void k_real_space_scatter(const int4* __restrict__ rep, int n_rep, const double* __restrict__ gs,
-                                     float* __restrict__ out) {
-    const int Lh = c_tp.Lh;
+__global__ void k_real_space_scatter(const __grid_constant__ TabulateParams T, const int4* __restrict__ rep, int n_rep,
+                                     const double* __restrict__ gs, float* __restrict__ out) {
+    const int Lh = T.Lh;
     const long long per = (long long)(Lh + 1) * 6;
     const long long total = (long long)n_rep * per;
     for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < total;
@@ -553,8 +558,8 @@ __global__ void k_real_space_scatter(const int4* __restrict__ rep, int n_rep, co
         const long long r = t - (long long)di * per;
         const int4 d = rep[di];
         const float v = (float)gs[t];
-        out[((long long)(d.y - c_tp.box_y0) * c_tp.Dx + (d.x - c_tp.box_x0)) * per + r] = v;
-        if (d.z) out[((long long)(-d.y - c_tp.box_y0) * c_tp.Dx + (-d.x - c_tp.box_x0)) * per + r] = r % 6 < 4 ? v : -v;
+        out[((long long)(d.y - T.box_y0) * T.Dx + (d.x - T.box_x0)) * per + r] = v;
+        if (d.z) out[((long long)(-d.y - T.box_y0) * T.Dx + (-d.x - T.box_x0)) * per + r] = r % 6 < 4 ? v : -v;
     }
 }
 
@@ -564,7 +569,7 @@ cudaError_t launch_real_space_table(Plan& P, float* out, cudaStream_t st) {
     if (e) return e;
     const int kind = P.mat.kind == FBC_MATERIAL_ISOTROPIC ? kGreenIso : kGreenNodes;
     return tabulate_chunks(P, kind, st, [&](int d0, int nd, const double* gs) {
-        k_real_space_scatter<<<1216, 256, 0, st>>>(P.d_rep + d0, nd, gs, out);
+        k_real_space_scatter<<<1216, 256, 0, st>>>(P.tp, P.d_rep + d0, nd, gs, out);
         return cudaGetLastError();
     });
 }
