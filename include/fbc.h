@@ -147,7 +147,8 @@ typedef struct fbc_options {
     int32_t rich_n;     /* Richardson n (Eq. 36), default 4 */
     int32_t rich_N;     /* Richardson order N (Eq. 36), default 6; n_img = n + N */
     int32_t quad;       /* Barnett trapezoid nodes on [0, pi), default 64 */
-    int32_t max_rhs;    /* largest n_rhs fbc_apply will accept, default 1 */
+    int32_t max_rhs;    /* largest n_rhs fbc_apply will accept, default 1; small plans split their sums by it, so
+                           plans that differ in it alone may differ in the last bits */
     int32_t flags;      /* FBC_PLAN_* bits, default 0 */
 } fbc_options;
 
@@ -203,7 +204,12 @@ int fbc_plan_create(const fbc_geometry* geom, const fbc_material* mat, const fbc
  * reused by every apply (Sec. 3.2: the setup is reused across runs).
  * Asynchronous on `stream`, except that for the in-plane FFT forms the first
  * call also builds the grid (host structures and device buffers: synchronous,
- * allocates) before it queues the grid transform of the table. */
+ * allocates) before it queues the grid transform of the table.
+ * For a cubic medium that is not too far from isotropic (the rule stands in
+ * fbc_tabulate.cu) the FP64-accurate precisions evaluate Barnett's quadrature
+ * in another form than the FP32 and reduced ones, as exact but with other
+ * last bits: the table has the bits of the precision set at this call.  Plans
+ * may be tabulated at the same time on different streams. */
 int fbc_tabulate_kernel(fbc_plan* plan, void* stream);
 
 /* The pad update (see the top of this file) for n_rhs right-hand sides:
@@ -235,8 +241,9 @@ int fbc_apply(fbc_plan* plan, const double* f, double* u, int32_t n_rhs, double 
  *   f_new, f_old: DEVICE double [n_rhs][n_i][L][3]; u: DEVICE double
  *   [n_rhs][n_p][L][3] (updated in place); alpha_io: DEVICE double [n_rhs].
  * Asynchronous on `stream`; no allocation and no host synchronisation (alpha is
- * computed on the device).  The plan's contracted modes are transformed twice
- * (once for the maximum, once for the update) when du_max > 0. */
+ * computed on the device).  When du_max > 0 the forms with FP32 line transforms
+ * transform the contracted modes twice (once for the maximum, once for the
+ * update); the others keep G f_new from the first pass. */
 int fbc_apply_relaxed(fbc_plan* plan, const double* f_new, const double* f_old, double* u, int32_t n_rhs,
                       double* alpha_io, double du_max, uint32_t flags, void* stream);
 
@@ -258,7 +265,9 @@ int fbc_apply_host(fbc_plan* plan, const double* f_host, double* u_host, int32_t
  * precision's derived table from the FP64 table on first use (allocates;
  * call outside stream capture): the FP32 or double-float table, or for the
  * in-plane FFT forms the grid and its transformed kernel (K x Mx x My x 6
- * reals in FP64, plus an FP32 copy for FBC_PREC_FFT32).  Synchronous. */
+ * reals in FP64, plus an FP32 copy for FBC_PREC_FFT32).  The FP64 table itself
+ * stays as it was tabulated (see fbc_tabulate_kernel on its last bits).
+ * Synchronous. */
 int fbc_plan_set_precision(fbc_plan* plan, int32_t precision);
 
 /* Bound of the pipeline waits of the tensor-core contraction (the hand-offs
