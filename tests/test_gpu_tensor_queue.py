@@ -7,7 +7,7 @@ import pytest
 
 from conftest import ISO
 from paper_2105_08798_gb300 import inputs
-from test_gpu_tensor_shapes import _sites
+from test_gpu_tensor_shapes import _sites, test_shapes as _test_shapes
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -42,3 +42,19 @@ def test_mixed_staging(precision, R):
                 v.fill_(float("nan"))
     for p in plans:
         p.close()
+
+
+@pytest.mark.parametrize("kind,n_i,n_p,step,L,R,mat", next(m.args[1] for m in _test_shapes.pytestmark if m.name == "parametrize"))
+def test_every_form_takes_every_shape(kind, n_i, n_p, step, L, R, mat):
+    """None of the geometries of those tests is too large for a form's shared memory: no form may refuse one."""
+    from paper_2105_08798_gb300 import fbc
+
+    xy_i, xy_p = _sites(kind, n_i, n_p, step)
+    f = torch.from_numpy(inputs.forces(R, len(xy_i), L, seed=1)).cuda()
+    with fbc.Plan(xy_i, xy_p, L, mat, max_rhs=R) as plan:
+        plan.tabulate()
+        for precision in ("tf32", "bf16x2", "bf16x3"):
+            plan.set_precision(precision)
+            plan.apply(f, torch.empty((R, len(xy_p), L, 3), dtype=torch.float64, device="cuda"))
+            torch.cuda.synchronize()
+            plan.sync_status()
