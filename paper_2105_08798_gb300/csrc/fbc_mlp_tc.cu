@@ -25,8 +25,8 @@
 //
 // What bounds it: the epilogues, 3 H SiLU a row.  Their special-function
 // instructions (two a value would be 20 us more than the pair's three) and the
-// rest, about 9 issue slots a value, take half the issue slots; the tensor pipe
-// runs 35 % of the time.  10^6 rows, H = 128: 1.18 ms with one tile in flight,
+// rest, about 9 issue slots a value, take 61 % of the issue slots; the tensor pipe
+// runs 39 % of the time.  10^6 rows, H = 128: 1.18 ms with one tile in flight,
 // barriers of the whole CTA, expf and a rounded reciprocal; 0.24 ms with two
 // tiles, 0.17 ms with the products started by column chunks of 16 (0.19 of 32)
 // and the biases in the products.  Against 64 bits the outputs of 2 * 10^5 rows

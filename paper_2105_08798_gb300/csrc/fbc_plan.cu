@@ -755,7 +755,7 @@ int fbc_apply_host(fbc_plan* plan, const double* f_host, double* u_host, int32_t
     // The tensor-core forms' chunks hold whole right-hand-side groups (a CTA's work hardly depends on its
     // group's fill), the part-filled one first: it is the quickest to copy in, and the others' copies run
     // beside its applies (BF16X6, 1777 + 2666 columns, L = 128, 40 right-hand sides: 20.8 ms as one
-    // chunk, 18.7 as 8 and 32).
+    // chunk, 18.7 as 8 and 32; hosts whose copies vary took up to 20.9).
     const int gran = P.precision == FBC_PREC_BF16X6  ? fbc::contract_oz_rhs_group()
                      : fbc::is_tensor_precision(P.precision) ? fbc::contract_tc_max_rpc(P)
                                                              : fbc::kHostChunkRhs;
