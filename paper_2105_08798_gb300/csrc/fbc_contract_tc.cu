@@ -490,7 +490,7 @@ __device__ __forceinline__ void tc_item(const TcJob& J, const int4 wk, const uin
             int il = 0, gpos = 0;  // stage of the item and its position in the accumulation group
             int j = 0;             // A buffer
             const bool bulk = J.bulk;
-            const int pitch = J.pitch, om = bulk ? 1 : 24;  // bytes of a sub-box row, of a unit of s_off
+            const unsigned pitch = (unsigned)J.pitch, om = bulk ? 1u : 24u;  // bytes of a sub-box row, of a unit of s_off
             if (!bulk && nbuf == 2) stage_async(0, 0);
             for (int tB = 0, buf = 0; tB < A.n_tb; tB++, buf = buf + 1 == nbuf ? 0 : buf + 1) {
                 const int4 bB = A.bbox_b[tB];
@@ -511,9 +511,12 @@ __device__ __forceinline__ void tc_item(const TcJob& J, const int4 wk, const uin
                 const unsigned char* tab_b = s_tab + (size_t)buf * J.tab_bytes;
                 const int* off_b = s_off + buf * kTileB;
                 const int ox = bA.x - bB.y, oy = bA.z - bB.w;
-                // byte offset of entries 2 pl of this row's difference to the origin; behind a shift of 0 or 8
-                const int odd = (((k - A.kbase) * A.Dy + oy - A.box_y0) * A.Dx + ox - A.box_x0) & 1;
-                const int base = 24 * (xa.x - ox) + (int)((unsigned)pitch * (unsigned)(xa.y - oy)) + 8 * pl + (bulk ? 8 * odd : 0);
+                // byte offset of entries 2 pl of this row's difference to the origin, behind a shift of 0 or 8.  Modulo 2^32,
+                // as the columns' offsets: sites may lie so far out that their own offsets wrap, their differences do not.
+                const unsigned odd =
+                    (((unsigned)(k - A.kbase) * (unsigned)A.Dy + (unsigned)(oy - A.box_y0)) * (unsigned)A.Dx + (unsigned)(ox - A.box_x0)) & 1u;
+                const unsigned base = 24u * (unsigned)(xa.x - ox) + pitch * (unsigned)(xa.y - oy) + 8u * (unsigned)pl + (bulk ? 8u * odd : 0u);
+                auto entries = [&](int o) { return *(const float2*)(tab_b + (int)(base - om * (unsigned)o)); };
                 for (int st = 0; st < kStagesPerTile; st++, il++) {
                     const uint32_t it = it_base + il;
                     const int s = it % S;
@@ -537,10 +540,7 @@ __device__ __forceinline__ void tc_item(const TcJob& J, const int4 wk, const uin
 #pragma unroll
                     for (int i = 0; i < kKC; i += 4) {
                         const int4 o = *(const int4*)(off_b + st * kKC + i);
-                        v[i] = *(const float2*)(tab_b + (base - om * o.x));
-                        v[i + 1] = *(const float2*)(tab_b + (base - om * o.y));
-                        v[i + 2] = *(const float2*)(tab_b + (base - om * o.z));
-                        v[i + 3] = *(const float2*)(tab_b + (base - om * o.w));
+                        v[i] = entries(o.x), v[i + 1] = entries(o.y), v[i + 2] = entries(o.z), v[i + 3] = entries(o.w);
                     }
                     // split into NS pieces: w[(entry, piece)][32-bit words of 16 elements], packed round-to-nearest
                     // conversions with exact FP32 remainders (bf16), or one tf32 word per element
