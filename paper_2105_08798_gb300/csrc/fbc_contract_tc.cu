@@ -687,6 +687,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         tc_item<PREC>(s_job, s_wk, it_base, n_done, sy, smem, wl, aph);
         it_base += (uint32_t)(s_job.A.n_tb * kStagesPerTile);
         n_done++;
+        // a table buffer that the builders filled themselves may be the next item's target of bulk copies: their writes
+        // come before those of the other proxy
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncthreads();  // every role is done with s_job and s_wk before thread 0 overwrites them
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
